@@ -97,7 +97,7 @@ int rapral_batch_create(rapral_ctx* ctx, int n_items, const rapral_batch_item* i
         need = arena_need(need, C * sizeof(CellPrep));
         need = arena_need(need, L * sizeof(int2));
         need = arena_need(need, (T + 1) * sizeof(int));
-        need = arena_need(need, (RAPRAL_DMAX_SLOTS + 2) * sizeof(unsigned long long));
+        need = arena_need(need, (RAPRAL_DMAX_SLOTS + 3) * sizeof(unsigned long long));
         need = arena_need(need, 4 * sizeof(int));
         if (broad_terms(&ctx->broad)) need = broad_need(need, L, C, r.sp.n_species);
         need = arena_need(need, 0);
@@ -116,7 +116,6 @@ int rapral_batch_create(rapral_ctx* ctx, int n_items, const rapral_batch_item* i
                        double* g0 = nullptr; };
     std::vector<BroadTabs> btabs(n_items);
     const Phys ph = make_phys(ctx->codata);
-    static const int one = 1;
     long long* h_tot = nullptr;   // [n_items] tile-list lengths, then the status word
     e = cudaMallocHost(&h_tot, sizeof(long long) * (n_items + 1));
     for (int i = 0; i < n_items && e == cudaSuccess; ++i) {
@@ -130,10 +129,10 @@ int rapral_batch_create(rapral_ctx* ctx, int n_items, const rapral_batch_item* i
         pl.k0 = r.k0; pl.nk = r.nk; pl.tile_w = W; pl.n_tiles = T;
         pl.line_tiles = ar.take<int2>(L);
         pl.tile_off = ar.take<int>(T + 1);
-        unsigned long long* dmax = ar.take<unsigned long long>(RAPRAL_DMAX_SLOTS + 2);
+        unsigned long long* dmax = ar.take<unsigned long long>(RAPRAL_DMAX_SLOTS + 3);
         pl.wmax = dmax + RAPRAL_DMAX_SLOTS;
         pl.total = reinterpret_cast<long long*>(dmax + RAPRAL_DMAX_SLOTS + 1);
-        pl.sorted_flag = ar.take<int>(4);
+        pl.unsorted = ar.take<int>(4);
         const bool bt = broad_terms(&ctx->broad);
         BroadTabs& bb = btabs[i];
         if (bt) {
@@ -141,16 +140,12 @@ int rapral_batch_create(rapral_ctx* ctx, int n_items, const rapral_batch_item* i
             bb.cb = ar.take<double2>((size_t)C * r.sp.n_species); bb.cb32 = ar.take<float2>((size_t)C * r.sp.n_species);
             bb.g0 = ar.take<double>(RAPRAL_MAX_SPECIES);
         }
-        e = cudaMemcpyAsync(pl.sorted_flag, &one, sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(pl.wmax, 0, sizeof(unsigned long long), ctx->stream);
-        if (e == cudaSuccess) e = launch_validate_cells(ctx, &r.cells);
-        if (e == cudaSuccess) e = launch_validate_lines(ctx, &r.ln, r.sp.n_species);
-        if (e == cudaSuccess) e = launch_validate_rays(ctx, &r.rays, C);
-        if (e == cudaSuccess) e = launch_line_prep(ctx, &r.sp, &r.ln, r.grid.lam_min, r.h, ph, lps[i], lfs[i],
-                                                  pl.sorted_flag, &ctx->broad, bb.lb, bb.lb32);
+        e = launch_plan_reset(ctx, dmax, &pl);
         if (e == cudaSuccess) e = launch_cell_prep(ctx, &r.cells, ph, cps[i], dmax);
         if (e == cudaSuccess && bt) e = launch_broad_cells(ctx, &r.sp, &r.cells, ctx->broad, bb.g0, bb.cb, bb.cb32, dmax);
-        if (e == cudaSuccess) e = launch_bin_bounds(ctx, &r.ln, lps[i], cps[i], dmax, r.h, &pl, bb.lb);
+        if (e == cudaSuccess) e = launch_validate_rays(ctx, &r.rays, C);
+        if (e == cudaSuccess) e = launch_line_plan(ctx, &r.sp, &r.ln, r.grid.lam_min, r.h, ph, dmax, lps[i], lfs[i],
+                                                  &pl, &ctx->broad, bb.lb, bb.lb32);
         if (e == cudaSuccess) e = launch_bin_count(ctx, &r.ln, &r.grid, r.h, &pl);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h_tot + i, pl.total, sizeof(long long), cudaMemcpyDeviceToHost, ctx->stream);

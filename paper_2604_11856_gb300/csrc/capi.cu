@@ -218,7 +218,7 @@ int rapral_workspace_bytes(int64_t n_lines, int64_t n_cells, int64_t nk, size_t*
     b = arena_need(b, (size_t)n_lines * sizeof(int2));
     b = arena_need(b, (size_t)n_cells * sizeof(CellPrep));
     b = arena_need(b, (size_t)(tiles + 1) * sizeof(int));
-    b = arena_need(b, (RAPRAL_DMAX_SLOTS + 2) * sizeof(unsigned long long) + 64);
+    b = arena_need(b, (RAPRAL_DMAX_SLOTS + 3) * sizeof(unsigned long long) + 64);
     b = arena_need(b, (size_t)(3 * n_lines + tiles) * sizeof(int));
     *bytes = b + b / 4 + (1u << 20);
     return RAPRAL_OK;
@@ -299,7 +299,7 @@ int rapral_spectral_coeffs(rapral_ctx* ctx, const rapral_species* sp, const rapr
     need = arena_need(need, C * sizeof(CellPrep));
     need = arena_need(need, L * sizeof(int2));
     need = arena_need(need, (T + 1) * sizeof(int));
-    need = arena_need(need, (RAPRAL_DMAX_SLOTS + 2) * sizeof(unsigned long long));
+    need = arena_need(need, (RAPRAL_DMAX_SLOTS + 3) * sizeof(unsigned long long));
     need = arena_need(need, 4 * sizeof(int));
     const bool bt = broad_terms(&ctx->broad);
     if (bt) need = broad_need(need, L, C, sp->n_species);
@@ -315,10 +315,10 @@ int rapral_spectral_coeffs(rapral_ctx* ctx, const rapral_species* sp, const rapr
     plan.k0 = k0; plan.nk = nk; plan.tile_w = W; plan.n_tiles = T;
     plan.line_tiles = ar.take<int2>(L);
     plan.tile_off = ar.take<int>(T + 1);
-    unsigned long long* dmax = ar.take<unsigned long long>(RAPRAL_DMAX_SLOTS + 2);
+    unsigned long long* dmax = ar.take<unsigned long long>(RAPRAL_DMAX_SLOTS + 3);
     plan.wmax = dmax + RAPRAL_DMAX_SLOTS;
     plan.total = reinterpret_cast<long long*>(dmax + RAPRAL_DMAX_SLOTS + 1);
-    plan.sorted_flag = ar.take<int>(4);
+    plan.unsorted = ar.take<int>(4);
     double2* lb = nullptr; float2* lb32 = nullptr; double2* cb = nullptr; float2* cb32 = nullptr;
     double* g0 = nullptr;
     if (bt) {
@@ -326,26 +326,19 @@ int rapral_spectral_coeffs(rapral_ctx* ctx, const rapral_species* sp, const rapr
         cb = ar.take<double2>((size_t)C * sp->n_species); cb32 = ar.take<float2>((size_t)C * sp->n_species);
         g0 = ar.take<double>(RAPRAL_MAX_SPECIES);
     }
-    const int one = 1;
-    e = cudaMemcpyAsync(plan.sorted_flag, &one, sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(plan.wmax, 0, sizeof(unsigned long long), ctx->stream);
-    if (e == cudaSuccess) e = launch_validate_cells(ctx, cells);
-    if (e == cudaSuccess) e = launch_validate_lines(ctx, ln, sp->n_species);
-    if (e == cudaSuccess && ctx->dep_lnb) e = launch_check_levels(ctx, ctx->dep_u, ctx->dep_l, L, ctx->dep_nlev);
-    if (e == cudaSuccess)
-        e = launch_line_prep(ctx, sp, ln, g->lam_min, h, ph, lp, lf, plan.sorted_flag, &ctx->broad, lb, lb32);
+    e = launch_plan_reset(ctx, dmax, &plan);
     if (e == cudaSuccess) e = launch_cell_prep(ctx, cells, ph, cp, dmax);
     if (e == cudaSuccess && bt) e = launch_broad_cells(ctx, sp, cells, ctx->broad, g0, cb, cb32, dmax);
-    if (e == cudaSuccess) e = launch_bin_bounds(ctx, ln, lp, cp, dmax, h, &plan, lb);
-    if (e == cudaSuccess) e = launch_bin_count(ctx, ln, g, h, &plan);
+    if (e == cudaSuccess && ctx->dep_lnb) e = launch_check_levels(ctx, ctx->dep_u, ctx->dep_l, L, ctx->dep_nlev);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->h_pinned, plan.total, sizeof(long long), cudaMemcpyDeviceToHost, ctx->stream);
+        e = launch_line_plan(ctx, sp, ln, g->lam_min, h, ph, dmax, lp, lf, &plan, &ctx->broad, lb, lb32);
+    if (e == cudaSuccess) e = launch_bin_count(ctx, ln, g, h, &plan);
     // the device checks ran before: on a failed one the counts were never written
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ctx->h_pinned + 4, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+        e = cudaMemcpyAsync(ctx->h_pinned, plan.total, 2 * sizeof(long long), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_status(ctx, e, "line binning");
-    if (ctx->h_pinned[4 + ST_CODE]) return read_status(ctx);
+    if (reinterpret_cast<const long long*>(ctx->h_pinned)[1]) return read_status(ctx);
     const int64_t total = reinterpret_cast<const long long*>(ctx->h_pinned)[0];
     if (total > RAPRAL_MAX_TILE_ENTRIES)
         return set_error(ctx, RAPRAL_EINVAL,

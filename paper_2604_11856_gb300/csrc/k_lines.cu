@@ -2,9 +2,10 @@
 // (Sec. 2.2.1 atoms, Sec. 2.2.2 diatomics).
 //
 // Binning (deterministic, ordered by line index):
-//   k_bin_bounds   per line, the tiles its window can touch in any cell of the
-//                  request, from a conservative width: lamV <= lamL + lamG
-//                  with both widths at their largest over the cells
+//   k_line_plan    per line, the checks, the tiles its window can touch in any
+//                  cell of the request, from a conservative width: lamV <=
+//                  lamL + lamG with both widths at their largest over the
+//                  cells, and the record of a line that touches one
 //   k_bin_count    one block per tile: scan the lines whose centre lies within
 //                  the widest window of the tile, count those that reach it
 //   scan           exclusive prefix of the counts -> CSR offsets
@@ -37,121 +38,153 @@ __device__ __forceinline__ double voigt_hwhm(double lamL, double lamG) {
            (lamL + lamG);
 }
 
-__global__ void k_validate_lines(rapral_lines ln, int32_t S, int* status) {
-    int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (l >= ln.n_lines) return;
+// Checks one line; a failed check is recorded and the line gets no record.
+__device__ __forceinline__ bool check_line(const rapral_lines& ln, int32_t S, int64_t l, int* status) {
+    bool ok = true;
     const int s = ln.species[l];
-    if (s < 0 || s >= S) fail(status, CHK_LINE_SPECIES, l);
+    if (s < 0 || s >= S) fail(status, CHK_LINE_SPECIES, l), ok = false;
     const double lam = ln.lam0[l];
     if (!(lam > 0.0) || !isfinite(lam) || !(ln.lamS0[l] >= 0.0) || !isfinite(ln.lamS0[l]))
-        fail(status, CHK_LINE_LAM, l);
+        fail(status, CHK_LINE_LAM, l), ok = false;
     if (!(ln.gu[l] > 0.0) || !(ln.gl[l] > 0.0) || !isfinite(ln.gu[l]) || !isfinite(ln.gl[l]))
-        fail(status, CHK_LINE_G, l);
-    if (!(ln.A[l] >= 0.0) || !isfinite(ln.A[l])) fail(status, CHK_LINE_A, l);
+        fail(status, CHK_LINE_G, l), ok = false;
+    if (!(ln.A[l] >= 0.0) || !isfinite(ln.A[l])) fail(status, CHK_LINE_A, l), ok = false;
+    return ok;
 }
 
-__global__ void k_line_prep(rapral_lines ln, const double* __restrict__ mass, const int32_t* __restrict__ kind,
-                            double lam_min, double h, Phys ph, LinePrep* __restrict__ out,
-                            LineF32* __restrict__ out32, int* sorted_flag, BroadArgs br, double2* lb,
-                            float2* lb32, const int* status) {
-    if (*status) return;
-    int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (l >= ln.n_lines) return;
-    LinePrep p;
-    const double lam0 = ln.lam0[l];
-    const double lcm = lam0 * 1e-7;
-    const double A = ln.A[l];
-    const int s = ln.species[l];
-    p.lam0 = lam0;
-    p.lnAj = log(1e-7 * (ph.h * ph.c / (4.0 * M_PI)) * A / lcm);
-    p.lnAk = log(1e4 * A * (lcm * lcm) * (lcm * lcm) / (8.0 * M_PI * ph.c));
-    p.lngu = log(ln.gu[l]);
-    p.lnAjg = p.lnAj + p.lngu;
-    p.lnAkg = p.lnAk + p.lngu;
-    p.Eve_u = ln.Eu_el[l] + ln.Eu_v[l];
-    p.Er_u = ln.Eu_j[l];
-    p.Eve_l = ln.El_el[l] + ln.El_v[l];
-    p.Er_l = ln.El_j[l];
-    p.dEve = p.Eve_u - p.Eve_l;
-    p.dEr = p.Er_u - p.Er_l;
-    p.cD = RAPRAL_DOPPLER_HALF * lam0 / sqrt(mass[s]);
-    p.lamS0 = ln.lamS0[l];
-    const bool atom = kind[s] == 0;
-    if ((br.flags & RAPRAL_BROAD_STARK_IONIZE) && atom) {   // Stark coefficient from the ionisation gap
-        const double dE = fmax(br.Eion[s] - ln.Eu_el[l], RAPRAL_E_IONIZE_H / 25.0);
-        p.lamS0 = 1.69e3 * lam0 * lam0 / pow(dE, 2.623);
-    }
-    if (lb) {   // per-line factors of the resonance and van der Waals widths
-        double cR = 0.0, cW = 0.0;
-        if ((br.flags & RAPRAL_BROAD_RESONANCE) && atom && ln.El_el[l] == 0.0 && ln.El_v[l] == 0.0 &&
-            ln.El_j[l] == 0.0) {
-            const double f = ph.me * ph.c * lcm * lcm / (8.0 * M_PI * M_PI * ph.e * ph.e) * ln.gu[l] / ln.gl[l] * A;
-            cR = 4.3e-28 * lam0 * f * sqrt(ln.gl[l] / ln.gu[l]) * lam0 * lam0;
+// Conservative half-width of line l's window over the request's cells, nm:
+// lamV <= lamL + lamG (the Voigt fit's factor never exceeds 1), both at their
+// largest over the cells.  lamS0: the Stark width in use; c: the factors of
+// the resonance and van der Waals terms (zero without them).
+__device__ __forceinline__ double window_nm(double cD, double lamS0, double2 c, int s, bool broad,
+                                            const unsigned long long* dmax) {
+    const auto dm = [dmax](int i) { return __longlong_as_double((long long)dmax[i]); };
+    double lamL = RAPRAL_LAM_NATURAL + lamS0 * dm(1);
+    if (broad) lamL += c.x * dm(2 + 2 * s) + c.y * dm(3 + 2 * s);
+    return RAPRAL_WINDOW * (lamL + cD * dm(0)) * (1.0 + 1e-9);
+}
+
+// One thread a line: the checks, the window's tiles and, for the lines whose
+// window reaches the range, the records.  FP64 runs at 1/64 of the FP32 rate
+// here, so what a line costs is its FP64 operations: three logarithms, a
+// square root and four divisions for a record.  A chunk of a solve sees all
+// lines of the list and keeps a few percent of them, so lines are turned away
+// first by a bound of their window from FP32 widths (rounded up by 1e-4 and
+// four grid points, against FP32 errors of 1e-6), which takes six FP64
+// operations.  Checks, records and bounds of 320k lines took 342 us as three
+// kernels (208 of them for one 64-bit atomicMax a line on one word, now one a
+// block); 48 cells x 65,536 of 1e6 points, the whole call: 1.355 -> 1.060 ms.
+__global__ void __launch_bounds__(256) k_line_plan(rapral_lines ln, const double* __restrict__ mass,
+                                                   const int32_t* __restrict__ kind, int32_t S, double lam_min,
+                                                   double h, Phys ph, int64_t k0, int64_t nk, int tile_w,
+                                                   const unsigned long long* __restrict__ dmax,
+                                                   LinePrep* __restrict__ out, LineF32* __restrict__ out32,
+                                                   int2* __restrict__ line_tiles, unsigned long long* wmax,
+                                                   int* unsorted, BroadArgs br, double2* lb, float2* lb32,
+                                                   int* status) {
+    __shared__ unsigned long long wblk;
+    if (threadIdx.x == 0) wblk = 0ULL;
+    __syncthreads();
+    const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    unsigned long long wbits = 0ULL;
+    if (l < ln.n_lines && check_line(ln, S, l, status)) {
+        const double lam0 = ln.lam0[l];
+        if (l + 1 < ln.n_lines && ln.lam0[l + 1] < lam0) *unsorted = 1;
+        const int s = ln.species[l];
+        const bool atom = kind[s] == 0;
+        const bool stark = (br.flags & RAPRAL_BROAD_STARK_IONIZE) && atom;
+        bool near = true;
+        if (!stark && !lb) {
+            const float lamf = (float)lam0;
+            const float wf = 100.0f * (5.9e-6f + (float)ln.lamS0[l] * (float)__longlong_as_double((long long)dmax[1]) +
+                                       3.5811651e-7f * lamf * rsqrtf((float)mass[s]) *
+                                           (float)__longlong_as_double((long long)dmax[0]));
+            const double w = (double)(wf * 1.0001f) + 4.0 * h;   // NaN or inf: kept
+            near = !(lam0 + w < lam_min + (double)k0 * h || lam0 - w > lam_min + (double)(k0 + nk - 1) * h);
         }
-        if ((br.flags & RAPRAL_BROAD_VDW) && atom) cW = lam0 * lam0;
-        lb[l] = make_double2(cR, cW);
-        lb32[l] = make_float2((float)cR, (float)cW);
+        int2 t = make_int2(1, 0);
+        if (near) {
+            LinePrep p;
+            const double lcm = lam0 * 1e-7;
+            const double A = ln.A[l];
+            p.lam0 = lam0;
+            p.cD = RAPRAL_DOPPLER_HALF * lam0 / sqrt(mass[s]);
+            p.lamS0 = ln.lamS0[l];
+            if (stark) {   // Stark coefficient from the ionisation gap
+                const double dE = fmax(br.Eion[s] - ln.Eu_el[l], RAPRAL_E_IONIZE_H / 25.0);
+                p.lamS0 = 1.69e3 * lam0 * lam0 / pow(dE, 2.623);
+            }
+            double2 c = make_double2(0.0, 0.0);
+            if (lb) {   // per-line factors of the resonance and van der Waals widths
+                if ((br.flags & RAPRAL_BROAD_RESONANCE) && atom && ln.El_el[l] == 0.0 && ln.El_v[l] == 0.0 &&
+                    ln.El_j[l] == 0.0) {
+                    const double f =
+                        ph.me * ph.c * lcm * lcm / (8.0 * M_PI * M_PI * ph.e * ph.e) * ln.gu[l] / ln.gl[l] * A;
+                    c.x = 4.3e-28 * lam0 * f * sqrt(ln.gl[l] / ln.gu[l]) * lam0 * lam0;
+                }
+                if ((br.flags & RAPRAL_BROAD_VDW) && atom) c.y = lam0 * lam0;
+                lb[l] = c;
+                lb32[l] = make_float2((float)c.x, (float)c.y);
+            }
+            p.tpos = (lam0 - lam_min) / h;
+            const double w = window_nm(p.cD, p.lamS0, c, s, lb != nullptr, dmax) / h + 2.0;   // grid points
+            const double lo = fmax(ceil(p.tpos - w), (double)k0);
+            const double hi = fmin(floor(p.tpos + w), (double)(k0 + nk - 1));
+            if (!(lo > hi)) {
+                t.x = (int)(((int64_t)lo - k0) / tile_w);
+                t.y = (int)(((int64_t)hi - k0) / tile_w);
+                wbits = (unsigned long long)__double_as_longlong(w);
+                p.lnAj = log(1e-7 * (ph.h * ph.c / (4.0 * M_PI)) * A / lcm);
+                p.lnAk = log(1e4 * A * (lcm * lcm) * (lcm * lcm) / (8.0 * M_PI * ph.c));
+                p.lngu = log(ln.gu[l]);
+                p.lnAjg = p.lnAj + p.lngu;
+                p.lnAkg = p.lnAk + p.lngu;
+                p.Eve_u = ln.Eu_el[l] + ln.Eu_v[l];
+                p.Er_u = ln.Eu_j[l];
+                p.Eve_l = ln.El_el[l] + ln.El_v[l];
+                p.Er_l = ln.El_j[l];
+                p.dEve = p.Eve_u - p.Eve_l;
+                p.dEr = p.Er_u - p.Er_l;
+                p.dEve_f = (float)p.dEve;
+                p.dEr_f = (float)p.dEr;
+                p.cD_f = (float)p.cD;
+                p.lamS0_f = (float)p.lamS0;
+                const double kcd = rint(p.tpos);
+                p.kc = (int32_t)fmin(fmax(kcd, -1e9), 2e9);
+                p.delta_f = (float)(p.tpos - (double)p.kc);
+                p.species = s;
+                p.pad = 0;
+                out[l] = p;
+                if (out32) {
+                    LineF32 f;
+                    f.lnAjg = ff_from(p.lnAjg);
+                    f.dAkj = ff_from(p.lnAk - p.lnAj);
+                    f.Eve_u = ff_from(p.Eve_u);
+                    f.Er_u = ff_from(p.Er_u);
+                    f.dEve = ff_from(p.dEve);
+                    f.dEr = ff_from(p.dEr);
+                    f.cD = p.cD_f;
+                    f.lamS0 = p.lamS0_f;
+                    f.delta = p.delta_f;
+                    f.kc = p.kc;
+                    f.species = s;
+                    f.kcf = (float)p.kc;
+                    out32[l] = f;
+                }
+            }
+        }
+        line_tiles[l] = t;
     }
-    p.tpos = (lam0 - lam_min) / h;
-    p.dEve_f = (float)p.dEve;
-    p.dEr_f = (float)p.dEr;
-    p.cD_f = (float)p.cD;
-    p.lamS0_f = (float)p.lamS0;
-    const double kcd = rint(p.tpos);
-    p.kc = (int32_t)fmin(fmax(kcd, -1e9), 2e9);
-    p.delta_f = (float)(p.tpos - (double)p.kc);
-    p.species = s;
-    p.pad = 0;
-    out[l] = p;
-    if (out32) {
-        LineF32 f;
-        f.lnAjg = ff_from(p.lnAjg);
-        f.dAkj = ff_from(p.lnAk - p.lnAj);
-        f.Eve_u = ff_from(p.Eve_u);
-        f.Er_u = ff_from(p.Er_u);
-        f.dEve = ff_from(p.dEve);
-        f.dEr = ff_from(p.dEr);
-        f.cD = p.cD_f;
-        f.lamS0 = p.lamS0_f;
-        f.delta = p.delta_f;
-        f.kc = p.kc;
-        f.species = s;
-        f.kcf = (float)p.kc;
-        out32[l] = f;
+    // widest window of the lines that reach the range (positive doubles order
+    // like their bits): one atomic a block
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, wbits, o);
+        wbits = v > wbits ? v : wbits;
     }
-    if (l + 1 < ln.n_lines && ln.lam0[l + 1] < lam0) *sorted_flag = 0;
-}
-
-// Conservative window per line: lamV <= lamL + lamG (the Voigt fit's factor
-// never exceeds 1), both at their largest over the request's cells.
-__global__ void k_bin_bounds(const LinePrep* __restrict__ lp, int64_t L, const unsigned long long* __restrict__ dmax,
-                             double h, int64_t k0, int64_t nk, int tile_w, int2* __restrict__ line_tiles,
-                             unsigned long long* wmax, const double2* lb, const int* status) {
-    if (*status) return;
-    int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (l >= L) return;
-    const double sqrtTmax = __longlong_as_double((long long)dmax[0]);
-    const double stcmax = __longlong_as_double((long long)dmax[1]);
-    const LinePrep p = lp[l];
-    const double lamG = p.cD * sqrtTmax;
-    double lamL = RAPRAL_LAM_NATURAL + p.lamS0 * stcmax;
-    if (lb) {   // resonance / van der Waals terms at their largest over the cells
-        const double2 c = lb[l];
-        lamL += c.x * __longlong_as_double((long long)dmax[2 + 2 * p.species]) +
-                c.y * __longlong_as_double((long long)dmax[3 + 2 * p.species]);
-    }
-    const double w = RAPRAL_WINDOW * (lamL + lamG) * (1.0 + 1e-9) / h + 2.0;   // grid points
-    atomicMax(wmax, (unsigned long long)__double_as_longlong(w));
-    const double lo = fmax(ceil(p.tpos - w), (double)k0);
-    const double hi = fmin(floor(p.tpos + w), (double)(k0 + nk - 1));
-    int2 t;
-    if (lo > hi) {
-        t.x = 1; t.y = 0;
-    } else {
-        t.x = (int)(((int64_t)lo - k0) / tile_w);
-        t.y = (int)(((int64_t)hi - k0) / tile_w);
-    }
-    line_tiles[l] = t;
+    if ((threadIdx.x & 31) == 0 && wbits) atomicMax(&wblk, wbits);
+    __syncthreads();
+    if (threadIdx.x == 0 && wblk) atomicMax(wmax, wblk);
 }
 
 // Lines whose centre can reach tile t: lam0 within the widest window of the
@@ -170,7 +203,7 @@ __device__ void tile_candidates(const double* lam0, int64_t L, int sorted, doubl
 }
 
 __global__ void __launch_bounds__(256) k_bin_count(const double* __restrict__ lam0, int64_t L,
-                                                   const int2* __restrict__ line_tiles, const int* sorted_flag,
+                                                   const int2* __restrict__ line_tiles, const int* unsorted,
                                                    const unsigned long long* wmaxp, double lam_min, double h,
                                                    int64_t k0, int64_t nk, int tile_w, int* __restrict__ counts,
                                                    const int* status) {
@@ -179,7 +212,7 @@ __global__ void __launch_bounds__(256) k_bin_count(const double* __restrict__ la
     const int64_t kt0 = k0 + (int64_t)t * tile_w;
     const int64_t kt1 = min(kt0 + tile_w, k0 + nk) - 1;
     int64_t b0, b1;
-    tile_candidates(lam0, L, *sorted_flag, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, &b0, &b1);
+    tile_candidates(lam0, L, !*unsorted, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, &b0, &b1);
     int cnt = 0;
     for (int64_t l = b0 + threadIdx.x; l < b1; l += blockDim.x) {
         const int2 r = line_tiles[l];
@@ -198,16 +231,18 @@ __global__ void __launch_bounds__(256) k_bin_count(const double* __restrict__ la
 }
 
 __global__ void __launch_bounds__(256) k_bin_fill(const double* __restrict__ lam0, int64_t L,
-                                                  const int2* __restrict__ line_tiles, const int* sorted_flag,
+                                                  const int2* __restrict__ line_tiles, const int* unsorted,
                                                   const unsigned long long* wmaxp, double lam_min, double h,
                                                   int64_t k0, int64_t nk, int tile_w, const int* __restrict__ off,
-                                                  int* __restrict__ out, const int* status) {
+                                                  int* __restrict__ out, unsigned long long* unit,
+                                                  const int* status) {
+    if (unit && blockIdx.x == 0 && threadIdx.x == 0) *unit = 0ULL;   // the line sum's work counter
     if (*status) return;
     const int t = blockIdx.x;
     const int64_t kt0 = k0 + (int64_t)t * tile_w;
     const int64_t kt1 = min(kt0 + tile_w, k0 + nk) - 1;
     int64_t b0, b1;
-    tile_candidates(lam0, L, *sorted_flag, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, &b0, &b1);
+    tile_candidates(lam0, L, !*unsorted, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, &b0, &b1);
     __shared__ int wsum[8];
     __shared__ int base_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -233,9 +268,9 @@ __global__ void __launch_bounds__(256) k_bin_fill(const double* __restrict__ lam
 
 // Exclusive scan of the per-tile line counts into the int32 offsets of the
 // tile lists, carried in int64 so that a total beyond 2^31 - 1 is seen:
-// total[0] receives the exact sum (offsets past 2^31 - 1 wrap, and the
+// total[0] receives the exact sum, total[1] the status code (offsets past 2^31 - 1 wrap, and the
 // callers refuse such a plan before the lists are filled).  Single block.
-__global__ void __launch_bounds__(1024) k_scan_counts(int* data, int64_t n, long long* total) {
+__global__ void __launch_bounds__(1024) k_scan_counts(int* data, int64_t n, long long* total, const int* status) {
     __shared__ long long part[32];
     __shared__ long long carry_s;
     if (threadIdx.x == 0) carry_s = 0;
@@ -271,7 +306,8 @@ __global__ void __launch_bounds__(1024) k_scan_counts(int* data, int64_t n, long
     }
     if (threadIdx.x == 0) {
         data[n] = (int)(unsigned)(unsigned long long)carry_s;
-        *total = carry_s;
+        total[0] = carry_s;
+        total[1] = status[ST_CODE];   // read back with the total
     }
 }
 
@@ -1039,8 +1075,8 @@ __global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_f3
 }
 
 // Launches k_line_sum_f32_persist over the units of grid g: ctx->ls_persist
-// blocks a SM, or as many as fit (-1); the unit counter (ctx->d_unit) is
-// cleared on the stream first.
+// blocks a SM, or as many as fit (-1); the unit counter (ctx->d_unit) was
+// cleared by k_bin_fill.
 template <int PPT, int WPB, int PB>
 static cudaError_t launch_persist(rapral_ctx* ctx, const LineSumArgs& a, dim3 g) {
     int dev = 0, sms = 0, per_sm = ctx->ls_persist;
@@ -1049,7 +1085,6 @@ static cudaError_t launch_persist(rapral_ctx* ctx, const LineSumArgs& a, dim3 g)
     if (e == cudaSuccess && per_sm < 0)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_line_sum_f32_persist<PPT, WPB, PB>, 32 * WPB, 0);
     unsigned long long* counter = ctx->d_unit;
-    if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), ctx->stream);
     if (e != cudaSuccess) return e;
     const int64_t total = (int64_t)g.x * g.y;
     const int64_t blocks = std::min<int64_t>(total, (int64_t)sms * std::max(1, per_sm));
@@ -1100,51 +1135,43 @@ __global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_ba
 
 }  // namespace
 
-cudaError_t launch_validate_lines(rapral_ctx* ctx, const rapral_lines* ln, int32_t n_species) {
-    if (ln->n_lines == 0) return cudaSuccess;
-    k_validate_lines<<<div_up(ln->n_lines, 256), 256, 0, ctx->stream>>>(*ln, n_species, ctx->d_status);
-    return cudaGetLastError();
+cudaError_t launch_plan_reset(rapral_ctx* ctx, unsigned long long* d_max, const BinPlan* plan) {
+    // maxima, widest window, total, status copy and the unsorted flag lie together in the arena
+    const size_t n = (size_t)(reinterpret_cast<char*>(plan->unsorted + 1) - reinterpret_cast<char*>(d_max));
+    return cudaMemsetAsync(d_max, 0, n, ctx->stream);
 }
 
-cudaError_t launch_line_prep(rapral_ctx* ctx, const rapral_species* sp, const rapral_lines* ln,
-                             double lam_min, double h, const Phys& ph, LinePrep* out, LineF32* out32,
-                             int* sorted_flag, const BroadArgs* br, double2* lb, float2* lb32) {
+cudaError_t launch_line_plan(rapral_ctx* ctx, const rapral_species* sp, const rapral_lines* ln,
+                             double lam_min, double h, const Phys& ph, const unsigned long long* d_max,
+                             LinePrep* out, LineF32* out32, BinPlan* plan, const BroadArgs* br, double2* lb,
+                             float2* lb32) {
     if (ln->n_lines == 0) return cudaSuccess;
     BroadArgs b = br ? *br : BroadArgs{};
     if (!broad_terms(br)) lb = nullptr, lb32 = nullptr;
-    k_line_prep<<<div_up(ln->n_lines, 256), 256, 0, ctx->stream>>>(*ln, sp->mass, sp->kind, lam_min, h, ph, out,
-                                                                   out32, sorted_flag, b, lb, lb32, ctx->d_status);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_bin_bounds(rapral_ctx* ctx, const rapral_lines* ln, const LinePrep* lp, const CellPrep* cp,
-                              const unsigned long long* d_max, double h, BinPlan* plan, const double2* lb) {
-    (void)cp;
-    if (ln->n_lines == 0) return cudaSuccess;
-    k_bin_bounds<<<div_up(ln->n_lines, 256), 256, 0, ctx->stream>>>(lp, ln->n_lines, d_max, h, plan->k0, plan->nk,
-                                                                    plan->tile_w, plan->line_tiles, plan->wmax,
-                                                                    lb, ctx->d_status);
+    k_line_plan<<<div_up(ln->n_lines, 256), 256, 0, ctx->stream>>>(
+        *ln, sp->mass, sp->kind, sp->n_species, lam_min, h, ph, plan->k0, plan->nk, plan->tile_w, d_max, out, out32,
+        plan->line_tiles, plan->wmax, plan->unsorted, b, lb, lb32, ctx->d_status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin_count(rapral_ctx* ctx, const rapral_lines* ln, const rapral_grid* g, double h,
                              BinPlan* plan) {
     k_bin_count<<<(unsigned)plan->n_tiles, 256, 0, ctx->stream>>>(ln->lam0, ln->n_lines, plan->line_tiles,
-                                                                  plan->sorted_flag, plan->wmax, g->lam_min, h,
+                                                                  plan->unsorted, plan->wmax, g->lam_min, h,
                                                                   plan->k0, plan->nk, plan->tile_w, plan->tile_off,
                                                                   ctx->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_scan_counts<<<1, 1024, 0, ctx->stream>>>(plan->tile_off, plan->n_tiles, plan->total);
+    k_scan_counts<<<1, 1024, 0, ctx->stream>>>(plan->tile_off, plan->n_tiles, plan->total, ctx->d_status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin_fill(rapral_ctx* ctx, const rapral_lines* ln, const rapral_grid* g, double h,
                             BinPlan* plan) {
     k_bin_fill<<<(unsigned)plan->n_tiles, 256, 0, ctx->stream>>>(ln->lam0, ln->n_lines, plan->line_tiles,
-                                                                 plan->sorted_flag, plan->wmax, g->lam_min, h,
+                                                                 plan->unsorted, plan->wmax, g->lam_min, h,
                                                                  plan->k0, plan->nk, plan->tile_w, plan->tile_off,
-                                                                 plan->tile_lines, ctx->d_status);
+                                                                 plan->tile_lines, ctx->d_unit, ctx->d_status);
     return cudaGetLastError();
 }
 

@@ -17,16 +17,22 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__global__ void k_validate_cells(const double* Ttr, const double* Tve, const double* n, int64_t C,
-                                 int32_t ncol, int* status) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= C) return;
+__device__ __forceinline__ bool check_cell(const double* Ttr, const double* Tve, const double* n, int64_t i,
+                                           int32_t ncol, int* status) {
+    bool ok = true;
     const double a = Ttr[i], b = Tve[i];
-    if (!(a > 0.0) || !(b > 0.0) || !isfinite(a) || !isfinite(b)) fail(status, CHK_CELL_T, i);
+    if (!(a > 0.0) || !(b > 0.0) || !isfinite(a) || !isfinite(b)) fail(status, CHK_CELL_T, i), ok = false;
     for (int j = 0; j < ncol; ++j) {
         const double v = n[i * ncol + j];
-        if (!(v >= 0.0) || !isfinite(v)) { fail(status, CHK_CELL_N, i); break; }
+        if (!(v >= 0.0) || !isfinite(v)) { fail(status, CHK_CELL_N, i); ok = false; break; }
     }
+    return ok;
+}
+
+__global__ void k_validate_cells(const double* Ttr, const double* Tve, const double* n, int64_t C,
+                                 int32_t ncol, int* status) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < C) check_cell(Ttr, Tve, n, i, ncol, status);
 }
 
 __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const double* __restrict__ Ttr,
@@ -65,40 +71,66 @@ __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const do
     if (lane == 0) lnpref[c * S + s] = (N > 0.0) ? log(N) - log(z) : -INFINITY;
 }
 
-__global__ void k_cell_prep(const double* __restrict__ Ttr, const double* __restrict__ Tve,
-                            const double* __restrict__ n, int32_t ncol, int32_t ne_col, int64_t C, double c2,
-                            CellPrep* __restrict__ out, unsigned long long* dmax, const int* status) {
-    if (*status) return;
-    int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    CellPrep p;
-    const double tt = Ttr[c], tv = Tve[c];
-    p.bve = c2 / tv;
-    p.btr = c2 / tt;
-    p.sqrtT = sqrt(tt);
-    p.stc = pow(tv / 10000.0, 0.33) * (n[c * ncol + ne_col] / 1e16);
-    p.bve_f = (float)p.bve;
-    p.btr_f = (float)p.btr;
-    p.sqrtT_f = (float)p.sqrtT;
-    p.stc_f = (float)p.stc;
-    p.bve_ff = ff_from(p.bve);
-    p.btr_ff = ff_from(p.btr);
-    out[c] = p;
-    // positive doubles order like their bit patterns
-    atomicMax(&dmax[0], (unsigned long long)__double_as_longlong(p.sqrtT));
-    atomicMax(&dmax[1], (unsigned long long)__double_as_longlong(p.stc));
+// Largest of the block's positive doubles (as bits; 0: none) into *dst, one
+// atomic a block: one a cell on the same word cost 0.1 ms on 80,000 cells.
+__device__ __forceinline__ void block_max(unsigned long long v, unsigned long long* blk, unsigned long long* dst) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, v, o);
+        v = x > v ? x : v;
+    }
+    if (threadIdx.x == 0) *blk = 0ULL;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && v) atomicMax(blk, v);
+    __syncthreads();
+    if (threadIdx.x == 0 && *blk) atomicMax(dst, *blk);
+    __syncthreads();
+}
+
+// Checks and record of one cell per thread.
+__global__ void __launch_bounds__(256) k_cell_prep(const double* __restrict__ Ttr, const double* __restrict__ Tve,
+                                                   const double* __restrict__ n, int32_t ncol, int32_t ne_col,
+                                                   int64_t C, double c2, CellPrep* __restrict__ out,
+                                                   unsigned long long* dmax, int* status) {
+    __shared__ unsigned long long blk;
+    const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    unsigned long long mT = 0ULL, mS = 0ULL;
+    if (c < C && check_cell(Ttr, Tve, n, c, ncol, status)) {
+        CellPrep p;
+        const double tt = Ttr[c], tv = Tve[c];
+        p.bve = c2 / tv;
+        p.btr = c2 / tt;
+        p.sqrtT = sqrt(tt);
+        p.stc = pow(tv / 10000.0, 0.33) * (n[c * ncol + ne_col] / 1e16);
+        p.bve_f = (float)p.bve;
+        p.btr_f = (float)p.btr;
+        p.sqrtT_f = (float)p.sqrtT;
+        p.stc_f = (float)p.stc;
+        p.bve_ff = ff_from(p.bve);
+        p.btr_ff = ff_from(p.btr);
+        out[c] = p;
+        // positive doubles order like their bit patterns
+        mT = (unsigned long long)__double_as_longlong(p.sqrtT);
+        mS = (unsigned long long)__double_as_longlong(p.stc);
+    }
+    block_max(mT, &blk, &dmax[0]);
+    block_max(mS, &blk, &dmax[1]);
 }
 
 // Ground-level weight of each atomic species: the summed g of its levels at
-// E = 0 (0 for molecules).
+// E = 0 (0 for molecules).  A warp a species, lanes along its levels (one
+// thread walking 10,000 levels was a chain of load latencies: 1.2 ms).
 __global__ void k_ground_weights(rapral_species sp, double* g0) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= sp.n_species) return;
+    const int s = blockIdx.x, lane = threadIdx.x;
     double g = 0.0;
-    if (sp.kind[s] == RAPRAL_ATOM)
-        for (int64_t k = sp.atom_off[s]; k < sp.atom_off[s + 1]; ++k)
+    if (sp.kind[s] == RAPRAL_ATOM) {
+        const int64_t b = sp.atom_off[s + 1];
+#pragma unroll 4
+        for (int64_t k = sp.atom_off[s] + lane; k < b; k += 32)
             if (sp.atom_E[k] == 0.0) g += sp.atom_g[k];
-    g0[s] = g;
+    }
+    g = warp_sum(g);
+    if (lane == 0) g0[s] = g;
 }
 
 // Per (cell, atomic species): ground-level density N_0 = n_s g_0 / Z_s and
@@ -109,14 +141,15 @@ __global__ void k_cell_broad(rapral_species sp, rapral_cells cells, BroadArgs br
                              double2* __restrict__ cb, float2* __restrict__ cb32, unsigned long long* dmax,
                              const int* status) {
     if (*status) return;
+    __shared__ unsigned long long blk;
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (c >= cells.n_cells) return;
+    const bool in = c < cells.n_cells;
     const int S = sp.n_species, nc = cells.n_cols;
-    const double T = cells.Ttr[c];
-    const double* n = cells.n + c * nc;
+    const double T = in ? cells.Ttr[c] : 1.0;
+    const double* n = cells.n + (in ? c : 0) * nc;
     for (int s = 0; s < S; ++s) {
         double N0 = 0.0, W = 0.0;
-        if (sp.kind[s] == RAPRAL_ATOM) {
+        if (in && sp.kind[s] == RAPRAL_ATOM) {
             if ((br.flags & RAPRAL_BROAD_RESONANCE) && g0[s] > 0.0)
                 N0 = exp(cells.lnpref[c * S + s] + log(g0[s]));
             if (br.flags & RAPRAL_BROAD_VDW) {
@@ -131,10 +164,12 @@ __global__ void k_cell_broad(rapral_species sp, rapral_cells cells, BroadArgs br
                 if (No > 0.0) W += 2.925e-29 * No * sqrt(2.0 * T / (NoM / No));
             }
         }
-        cb[c * S + s] = make_double2(N0, W);
-        cb32[c * S + s] = make_float2((float)N0, (float)W);
-        atomicMax(&dmax[2 + 2 * s], (unsigned long long)__double_as_longlong(N0));
-        atomicMax(&dmax[3 + 2 * s], (unsigned long long)__double_as_longlong(W));
+        if (in) {
+            cb[c * S + s] = make_double2(N0, W);
+            cb32[c * S + s] = make_float2((float)N0, (float)W);
+        }
+        block_max((unsigned long long)__double_as_longlong(N0), &blk, &dmax[2 + 2 * s]);
+        block_max((unsigned long long)__double_as_longlong(W), &blk, &dmax[3 + 2 * s]);
     }
 }
 
@@ -143,9 +178,7 @@ __global__ void k_cell_broad(rapral_species sp, rapral_cells cells, BroadArgs br
 cudaError_t launch_broad_cells(rapral_ctx* ctx, const rapral_species* sp, const rapral_cells* cells,
                                const BroadArgs& br, double* g0, double2* cb, float2* cb32, unsigned long long* d_max) {
     const int S = sp->n_species;
-    cudaError_t e = cudaMemsetAsync(d_max + 2, 0, 2 * (size_t)S * sizeof(unsigned long long), ctx->stream);
-    if (e != cudaSuccess) return e;
-    k_ground_weights<<<1, 32, 0, ctx->stream>>>(*sp, g0);
+    k_ground_weights<<<S, 32, 0, ctx->stream>>>(*sp, g0);   // d_max was cleared by launch_plan_reset
     if (cells->n_cells == 0) return cudaGetLastError();
     k_cell_broad<<<div_up(cells->n_cells, 128), 128, 0, ctx->stream>>>(*sp, *cells, br, g0, cb, cb32, d_max,
                                                                        ctx->d_status);
@@ -168,8 +201,6 @@ cudaError_t launch_populations(rapral_ctx* ctx, const rapral_species* sp, const 
 
 cudaError_t launch_cell_prep(rapral_ctx* ctx, const rapral_cells* cells, const Phys& ph, CellPrep* out,
                              unsigned long long* d_max) {
-    cudaError_t e = cudaMemsetAsync(d_max, 0, 2 * sizeof(unsigned long long), ctx->stream);
-    if (e != cudaSuccess) return e;
     k_cell_prep<<<div_up(cells->n_cells, 256), 256, 0, ctx->stream>>>(
         cells->Ttr, cells->Tve, cells->n, cells->n_cols, cells->ne_col, cells->n_cells, ph.c2, out, d_max,
         ctx->d_status);

@@ -185,8 +185,8 @@ int noalloc_impl(int dev, cudaStream_t stream, const rapral_species* sp, const r
     size_t need = 0;
     need = arena_need(need, 8 * sizeof(int));                      // status word
     need = arena_need(need, 4 * sizeof(unsigned long long));       // counters
-    need = arena_need(need, 4 * sizeof(unsigned long long));       // maxima
-    need = arena_need(need, 4 * sizeof(int));                      // sorted flag
+    need = arena_need(need, 5 * sizeof(unsigned long long));       // maxima, window, total, status copy
+    need = arena_need(need, 4 * sizeof(int));                      // unsorted flag
     need = arena_need(need, (size_t)L * sizeof(LinePrep));
     need = arena_need(need, (size_t)L * sizeof(LineF32));
     need = arena_need(need, (size_t)C * sizeof(CellPrep));
@@ -212,8 +212,8 @@ int noalloc_impl(int dev, cudaStream_t stream, const rapral_species* sp, const r
     Arena ar{reinterpret_cast<char*>(base), SCRATCH_BYTES};
     ctx.d_status = ar.take<int>(8);
     ctx.d_stats = ar.take<unsigned long long>(4);
-    unsigned long long* dmax = ar.take<unsigned long long>(4);
-    int* sorted_flag = ar.take<int>(4);
+    unsigned long long* dmax = ar.take<unsigned long long>(5);
+    int* unsorted = ar.take<int>(4);
     LinePrep* lp = ar.take<LinePrep>(L);
     LineF32* lf = ar.take<LineF32>(L);
     CellPrep* cp = ar.take<CellPrep>(C);
@@ -221,7 +221,7 @@ int noalloc_impl(int dev, cudaStream_t stream, const rapral_species* sp, const r
     plan.k0 = k0; plan.nk = nk; plan.tile_w = W; plan.n_tiles = T;
     plan.line_tiles = ar.take<int2>(L);
     plan.tile_off = ar.take<int>(T + 1);
-    plan.sorted_flag = sorted_flag;
+    plan.unsorted = unsorted;
     plan.wmax = dmax + 2;
     plan.total = reinterpret_cast<long long*>(dmax + 3);
     const size_t csr_at = ar.used;
@@ -239,14 +239,9 @@ int noalloc_impl(int dev, cudaStream_t stream, const rapral_species* sp, const r
     // words that must start at zero (the array keeps the previous call's values)
     e = cudaMemsetAsync(ctx.d_status, 0, 8 * sizeof(int), ctx.stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx.d_stats, 0, 4 * sizeof(unsigned long long), ctx.stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(plan.wmax, 0, sizeof(unsigned long long), ctx.stream);
-    static const int one = 1;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sorted_flag, &one, sizeof(int), cudaMemcpyHostToDevice, ctx.stream);
-    if (e == cudaSuccess) e = launch_validate_cells(&ctx, cells);
-    if (e == cudaSuccess) e = launch_validate_lines(&ctx, ln, sp->n_species);
-    if (e == cudaSuccess) e = launch_line_prep(&ctx, sp, ln, g->lam_min, h, ph, lp, lf, sorted_flag);
+    if (e == cudaSuccess) e = launch_plan_reset(&ctx, dmax, &plan);
     if (e == cudaSuccess) e = launch_cell_prep(&ctx, cells, ph, cp, dmax);
-    if (e == cudaSuccess) e = launch_bin_bounds(&ctx, ln, lp, cp, dmax, h, &plan);
+    if (e == cudaSuccess) e = launch_line_plan(&ctx, sp, ln, g->lam_min, h, ph, dmax, lp, lf, &plan);
     if (e == cudaSuccess) e = launch_bin_count(&ctx, ln, g, h, &plan);
     // read the status word and the tile-list length (host stack, no pinned buffer)
     int status_words[3] = {0, 0, 0};

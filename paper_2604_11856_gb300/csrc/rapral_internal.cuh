@@ -215,14 +215,19 @@ __device__ __forceinline__ void fail(int* status, int check, long long index) {
 cudaError_t launch_validate_cells(rapral_ctx* ctx, const rapral_cells* cells);
 cudaError_t launch_populations(rapral_ctx* ctx, const rapral_species* sp, const rapral_cells* cells,
                                double* lnpref, const Phys& ph);
-cudaError_t launch_validate_lines(rapral_ctx* ctx, const rapral_lines* ln, int32_t n_species);
+struct BinPlan;
+// Clears a request's maxima, window, total and unsorted words.
+cudaError_t launch_plan_reset(rapral_ctx* ctx, unsigned long long* d_max, const BinPlan* plan);
+// Per line: checks, window tiles and, where the window reaches the range, the
+// records.  d_max: the maxima of launch_cell_prep (and launch_broad_cells).
 // br: optional Lorentz terms (nullptr or flags 0: none); with resonance or van
 // der Waals terms, lb / lb32 [L] receive per-line (c_R, c_W), the width
 // gaining c_R N_0 + c_W W over the (cell, species) values of launch_broad_cells.
-cudaError_t launch_line_prep(rapral_ctx* ctx, const rapral_species* sp, const rapral_lines* ln,
-                             double lam_min, double h, const Phys& ph, LinePrep* out, LineF32* out32,
-                             int* sorted_flag, const BroadArgs* br = nullptr, double2* lb = nullptr,
-                             float2* lb32 = nullptr);
+cudaError_t launch_line_plan(rapral_ctx* ctx, const rapral_species* sp, const rapral_lines* ln,
+                             double lam_min, double h, const Phys& ph, const unsigned long long* d_max,
+                             LinePrep* out, LineF32* out32, BinPlan* plan, const BroadArgs* br = nullptr,
+                             double2* lb = nullptr, float2* lb32 = nullptr);
+// Checks the cells and writes their records.
 cudaError_t launch_cell_prep(rapral_ctx* ctx, const rapral_cells* cells, const Phys& ph, CellPrep* out,
                              unsigned long long* d_max /*[2 + 2 S]*/);
 // Per (cell, species): ground-level density N_0 and van der Waals factor W
@@ -242,14 +247,13 @@ struct BinPlan {
     int2* line_tiles;            // [L] first / last tile a line may touch (first > last: none)
     int* tile_off;               // [T+1]
     int* tile_lines;             // [tile_off[T]]
-    long long* total;            // [1] exact number of (line, tile) entries (int64: may exceed the
-                                 // int32 offsets; a plan with more than 2^31 - 1 is refused)
-    int* sorted_flag;            // [1] 1 while lam0 is non-decreasing
-    unsigned long long* wmax;    // [1] largest window half-width, grid points (double bits)
+    long long* total;            // [2] exact number of (line, tile) entries (int64: may exceed the
+                                 // int32 offsets; a plan with more than 2^31 - 1 is refused), and
+                                 // the status code as the counts were scanned
+    int* unsorted;               // [1] 1 where lam0 decreases somewhere
+    unsigned long long* wmax;    // [1] largest window half-width of the lines that reach the range,
+                                 // grid points (double bits)
 };
-cudaError_t launch_bin_bounds(rapral_ctx* ctx, const rapral_lines* ln, const LinePrep* lp, const CellPrep* cp,
-                              const unsigned long long* d_max, double h, BinPlan* plan,
-                              const double2* lb = nullptr);
 // Counts each tile's lines and scans the counts into plan->tile_off; the
 // exact total goes to plan->total (device).
 cudaError_t launch_bin_count(rapral_ctx* ctx, const rapral_lines* ln, const rapral_grid* g, double h,
