@@ -12,28 +12,15 @@
 
 namespace {
 
-// Segment coefficients: e = e^{-dtau}, far-node coefficient ca = (f - e)/kappa
-// and near-node coefficient cb = (1 - f)/kappa, f = (1 - e)/dtau, with their
-// series for small |dtau|.
-//   FP64: |dtau| < 4e-4 takes three terms of each series; e from expm1.
-//   FP32: |dtau| < 0.5 takes seven terms (truncation <= 4e-7 relative), so
-//   the closed form is used only where 1 - e >= 0.39 and an approximate ex2
-//   for e keeps FP32 accuracy without expm1f.
-__device__ __forceinline__ void seg_coeffs(double kap, double s, double inv_k, double /*inv_s*/, double* e,
-                                           double* ca, double* cb) {
-    const double dtau = kap * s;
-    const double em1 = expm1(-dtau);   // e^{-dtau} - 1
-    *e = 1.0 + em1;
-    if (fabs(dtau) < RAPRAL_THIN_F64) {
-        *ca = s * (0.5 - dtau * (1.0 / 3.0) + dtau * dtau * 0.125);
-        *cb = s * (0.5 - dtau * (1.0 / 6.0) + dtau * dtau * (1.0 / 24.0));
-    } else {
-        const double f = -em1 / dtau;
-        *ca = (f - *e) * inv_k;
-        *cb = (1.0 - f) * inv_k;
-    }
-}
-
+// One segment of the march for one direction is I <- I e + ca j_far + cb j_near
+// with t = dtau, e = e^{-t}, f = (1 - e)/t, the far-node coefficient
+// ca = (f - e)/kappa and the near-node coefficient cb = (1 - f)/kappa.  With
+// p = (1 - f)/t = sum_n (-t)^n / (n + 2)! it is
+//   I + s B,  A = j_far - kappa I,  B = A + p ((j_near - j_far) - t A),
+// which takes no exponential and no division where the series is short: FP64
+// for |t| < 1/2, FP32 (seven terms, truncation below 4e-8 relative) likewise;
+// beyond, the closed form loses at most two bits to 1 - e >= 0.39, and FP32
+// takes e from an approximate ex2.
 __device__ __forceinline__ float ex2f_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -46,18 +33,58 @@ __device__ __forceinline__ float recip(float x) {
     return y;
 }
 
-// The same coefficients for one direction per segment: the closed form takes
-// a single reciprocal, of dtau, inside its branch (1/kappa = s / dtau).
-__device__ __forceinline__ void seg_coeffs1(double kap, double s, double* e, double* ca, double* cb) {
-    seg_coeffs(kap, s, 1.0 / kap, 0.0, e, ca, cb);
+// FP64.  The FP64 pipe has 1/64 of the FP32 rate here, so a step costs its
+// count of FP64 operations.  The series is entered at the length |t| needs
+// (truncation below 1e-17 relative: 3 terms below 2^-17, 5 below 2^-10, 9
+// below 2^-4, 14 below 1/2; the lanes of a warp share the tail), and |t| is
+// compared by its high word on the integer pipe.  A thin step is 8 to 20 FP64
+// operations; with an expm1 and two divisions whatever its t it took the
+// time of 75 (61 cells x 25 directions x 100,001 points: 18.6 -> 5.6 ms).
+constexpr int T64_17 = 0x3EE00000, T64_10 = 0x3F500000, T64_4 = 0x3FB00000, T64_1 = 0x3FE00000;   // 2^-k
+__device__ __forceinline__ int abs_hi(double t) { return __double2hiint(t) & 0x7fffffff; }
+__device__ __forceinline__ double thin_series(double t, int hi) {
+    double p;
+    if (hi < T64_17) {
+        p = 1.0 / 24.0;
+    } else {
+        if (hi < T64_10) {
+            p = 1.0 / 720.0;
+        } else {
+            if (hi < T64_4) {
+                p = 1.0 / 3628800.0;
+            } else {
+                p = fma(t, -1.0 / 1307674368000.0, 1.0 / 87178291200.0);
+                p = fma(t, p, -1.0 / 6227020800.0);
+                p = fma(t, p, 1.0 / 479001600.0);
+                p = fma(t, p, -1.0 / 39916800.0);
+                p = fma(t, p, 1.0 / 3628800.0);
+            }
+            p = fma(t, p, -1.0 / 362880.0);
+            p = fma(t, p, 1.0 / 40320.0);
+            p = fma(t, p, -1.0 / 5040.0);
+            p = fma(t, p, 1.0 / 720.0);
+        }
+        p = fma(t, p, -1.0 / 120.0);
+        p = fma(t, p, 1.0 / 24.0);
+    }
+    p = fma(t, p, -1.0 / 6.0);
+    return fma(t, p, 0.5);
 }
-// One segment of the march for one direction: I <- I e + ca j_far + cb j_near.
-// FP32 folds the common factor of ca and cb (s, or s / dtau) into one
-// multiply: I e + m (a j_far + b j_near).
+__device__ __noinline__ double thick_step(double I, double kf, double t, double jf, double jn) {
+    const double em1 = expm1(-t), ik = 1.0 / kf;
+    const double f = -em1 / t, e = 1.0 + em1;
+    return I * e + (f - e) * ik * jf + (1.0 - f) * ik * jn;
+}
 __device__ __forceinline__ void seg_step(double& I, double kf, double s, double jf, double jn) {
-    double e, ca, cb;
-    seg_coeffs1(kf, s, &e, &ca, &cb);
-    I = I * e + ca * jf + cb * jn;
+    const double t = kf * s;
+    const int hi = abs_hi(t);
+    if (hi < T64_1) {
+        const double p = thin_series(t, hi);
+        const double A = fma(-kf, I, jf);
+        I = fma(s, fma(p, fma(-t, A, jn - jf), A), I);
+    } else {
+        I = thick_step(I, kf, t, jf, jn);
+    }
 }
 // FP32, thin (|dtau| < 0.5): with p = (1 - f)/dtau from its series
 // p = sum_n (-dtau)^n / (n + 2)!, n = 0..6 (truncation below 4e-8 relative)
@@ -116,17 +143,33 @@ __device__ __forceinline__ void seg_step2(float& I0, float& I1, float k0, float 
     }
 }
 
-// the MAXD directions of one column: packed in pairs in FP32
+// The nd directions of one column (nd <= MAXD, the same for the whole warp):
+// packed in pairs in FP32.  FP64 shares kappa s, s j_far and s (j_near -
+// j_far) of the common length s between the directions.
 template <class T, int MAXD>
-__device__ __forceinline__ void dir_steps(T (&I)[MAXD], T kf, T ds, const T* sc, T jf, T jn) {
-    if constexpr (sizeof(T) == 4 && MAXD > 1) {
+__device__ __forceinline__ void dir_steps(T (&I)[MAXD], T kf, T ds, const T* sc, int nd, T jf, T jn) {
+    if constexpr (MAXD == 1) {
+        seg_step(I[0], kf, ds, jf, jn);
+    } else if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int d = 0; d + 1 < MAXD; d += 2)
             seg_step2(I[d], I[d + 1], kf, kf, ds * sc[d], ds * sc[d + 1], jf, jf, jn, jn);
         if (MAXD & 1) seg_step(I[MAXD - 1], kf, ds * sc[MAXD - 1], jf, jn);
     } else {
+        const T t0 = kf * ds, jd = ds * jf, dj = ds * (jn - jf);
 #pragma unroll
-        for (int d = 0; d < MAXD; ++d) seg_step(I[d], kf, MAXD == 1 ? ds : ds * sc[d], jf, jn);
+        for (int d = 0; d < MAXD; ++d) {
+            if (d >= nd) break;
+            const T t = t0 * sc[d];
+            const int hi = abs_hi(t);
+            if (hi < T64_1) {
+                const T p = thin_series(t, hi);
+                const T A = fma(-t0, I[d], jd);
+                I[d] = fma(sc[d], fma(p, fma(-t, A, dj), A), I[d]);
+            } else {
+                I[d] = thick_step(I[d], kf, t, jf, jn);
+            }
+        }
     }
 }
 
@@ -333,7 +376,7 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
                 seg_step2(I[0][0], I[1][0], kf[0], kf[1], ds, ds, jf[0], jf[1], jn[0], jn[1]);
             } else {
 #pragma unroll
-                for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, jf[v], jn[v]);
+                for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, nd, jf[v], jn[v]);
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -349,7 +392,7 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
             seg_step2(I[0][0], I[1][0], kf[0], kf[1], ds, ds, jf[0], jf[1], jc[0], jc[1]);
         } else {
 #pragma unroll
-            for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, jf[v], jc[v]);
+            for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, nd, jf[v], jc[v]);
         }
     }
 }
