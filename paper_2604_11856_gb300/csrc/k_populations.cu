@@ -1,13 +1,14 @@
 // Populations (Sec. 2.1) and per-cell preparation.
 //
-// k_populations: one warp per (cell, species).  Atoms: lanes stride over the
-// level list and sum g exp(-c2 E / T_ve).  Diatomics: lanes stride over the
-// rotational ladder of each (state, V) and add
+// k_populations: one block per (cell group, species).  Atoms: threads stride
+// over the level list and sum g exp(-c2 E / T_ve).  Diatomics: threads stride
+// over the rotational quantum number of each state and add
 //   g_i exp(-c2 E_i / T_ve) exp(-c2 E_V / T_ve) / sigma (2J+1) L_alter exp(-c2 E_J / T_tr),
-// which is the product form of g_i exp(-c2E_i/T_ee) Q_vr,i.  One fixed-order
-// warp reduction per (cell, species) keeps the result deterministic.  FP64
+// which is the product form of g_i exp(-c2E_i/T_ee) Q_vr,i.  Fixed-order warp
+// and block reductions keep the result deterministic.  FP64 accuracy
 // throughout (partition sums are FP64 in both precisions).
 #include "rapral_internal.cuh"
+#include "exp_fix.cuh"
 
 namespace {
 
@@ -35,40 +36,96 @@ __global__ void k_validate_cells(const double* Ttr, const double* Tve, const dou
     if (i < C) check_cell(Ttr, Tve, n, i, ncol, status);
 }
 
+// A block: one species, CC cells, its 256 threads along the levels (atoms) or
+// the rotational ladders (diatomics).  What a term costs is its exponential;
+// with expfix_boltzmann it is 95 integer operations and one FP64 multiply-add
+// beside them (exp(double) kept the FP64 pipe busy at 21 operation times a
+// term: 5000 cells, 53,000 terms a cell, 9.7 -> 1.2 ms).  A level is read and
+// turned into fixed point once for its CC cells.
+// The order of a cell's sum does not depend on CC.
+template <int CC>
 __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const double* __restrict__ Ttr,
                                                      const double* __restrict__ Tve, const double* __restrict__ n,
                                                      int32_t ncol, int64_t C, double c2, double* __restrict__ lnpref,
                                                      const int* status) {
     if (*status) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int S = sp.n_species;
-    if (w >= C * S) return;
-    const int64_t c = w / S;
-    const int s = (int)(w - c * S);
-    const double bve = c2 / Tve[c], btr = c2 / Ttr[c];
-    const double N = n[c * ncol + sp.density_col[s]];
-    double z = 0.0;
+    __shared__ uint64_t tab[EXPFIX_N];
+    __shared__ double pv[CC][32];      // Boltzmann factors of 32 vibrational levels of a state, with its weight
+    __shared__ double red[CC][8];
+    expfix_load(tab);
+    const int S = sp.n_species, s = blockIdx.y;
+    const int64_t c0 = (int64_t)blockIdx.x * CC;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double bve[CC], btr[CC], z[CC];
+    ExpFixScale sc[CC];
+#pragma unroll
+    for (int q = 0; q < CC; ++q) {
+        const int64_t c = c0 + q < C ? c0 + q : C - 1;
+        bve[q] = c2 / Tve[c];
+        btr[q] = c2 / Ttr[c];
+        z[q] = 0.0;
+    }
+    __syncthreads();
     if (sp.kind[s] == RAPRAL_ATOM) {
-        const int64_t a = sp.atom_off[s], b = sp.atom_off[s + 1];
-        for (int64_t l = a + lane; l < b; l += 32) z += sp.atom_g[l] * exp(-bve * sp.atom_E[l]);
+        const int64_t b = sp.atom_off[s + 1];
+#pragma unroll
+        for (int q = 0; q < CC; ++q) sc[q] = expfix_scale(bve[q]);
+        for (int64_t l = sp.atom_off[s] + tid; l < b; l += 256) {
+            const double E = sp.atom_E[l], g = sp.atom_g[l];
+            const uint64_t Ef = expfix_energy(E);
+#pragma unroll
+            for (int q = 0; q < CC; ++q) z[q] = fma(g, expfix_boltzmann(Ef, sc[q], E, bve[q], tab), z[q]);
+        }
     } else {
-        const int64_t a = sp.st_off[s], b = sp.st_off[s + 1];
-        for (int64_t i = a; i < b; ++i) {
-            const double pre = sp.st_g[i] * exp(-bve * sp.st_E[i]) / sp.st_sigma[i];
+#pragma unroll
+        for (int q = 0; q < CC; ++q) sc[q] = expfix_scale(btr[q]);
+        for (int64_t i = sp.st_off[s]; i < sp.st_off[s + 1]; ++i) {
             const int nv = sp.st_nv[i], nj = sp.st_nj[i];
             const double La = sp.st_Lalt[2 * i], Lb = sp.st_Lalt[2 * i + 1];
             const double* rot = sp.rot_E + sp.st_rot_off[i];
             const double* vib = sp.vib_E + sp.st_vib_off[i];
-            for (int v = 0; v < nv; ++v) {
-                const double pv = pre * exp(-bve * vib[v]);
-                for (int J = lane; J < nj; J += 32)
-                    z += pv * ((2.0 * J + 1.0) * ((J & 1) ? Lb : La) * exp(-btr * rot[(int64_t)v * nj + J]));
+            for (int v0 = 0; v0 < nv; v0 += 32) {
+                const int nvc = nv - v0 < 32 ? nv - v0 : 32;
+                __syncthreads();
+                for (int x = tid; x < CC * nvc; x += 256) {   // a (cell, level) a thread
+                    const int q = x / nvc, v = x - q * nvc;
+                    const int64_t c = c0 + q < C ? c0 + q : C - 1;
+                    const double b = c2 / Tve[c];
+                    pv[q][v] = sp.st_g[i] * exp_fix(-b * sp.st_E[i], tab) / sp.st_sigma[i] *
+                               exp_fix(-b * vib[v0 + v], tab);
+                }
+                __syncthreads();
+                for (int J = tid; J < nj; J += 256) {
+                    double y[CC];
+#pragma unroll
+                    for (int q = 0; q < CC; ++q) y[q] = 0.0;
+                    for (int v = 0; v < nvc; ++v) {
+                        const double E = rot[(int64_t)(v0 + v) * nj + J];
+                        const uint64_t Ef = expfix_energy(E);
+#pragma unroll
+                        for (int q = 0; q < CC; ++q)
+                            y[q] = fma(pv[q][v], expfix_boltzmann(Ef, sc[q], E, btr[q], tab), y[q]);
+                    }
+                    const double w = (2.0 * J + 1.0) * ((J & 1) ? Lb : La);
+#pragma unroll
+                    for (int q = 0; q < CC; ++q) z[q] = fma(w, y[q], z[q]);
+                }
             }
         }
     }
-    z = warp_sum(z);
-    if (lane == 0) lnpref[c * S + s] = (N > 0.0) ? log(N) - log(z) : -INFINITY;
+#pragma unroll
+    for (int q = 0; q < CC; ++q) {
+        z[q] = warp_sum(z[q]);
+        if (lane == 0) red[q][warp] = z[q];
+    }
+    __syncthreads();
+    if (tid < CC && c0 + tid < C) {
+        const int64_t c = c0 + tid;
+        double Z = red[tid][0];
+        for (int w = 1; w < 8; ++w) Z += red[tid][w];
+        const double N = n[c * ncol + sp.density_col[s]];
+        lnpref[c * S + s] = (N > 0.0) ? log(N) - log(Z) : -INFINITY;
+    }
 }
 
 // Largest of the block's positive doubles (as bits; 0: none) into *dst, one
@@ -193,9 +250,15 @@ cudaError_t launch_validate_cells(rapral_ctx* ctx, const rapral_cells* cells) {
 
 cudaError_t launch_populations(rapral_ctx* ctx, const rapral_species* sp, const rapral_cells* cells,
                                double* lnpref, const Phys& ph) {
-    const int64_t warps = cells->n_cells * sp->n_species;
-    k_populations<<<div_up(warps * 32, 256), 256, 0, ctx->stream>>>(
-        *sp, cells->Ttr, cells->Tve, cells->n, cells->n_cols, cells->n_cells, ph.c2, lnpref, ctx->d_status);
+    // Four cells a block share a level's load and conversion; one cell a block
+    // where four would leave the chip with fewer than eight blocks an SM
+    const int64_t C = cells->n_cells, S = sp->n_species;
+    if (C * S >= 4 * 152 * 8)
+        k_populations<4><<<dim3(div_up(C, 4), (unsigned)S), 256, 0, ctx->stream>>>(
+            *sp, cells->Ttr, cells->Tve, cells->n, cells->n_cols, C, ph.c2, lnpref, ctx->d_status);
+    else
+        k_populations<1><<<dim3((unsigned)C, (unsigned)S), 256, 0, ctx->stream>>>(
+            *sp, cells->Ttr, cells->Tve, cells->n, cells->n_cols, C, ph.c2, lnpref, ctx->d_status);
     return cudaGetLastError();
 }
 
