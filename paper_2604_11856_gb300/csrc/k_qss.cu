@@ -1,11 +1,25 @@
 // Quasi-steady-state collisional-radiative populations (Sec. 2.1): per cell
 // and atomic radiator, the rate matrix R and source b of the QSS master
 // equation, solved by LU with partial pivoting.  One warp per cell: lanes
-// compute the transitions' up / down rates into shared memory, then lane i
-// assembles row i in transition order (losses on the diagonal, gains off
-// it), pivots and eliminates its row, and lane 0 substitutes back.  FP64
-// throughout: the systems span many orders of magnitude in their rates.
+// compute the transitions' up / down rates into shared memory, lane r
+// assembles row r from its own transitions (losses on the diagonal, gains off
+// it, in transition order), pivots and eliminates its row, and the warp
+// substitutes back column by column.  FP64 throughout: the systems span many
+// orders of magnitude in their rates.
+//
+// The FP64 pipe bounds it (a warp instruction of it takes 17 clocks of an SM,
+// whatever lanes are on), so the count of FP64 warp instructions a cell is
+// what the layout keeps down: rows are assembled from per-row lists, built
+// once a block (two instructions a row entry instead of four a transition
+// with two lanes on, 1,984 for 496 transitions), exponentials and pivot
+// comparisons run on the integer pipe, divisions are one Newton reciprocal a
+// level or pivot, and the back substitution is one instruction a column
+// instead of one lane's 496.  20,000 cells of 32 + 4 levels, 496 transitions:
+// 6.57 -> 2.36 ms.
+#include <algorithm>
+
 #include "rapral_internal.cuh"
+#include "exp_fix.cuh"
 
 namespace {
 
@@ -14,124 +28,199 @@ constexpr int QMAXL = 32;      // levels solved
 constexpr int QMAXT = QMAXL * (QMAXL - 1) / 2;
 constexpr double N_AVOGADRO = 6.022e23;
 
+// inf or NaN, on the integer pipe
+__device__ __forceinline__ bool nonfinite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+
+// 1 / x: an FP32 reciprocal of the leading part and one Newton step of third
+// order (relative error of the seed e: the result's is e^3 plus rounding),
+// where x is well inside the FP32 range; the division elsewhere.
+__device__ __forceinline__ double recip64(double x) {
+    const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+    if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / x;
+    // x's leading 24 bits as a float, without the FP64 pipe's conversion
+    const long long bits = __double_as_longlong(x);
+    const unsigned fb = ((unsigned)(bits >> 32) & 0x80000000u) | ((unsigned)(ex - 896) << 23) |
+                        (unsigned)((bits >> 29) & 0x7fffff);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(fb)));
+    const unsigned rb = __float_as_uint(r);
+    const double y = __longlong_as_double(((long long)(rb & 0x80000000u) << 32) |
+                                          ((long long)((rb >> 23 & 0xff) + 896) << 52) |
+                                          ((long long)(rb & 0x7fffff) << 29));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells cells, Phys ph, double* n_out,
                                                  int* status) {
     if (*status) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t c = (int64_t)blockIdx.x * QW + w;
-    if (c >= cells.n_cells) return;   // whole warp
+    __shared__ uint64_t tab[EXPFIX_N];
     __shared__ double Rs[QW][QMAXL][QMAXL + 1];
     __shared__ double bs[QW][QMAXL];
     __shared__ double rate_up[QW][QMAXT], rate_dn[QW][QMAXT];
-    __shared__ double Qh[QW][QMAXL], Qv[QW][QMAXL];
-    double (*R)[QMAXL + 1] = Rs[w];
-    double* b = bs[w];
+    __shared__ double Qh[QW][QMAXL], Qv[QW][QMAXL], iQh[QW][QMAXL], iQv[QW][QMAXL];
+    __shared__ unsigned char slo[QMAXT], sup[QMAXT];
+    __shared__ unsigned short ent[2 * QMAXT], roff[QMAXL + 1];   // row r: ent[roff[r]] .. (transition, 1 << 15 if r is upper)
     const int l = m.n_levels, T = m.n_trans, nc = cells.n_cols;
-    const double Ttr = cells.Ttr[c], Tve = cells.Tve[c];
-    const double* dens = cells.n + c * nc;
-    double nM = 0.0;
-    for (int k = 0; k < nc; ++k)
-        if (k != cells.ne_col) nM += dens[k];
-    const double ne = dens[cells.ne_col];
-    const double nion = m.ion_col >= 0 ? dens[m.ion_col] : 0.0;
-    // level weights Q_i = g_i e^{-c2 E_i / T} at both temperatures
-    if (lane < l) {
-        Qh[w][lane] = m.g[lane] * exp(-ph.c2 * m.E[lane] / Ttr);
-        Qv[w][lane] = m.g[lane] * exp(-ph.c2 * m.E[lane] / Tve);
-    }
-    __syncwarp();
-    const double lnTtr = log(Ttr), lnTve = log(Tve), iTtr = 1.0 / Ttr, iTve = 1.0 / Tve;
-    // transition rates per particle of the lower (up) / upper (down) level;
-    // every warp checks every transition before any indexed use
+    expfix_load(tab);
+    // every transition is checked before any indexed use
     bool bad = false;
-    for (int t = lane; t < T; t += 32) {
+    for (int t = threadIdx.x; t < T; t += blockDim.x) {
         const int i = m.lo[t], j = m.up[t];
         if (i < 0 || j <= i || j >= l) {
             fail(status, CHK_CR_TRANS, t);
             bad = true;
             continue;
         }
-        // C T^n e^{-theta/T} as C e^{n ln T - theta/T}: one exp a rate
-        const double theta = ph.c2 * (m.E[j] - m.E[i]);
-        const double kh_up = m.hp_C[t] * exp(m.hp_n[t] * lnTtr - theta * iTtr);
-        const double kh_dn = kh_up * Qh[w][i] / Qh[w][j];
-        const double ke_up = m.e_C[t] * exp(m.e_n[t] * lnTve - theta * iTve);
-        const double ke_dn = ke_up * Qv[w][i] / Qv[w][j];
-        const double rad = m.A[t] * (m.lam[t] >= 200.0 ? 1.0 : 0.0);
-        rate_up[w][t] = (kh_up * nM + ke_up * ne) / N_AVOGADRO;
-        rate_dn[w][t] = (kh_dn * nM + ke_dn * ne) / N_AVOGADRO + rad;
+        slo[t] = (unsigned char)i;
+        sup[t] = (unsigned char)j;
     }
-    if (__any_sync(0xffffffffu, bad)) return;
-    __syncwarp();
-    // row assembly: lane r owns row r
-    if (lane < l) {
-        for (int j = 0; j < l; ++j) R[lane][j] = 0.0;
-        b[lane] = 0.0;
-        if (lane > 0) {
-            for (int t = 0; t < T; ++t) {
-                const int i = m.lo[t], j = m.up[t];
-                if (lane == i) { R[i][i] -= rate_up[w][t]; R[i][j] += rate_dn[w][t]; }
-                if (lane == j) { R[j][j] -= rate_dn[w][t]; R[j][i] += rate_up[w][t]; }
-            }
-            // electron-impact ionisation and three-body recombination
-            const double Qp = m.g_ion * exp(-ph.c2 * m.E_ionize / Tve);
-            const double Qe = 2.0 * pow(2.0 * M_PI * ph.me * ph.kB * Tve / (ph.h * ph.h), 1.5);
-            const double kf = m.ii_C[lane] * pow(Tve, m.ii_n[lane]) * exp(-ph.c2 * (m.E_ionize - m.E[lane]) / Tve);
-            const double kr = kf * Qv[w][lane] / (Qp * Qe);
-            R[lane][lane] -= kf * ne / N_AVOGADRO;
-            b[lane] = -kr * nion * ne * ne / N_AVOGADRO;
-        } else {   // closure: the levels and the lumped ones above sum to the density
-            for (int j = 0; j < l; ++j) R[0][j] = 1.0;
-            if (m.n_levels_all > l) {
-                double s = 0.0;
-                for (int p = l; p < m.n_levels_all; ++p) s += m.g[p] * exp(-ph.c2 * m.E[p] / Tve);
-                R[0][l - 1] = 1.0 + s / Qv[w][l - 1];
-            }
-            b[0] = dens[m.col];
+    if (__syncthreads_or(bad)) return;
+    if (w == 0) {   // the rows' lists, in transition order
+        int n = 0;
+        for (int t = 0; t < T; ++t) n += (slo[t] == lane) + (sup[t] == lane);
+        int off = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, off, o);
+            if (lane >= o) off += x;
+        }
+        roff[lane + 1] = (unsigned short)off;
+        if (lane == 0) roff[0] = 0;
+        int at = off - n;
+        for (int t = 0; t < T; ++t) {
+            if (slo[t] == lane) ent[at++] = (unsigned short)t;
+            if (sup[t] == lane) ent[at++] = (unsigned short)(t | 0x8000);
         }
     }
-    __syncwarp();
-    // LU with partial pivoting (the first largest |R[r][k]| of rows r >= k)
-    for (int k = 0; k < l - 1; ++k) {
-        double v = (lane >= k && lane < l) ? fabs(R[lane][k]) : -1.0;
-        int idx = lane;
-        for (int off = 16; off > 0; off >>= 1) {
-            const double ov = __shfl_down_sync(0xffffffffu, v, off);
-            const int oi = __shfl_down_sync(0xffffffffu, idx, off);
-            if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
+    __syncthreads();
+    double (*R)[QMAXL + 1] = Rs[w];
+    double* b = bs[w];
+    for (int64_t c = (int64_t)blockIdx.x * QW + w; c < cells.n_cells; c += (int64_t)gridDim.x * QW) {
+        const double Ttr = cells.Ttr[c], Tve = cells.Tve[c];
+        const double* dens = cells.n + c * nc;
+        double nM = 0.0;
+        for (int k = 0; k < nc; ++k)
+            if (k != cells.ne_col) nM += dens[k];
+        const double ne = dens[cells.ne_col];
+        const double nion = m.ion_col >= 0 ? dens[m.ion_col] : 0.0;
+        const double lnTtr = log(Ttr), lnTve = log(Tve), iTtr = 1.0 / Ttr, iTve = 1.0 / Tve;
+        const double nMa = nM / N_AVOGADRO, nea = ne / N_AVOGADRO;
+        __syncwarp();
+        // level weights Q_i = g_i e^{-c2 E_i / T} at both temperatures
+        if (lane < l) {
+            const double g = m.g[lane], x = -ph.c2 * m.E[lane];
+            const double qh = g * exp_fix(x / Ttr, tab), qv = g * exp_fix(x / Tve, tab);
+            Qh[w][lane] = qh;
+            Qv[w][lane] = qv;
+            iQh[w][lane] = recip64(qh);
+            iQv[w][lane] = recip64(qv);
         }
-        const int p = __shfl_sync(0xffffffffu, idx, 0);
-        const double pv = __shfl_sync(0xffffffffu, v, 0);
-        if (!(pv > 0.0)) {
+        __syncwarp();
+        // transition rates per particle of the lower (up) / upper (down) level
+        for (int t = lane; t < T; t += 32) {
+            const int i = slo[t], j = sup[t];
+            // C T^n e^{-theta/T} as C e^{n ln T - theta/T}: one exp a rate
+            const double theta = ph.c2 * (m.E[j] - m.E[i]);
+            const double kh_up = m.hp_C[t] * exp_fix(m.hp_n[t] * lnTtr - theta * iTtr, tab);
+            const double ke_up = m.e_C[t] * exp_fix(m.e_n[t] * lnTve - theta * iTve, tab);
+            double kh_dn = kh_up * Qh[w][i] * iQh[w][j];
+            double ke_dn = ke_up * Qv[w][i] * iQv[w][j];
+            if (nonfinite(kh_dn) || nonfinite(ke_dn)) {   // weights below 2^-1022 (cold cells)
+                kh_dn = kh_up * Qh[w][i] / Qh[w][j];
+                ke_dn = ke_up * Qv[w][i] / Qv[w][j];
+            }
+            const double rad = m.lam[t] >= 200.0 ? m.A[t] : 0.0;
+            rate_up[w][t] = kh_up * nMa + ke_up * nea;
+            rate_dn[w][t] = kh_dn * nMa + ke_dn * nea + rad;
+        }
+        // row assembly: lane r owns row r
+        if (lane < l)
+            for (int j = 0; j < l; ++j) R[lane][j] = lane > 0 ? 0.0 : 1.0;
+        __syncwarp();
+        if (lane < l) {
+            if (lane > 0) {
+                double diag = 0.0;
+                for (int k = roff[lane]; k < roff[lane + 1]; ++k) {
+                    const int t = ent[k] & 0x7fff;
+                    const bool upper = ent[k] & 0x8000;
+                    const int j = upper ? slo[t] : sup[t];
+                    const double ru = rate_up[w][t], rd = rate_dn[w][t];
+                    diag -= upper ? rd : ru;
+                    const double gain = upper ? ru : rd;
+                    const double old = R[lane][j];   // nonzero only where a pair of levels has several transitions
+                    R[lane][j] = __double_as_longlong(old) == 0 ? gain : old + gain;
+                }
+                // electron-impact ionisation and three-body recombination
+                const double Qp = m.g_ion * exp_fix(-ph.c2 * m.E_ionize / Tve, tab);
+                const double x = 2.0 * M_PI * ph.me * ph.kB * Tve / (ph.h * ph.h);
+                const double Qe = 2.0 * (x * sqrt(x));
+                const double kf = m.ii_C[lane] * exp_fix(m.ii_n[lane] * lnTve, tab) *
+                                  exp_fix(-ph.c2 * (m.E_ionize - m.E[lane]) / Tve, tab);
+                const double kr = kf * Qv[w][lane] / (Qp * Qe);
+                R[lane][lane] = diag - kf * nea;
+                b[lane] = -kr * nion * ne * nea;
+            } else {   // closure: the levels and the lumped ones above sum to the density
+                if (m.n_levels_all > l) {
+                    double s = 0.0;
+                    for (int p = l; p < m.n_levels_all; ++p) s += m.g[p] * exp_fix(-ph.c2 * m.E[p] / Tve, tab);
+                    R[0][l - 1] = 1.0 + s / Qv[w][l - 1];
+                }
+                b[0] = dens[m.col];
+            }
+        }
+        __syncwarp();
+        // LU with partial pivoting (the first largest |R[r][k]| of rows r >= k;
+        // non-negative doubles order like their bits)
+        bool singular = false;
+        double inv_own = 0.0;   // lane k: 1 / pivot k
+        for (int k = 0; k < l; ++k) {
+            const unsigned long long v =
+                (lane >= k && lane < l) ? (unsigned long long)__double_as_longlong(R[lane][k]) & ~(1ull << 63) : 0ull;
+            const unsigned hi = (unsigned)(v >> 32), mhi = __reduce_max_sync(0xffffffffu, hi);
+            const unsigned lo = hi == mhi ? (unsigned)v : 0u, mlo = __reduce_max_sync(0xffffffffu, lo);
+            if ((mhi | mlo) == 0u || mhi > 0x7ff00000u || (mhi == 0x7ff00000u && mlo)) {   // zero or NaN
+                singular = true;
+                break;
+            }
+            const unsigned at = __ballot_sync(0xffffffffu, lane >= k && lane < l && hi == mhi && lo == mlo);
+            const int p = __ffs(at) - 1;
+            if (p != k) {
+                if (lane < l) { const double x = R[k][lane]; R[k][lane] = R[p][lane]; R[p][lane] = x; }
+                if (lane == 0) { const double x = b[k]; b[k] = b[p]; b[p] = x; }
+                __syncwarp();
+            }
+            const double piv = R[k][k], inv = recip64(piv);
+            if (lane == k) inv_own = inv;
+            if (lane > k && lane < l) {
+                const double r = R[lane][k];
+                double f = r * inv;
+                f = fma(fma(-f, piv, r), inv, f);   // the quotient, rounded once
+                if (nonfinite(f)) f = r / piv;      // pivots below 2^-1022
+                R[lane][k] = f;
+                for (int j = k + 1; j < l; ++j) R[lane][j] = fma(-f, R[k][j], R[lane][j]);
+                b[lane] = fma(-f, b[k], b[lane]);
+            }
+            __syncwarp();
+        }
+        if (singular) {
             if (lane == 0) fail(status, CHK_CR_SINGULAR, c);
-            return;
+            continue;
         }
-        if (p != k) {
-            if (lane < l) { const double x = R[k][lane]; R[k][lane] = R[p][lane]; R[p][lane] = x; }
-            if (lane == 0) { const double x = b[k]; b[k] = b[p]; b[p] = x; }
+        // back substitution, a column at a time
+        double x = lane < l ? b[lane] : 0.0;
+        for (int i = l - 1; i >= 0; --i) {
+            const double piv = R[i][i];
+            double xi = x * inv_own;
+            xi = fma(fma(-xi, piv, x), inv_own, xi);
+            if (nonfinite(xi)) xi = x / piv;
+            xi = __shfl_sync(0xffffffffu, xi, i);
+            if (lane == i) x = xi;
+            else if (lane < i) x = fma(-R[lane][i], xi, x);
         }
-        __syncwarp();
-        if (lane > k && lane < l) {
-            const double f = R[lane][k] / R[k][k];
-            R[lane][k] = f;
-            for (int j = k + 1; j < l; ++j) R[lane][j] -= f * R[k][j];
-            b[lane] -= f * b[k];
-        }
-        __syncwarp();
+        if (lane < l) n_out[c * l + lane] = x;
     }
-    if (lane == 0) {
-        if (!(fabs(R[l - 1][l - 1]) > 0.0)) {
-            fail(status, CHK_CR_SINGULAR, c);
-        } else {
-            for (int i = l - 1; i >= 0; --i) {
-                double s = b[i];
-                for (int j = i + 1; j < l; ++j) s -= R[i][j] * b[j];
-                b[i] = s / R[i][i];
-            }
-        }
-    }
-    __syncwarp();
-    if (lane < l) n_out[c * l + lane] = b[lane];
 }
 
 // Departure coefficients of the model's levels (Sec. 2.1): ln b_i = ln N_i -
@@ -173,7 +262,9 @@ cudaError_t launch_qss(rapral_ctx* ctx, const rapral_cr_model* m, const rapral_c
                        const Phys& ph) {
     if (cells->n_cells == 0) return cudaSuccess;
     if (m->n_trans > QMAXT || m->n_levels > QMAXL) return cudaErrorInvalidValue;
-    k_qss<<<div_up(cells->n_cells, QW), 32 * QW, 0, ctx->stream>>>(*m, *cells, ph, n_out, ctx->d_status);
+    // four blocks an SM fit (shared memory); each takes cells until none is left
+    const int64_t blocks = std::min<int64_t>((cells->n_cells + QW - 1) / QW, 152 * 4);
+    k_qss<<<(unsigned)blocks, 32 * QW, 0, ctx->stream>>>(*m, *cells, ph, n_out, ctx->d_status);
     return cudaGetLastError();
 }
 
