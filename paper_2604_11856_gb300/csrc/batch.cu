@@ -231,6 +231,8 @@ int rapral_batch_run(rapral_ctx* ctx, rapral_batch* B) {
     if (ctx->ev_after && e == cudaSuccess) e = cudaEventRecord(ctx->ev_after, ctx->stream);
     for (int i = 0; i < B->n && e == cudaSuccess; ++i) {
         const BatchReq& r = B->req[i];
+        e = launch_validate_rays(ctx, &r.rays, r.cells.n_cells, B->d_march[i]);   // and the march's FP32 copies
+        if (e != cudaSuccess) break;
         e = launch_march(ctx, &r.rays, r.kappa, r.emis, r.ld, &r.grid, r.h, r.k0, r.nk, RAPRAL_FP32, r.q_lambda,
                          nullptr, ph, B->d_march[i]);
         if (e == cudaSuccess)

@@ -409,7 +409,7 @@ int rapral_trace_rays(rapral_ctx* ctx, const rapral_rays* rays, int64_t n_cells,
     const Phys ph = make_phys(ctx->codata);
     st = ws_reserve(ctx, march_scratch_bytes(rays, nk, precision));
     if (st) return st;
-    cudaError_t e = launch_validate_rays(ctx, rays, n_cells);
+    cudaError_t e = launch_validate_rays(ctx, rays, n_cells, precision == RAPRAL_FP32 ? ctx->ws : nullptr);
     if (e == cudaSuccess)
         e = launch_march(ctx, rays, kappa, emis, ld, g, grid_h(g), k0, nk, precision, q_lambda, I_out, ph, ctx->ws);
     return cuda_status(ctx, e, "ray march");

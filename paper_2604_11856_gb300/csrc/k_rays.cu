@@ -173,18 +173,27 @@ __device__ __forceinline__ void dir_steps(T (&I)[MAXD], T kf, T ds, const T* sc,
     }
 }
 
-__global__ void k_validate_rays(const int32_t* seg_cell, const double* seg_ds, int64_t nseg, int64_t C,
-                                const double* dir_scale, int64_t ndir, int* status) {
+// Checks of the ray set and, with `f` (the FP32 march), the FP32 copies of
+// the path lengths (f), direction scales (fd) and weights (fw).
+__global__ void k_validate_rays(const int32_t* __restrict__ seg_cell, const double* __restrict__ seg_ds, int64_t nseg,
+                                int64_t C, const double* __restrict__ dir_scale,
+                                const double* __restrict__ dir_weight, int64_t ndir, float* __restrict__ f,
+                                float* __restrict__ fd, float* __restrict__ fw, int* status) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < nseg) {
         const int c = seg_cell[i];
         if (c < 0 || c >= C) fail(status, CHK_SEG_CELL, i);
         const double d = seg_ds[i];
         if (!(d >= 0.0) || !isfinite(d)) fail(status, CHK_SEG_DS, i);
+        if (f) f[i] = (float)d;
     }
     if (i < ndir) {
         const double s = dir_scale[i];
         if (!(s > 0.0) || !isfinite(s)) fail(status, CHK_DIR, i);
+        if (f) {
+            fd[i] = (float)s;
+            fw[i] = (float)dir_weight[i];
+        }
     }
 }
 
@@ -219,11 +228,6 @@ template <> __device__ __forceinline__ float seg_len<float>(const MarchArgs& a, 
 template <class T> __device__ __forceinline__ T dir_val(const double* d, const float* f, int64_t i);
 template <> __device__ __forceinline__ double dir_val<double>(const double* d, const float*, int64_t i) { return d[i]; }
 template <> __device__ __forceinline__ float dir_val<float>(const double*, const float* f, int64_t i) { return f[i]; }
-
-__global__ void k_to_float(const double* __restrict__ x, int64_t n, float* __restrict__ y) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = (float)x[i];
-}
 
 // Planck intensity, temperature form (Sec. 2.2), W/cm^2/sr/um.
 __device__ __forceinline__ double planck(double lam_nm, double T, const Phys& ph) {
@@ -516,13 +520,9 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ?
 //  * node values are carried doubled (K = kappa_a + kappa_b, the sum of the
 //    two cells at a face), with the segment length halved to match, which
 //    removes the averaging multiplies;
-//  * optically thin steps (|dtau| < 0.5) use I' = I + s f (j_f - kappa_f I)
-//    + s p (j_n - j_f), with p = (1 - f)/dtau from one degree-6 series and
-//    f = 1 - dtau p: one polynomial instead of two and no exponential.  With
-//    e = 1 - dtau f >= 0.6 the subtraction inside costs at most a factor
-//    1/e of relative rounding, so it stays in FP32 accuracy.  Thick steps use
-//    the exponential form I' = I e + s f j_f + s p (j_n - j_f) with
-//    f = (1 - e)/dtau, p = (1 - f)/dtau;
+//  * the step (m1_step) carries minus the intensity and minus the half length
+//    and takes the series as long as the depth needs;
+//  * equal rays of a point are marched once (k_ray_pairs);
 //  * the staged list holds, for step j, the segment's halved length (as the
 //    packed pair the step multiplies by) and the byte offset of the row of the
 //    cell PF steps ahead (row x ld, computed once by the staging lane), so a
@@ -547,77 +547,189 @@ constexpr int kM1Unroll = RAPRAL_M1_UNROLL;    // segment steps unrolled
 constexpr int M1_SLICES = 8;    // warps (bundle slices) per block
 
 struct __align__(16) M1Stage {
-    float2 sh;      // half the segment length (x the direction scale), twice: a packed pair
+    float2 nsh;     // minus half the segment length (x the direction scale), twice: a packed pair
     int64_t off;    // byte offset of the row of the cell step j + M1_PF needs (its next cell); 0 past the end
 };
 
-// The thin-step series p(t) = (1 - f)/t = sum_n (-t)^n / (n + 2)!, n = 0..6
-// (truncation below 4e-8 relative at |t| = 0.5), on a packed pair.
-__device__ __forceinline__ float2 m1_series(float2 t) {
-    const auto c2 = [](float c) { return make_float2(c, c); };
-    float2 p = __ffma2_rn(t, c2(1.0f / 40320.0f), c2(-1.0f / 5040.0f));
-    p = __ffma2_rn(t, p, c2(1.0f / 720.0f));
-    p = __ffma2_rn(t, p, c2(-1.0f / 120.0f));
-    p = __ffma2_rn(t, p, c2(1.0f / 24.0f));
-    p = __ffma2_rn(t, p, c2(-1.0f / 6.0f));
-    return __ffma2_rn(t, p, c2(0.5f));
-}
-
-// One step of one column with doubled node values Kf, Jf (far), Jn (near) and
-// half length sh: the thin or the thick form by |t|.
-__device__ __forceinline__ float m1_step1(float I, float Kf, float Jf, float Jn, float sh) {
-    const float t = Kf * sh;   // kappa_far x length
+// One step of one column with doubled node values Kf, Jf (far), Jn (near),
+// minus the half length, nsh, and minus the intensity, M.
+__device__ __forceinline__ float m1_step1(float M, float Kf, float Jf, float Jn, float nsh) {
+    const float t = Kf * nsh;   // minus kappa_far x length
+    const float dJ = Jn - Jf;
     if (fabsf(t) < (float)RAPRAL_THIN_F32) {
-        float p = fmaf(t, 1.0f / 40320.0f, -1.0f / 5040.0f);
+        float p = fmaf(t, 1.0f / 40320.0f, 1.0f / 5040.0f);
         p = fmaf(t, p, 1.0f / 720.0f);
-        p = fmaf(t, p, -1.0f / 120.0f);
+        p = fmaf(t, p, 1.0f / 120.0f);
         p = fmaf(t, p, 1.0f / 24.0f);
-        p = fmaf(t, p, -1.0f / 6.0f);
+        p = fmaf(t, p, 1.0f / 6.0f);
         p = fmaf(t, p, 0.5f);
-        const float f = fmaf(-t, p, 1.0f);
-        const float A = fmaf(-Kf, I, Jf);
-        return fmaf(sh, fmaf(f, A, p * (Jn - Jf)), I);
+        const float A = fmaf(Kf, M, Jf);
+        return fmaf(nsh, fmaf(p, fmaf(t, A, dJ), A), M);
     }
-    const float e = ex2f_approx(-1.44269504f * t);
+    const float e = ex2f_approx(1.44269504f * t);
     const float r = recip(t);
-    const float f = (1.0f - e) * r;
-    const float p = (1.0f - f) * r;
-    return fmaf(sh, fmaf(f, Jf, p * (Jn - Jf)), I * e);
+    const float f = (e - 1.0f) * r;
+    const float p = (f - 1.0f) * r;
+    return fmaf(nsh, fmaf(f, Jf, p * dJ), M * e);
 }
 
-// One step of both columns: packed when both are thin.
-__device__ __forceinline__ void m1_step(float2& I, float2 Kf, float2 Jf, float2 Jn, float2 sh2) {
-    const float sh = sh2.x;
-    const float2 t = __fmul2_rn(Kf, sh2);
-    if (fmaxf(fabsf(t.x), fabsf(t.y)) < (float)RAPRAL_THIN_F32) {
-        const float2 p = m1_series(t);
-        const float2 f = __ffma2_rn(make_float2(-t.x, -t.y), p, make_float2(1.0f, 1.0f));
-        const float2 A = __ffma2_rn(make_float2(-Kf.x, -Kf.y), I, Jf);
-        const float2 dJ = __fadd2_rn(Jn, make_float2(-Jf.x, -Jf.y));
-        const float2 B = __ffma2_rn(f, A, __fmul2_rn(p, dJ));
-        I = __ffma2_rn(sh2, B, I);
+// One step of both columns: packed when both are thin.  Carrying -I and -h
+// leaves no sign to flip (packed operands take none for free): 14 packed
+// operations, 11 where both depths are below 2^-5 (four terms of the series,
+// truncation 3e-9), as nearly all are.  FP32 and integer instructions share
+// one pipe here, and the march is bound by it: the form with signs, the full
+// series always and f beside p was 57 pipe slots for two columns.
+constexpr float M1_SHORT = 0.03125f;
+__device__ __forceinline__ void m1_step(float2& M, float2 Kf, float2 Jf, float2 Jn, float2 nsh) {
+    const float2 t = __fmul2_rn(Kf, nsh);
+    const float m = fmaxf(fabsf(t.x), fabsf(t.y));
+    if (m < (float)RAPRAL_THIN_F32) {
+        const auto c2 = [](float c) { return make_float2(c, c); };
+        float2 p = c2(1.0f / 120.0f);
+        if (m >= M1_SHORT) {
+            p = __ffma2_rn(t, c2(1.0f / 40320.0f), c2(1.0f / 5040.0f));
+            p = __ffma2_rn(t, p, c2(1.0f / 720.0f));
+            p = __ffma2_rn(t, p, c2(1.0f / 120.0f));
+        }
+        p = __ffma2_rn(t, p, c2(1.0f / 24.0f));
+        p = __ffma2_rn(t, p, c2(1.0f / 6.0f));
+        p = __ffma2_rn(t, p, c2(0.5f));
+        const float2 A = __ffma2_rn(Kf, M, Jf);
+        const float2 u = __ffma2_rn(t, A, __ffma2_rn(Jf, c2(-1.0f), Jn));
+        M = __ffma2_rn(nsh, __ffma2_rn(p, u, A), M);
     } else {
-        I.x = m1_step1(I.x, Kf.x, Jf.x, Jn.x, sh);
-        I.y = m1_step1(I.y, Kf.y, Jf.y, Jn.y, sh);
+        M.x = m1_step1(M.x, Kf.x, Jf.x, Jn.x, nsh.x);
+        M.y = m1_step1(M.y, Kf.y, Jf.y, Jn.y, nsh.x);
+    }
+}
+
+// Equal rays.  In an axisymmetric field a line of sight and its mirror image
+// cross the same cells with the same lengths, so half of the rays of such a
+// set repeat the other half: a ray whose cells, FP32 lengths, FP32 scale and
+// wall flag equal an earlier one's of its point, bit for bit, has the same
+// intensity bit for bit, and the two are marched once.  Whether a set has such
+// rays is found from its lists on every call (a hash a ray, then a full
+// comparison of the candidates); sets without them march as they are.  With
+// the step below, 100 x 50 cells, 20 points x 512 rays, 16,384 columns: 7.73 ->
+// 4.16 ms.
+constexpr int M1_PAIR_MAX = 2048;   // bundles of a point compared (16 KB of keys); more: no pairs
+
+__device__ __forceinline__ unsigned mix32(unsigned x) {
+    x ^= x >> 16; x *= 0x7feb352du;
+    x ^= x >> 15; x *= 0x846ca68bu;
+    return x ^ (x >> 16);
+}
+
+// key[b]: 64-bit hash of bundle b's segments, scale and wall flag (0: not one
+// direction, never paired).  One warp a bundle.
+__global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t B, unsigned long long* __restrict__ key) {
+    if (*a.status) return;
+    const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= B) return;
+    const int64_t s0 = a.seg_off[b], s1 = a.seg_off[b + 1], d0 = a.dir_off[b];
+    unsigned h0 = 0, h1 = 0;
+    for (int64_t i = s0 + lane; i < s1; i += 32) {
+        const unsigned x = mix32((unsigned)a.seg_cell[i] * 0x9e3779b1u + (unsigned)(i - s0));
+        const unsigned y = mix32(__float_as_uint(a.seg_ds_f[i]) ^ x);
+        h0 += y;
+        h1 += mix32(y + 0x68bc21ebu);
+    }
+    h0 = __reduce_add_sync(0xffffffffu, h0);
+    h1 = __reduce_add_sync(0xffffffffu, h1);
+    if (lane == 0) {
+        unsigned long long k = 0ULL;
+        if (a.dir_off[b + 1] - d0 == 1) {
+            h0 = mix32(h0 ^ __float_as_uint(a.dir_scale_f[d0]));
+            h1 = mix32(h1 + (unsigned)(s1 - s0) * 2u + (a.bundle_wall[b] != 0));
+            k = ((unsigned long long)h0 << 32 | h1) | 1ULL;
+        }
+        key[b] = k;
+    }
+}
+
+// Per point: partner[b] of every marched bundle (the equal bundle marched with
+// it, -1: none), and the marched bundles in index order (uniq, from the
+// point's first bundle) with their number (n_uniq).  A bundle of a key's odd
+// rank is the partner of the one before it, if the two are equal.
+__global__ void __launch_bounds__(256) k_ray_pairs(MarchArgs a, const unsigned long long* __restrict__ key,
+                                                   int32_t* __restrict__ partner, int32_t* __restrict__ uniq,
+                                                   int32_t* __restrict__ n_uniq) {
+    if (*a.status) return;
+    __shared__ unsigned long long ks[M1_PAIR_MAX];
+    __shared__ int16_t first[M1_PAIR_MAX];   // the bundle this one is a partner of, or -1
+    const int64_t pb0 = a.point_off[blockIdx.x];
+    const int64_t nb = a.point_off[blockIdx.x + 1] - pb0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) partner[pb0 + k] = -1;
+    if (nb > M1_PAIR_MAX) {
+        for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) uniq[pb0 + k] = (int32_t)(pb0 + k);
+        if (threadIdx.x == 0) n_uniq[blockIdx.x] = (int32_t)nb;
+        return;
+    }
+    const int n = (int)nb;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) ks[k] = key[pb0 + k];
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const unsigned long long x = ks[k];
+        int rank = 0, prev = -1;
+        for (int q = 0; q < k; ++q)
+            if (ks[q] == x) { ++rank; prev = q; }
+        first[k] = (int16_t)(x != 0ULL && (rank & 1) ? prev : -1);
+    }
+    __syncthreads();
+    for (int k = warp; k < n; k += blockDim.x >> 5) {   // the full comparison, a warp a candidate
+        const int q = first[k];
+        if (q < 0) continue;
+        const int64_t x0 = a.seg_off[pb0 + q], y0 = a.seg_off[pb0 + k];
+        const int64_t m = a.seg_off[pb0 + q + 1] - x0;
+        const int64_t dx = a.dir_off[pb0 + q], dy = a.dir_off[pb0 + k];
+        bool eq = m == a.seg_off[pb0 + k + 1] - y0 &&
+                  __float_as_uint(a.dir_scale_f[dx]) == __float_as_uint(a.dir_scale_f[dy]) &&
+                  (a.bundle_wall[pb0 + q] != 0) == (a.bundle_wall[pb0 + k] != 0);
+        for (int64_t i = lane; eq && i < m; i += 32)
+            eq = a.seg_cell[x0 + i] == a.seg_cell[y0 + i] &&
+                 __float_as_uint(a.seg_ds_f[x0 + i]) == __float_as_uint(a.seg_ds_f[y0 + i]);
+        eq = __all_sync(0xffffffffu, eq);
+        if (lane == 0) {
+            if (eq) partner[pb0 + q] = (int32_t)(pb0 + k);
+            else first[k] = -1;
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int out = 0;
+        for (int k0 = 0; k0 < n; k0 += 32) {
+            const bool keep = k0 + lane < n && first[k0 + lane] < 0;
+            const unsigned mk = __ballot_sync(0xffffffffu, keep);
+            if (keep) uniq[pb0 + out + __popc(mk & ((1u << lane) - 1u))] = (int32_t)(pb0 + k0 + lane);
+            out += __popc(mk);
+        }
+        if (lane == 0) n_uniq[blockIdx.x] = out;
     }
 }
 
 // Bundle plan: for each (point p, group g) the group's bundles (a contiguous
-// run of the point's bundles: with the rays of a point in angular order, the
-// neighbours a block marches cross the same cells near the point, which L1
-// then serves) dealt to M1_SLICES slices longest first (greedy to the
-// least-loaded slice, ties to the lower slice; equal lengths in index order).  plan[] lists each group's bundles slice by slice, starting at the
-// group's base; soff[(p G + g)(M1_SLICES + 1) + s] is where slice s starts.
-// Groups of more than 1024 bundles are dealt round-robin in index order.
+// run of the point's marched bundles: with the rays of a point in angular
+// order, the neighbours a block marches cross the same cells near the point,
+// which L1 then serves) dealt to M1_SLICES slices longest first (greedy to the
+// least-loaded slice, ties to the lower slice; equal lengths in index order).
+// plan[] lists each group's bundles slice by slice, starting at the group's
+// base; soff[(p G + g)(M1_SLICES + 1) + s] is where slice s starts.  Groups of
+// more than 1024 bundles are dealt round-robin in index order.
 __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ point_off,
-                                                    const int64_t* __restrict__ seg_off, int G,
-                                                    int32_t* __restrict__ plan, int32_t* __restrict__ soff) {
+                                                    const int64_t* __restrict__ seg_off,
+                                                    const int32_t* __restrict__ uniq,
+                                                    const int32_t* __restrict__ n_uniq, int G,
+                                                    int32_t* __restrict__ plan, int32_t* __restrict__ soff,
+                                                    const int* status) {
+    if (*status) return;
     const int64_t p = blockIdx.x / G;
     const int g = (int)(blockIdx.x % G);
     const int64_t pb0 = point_off[p];
-    const int64_t nb = point_off[p + 1] - pb0;
+    const int64_t nb = n_uniq[p];
     const int64_t m = nb > g ? (nb - g + G - 1) / G : 0;                     // bundles of this group
-    const int64_t base = pb0 + (int64_t)g * (nb / G) + (g < nb % G ? g : nb % G);   // the group's first bundle
+    const int64_t base = pb0 + (int64_t)g * (nb / G) + (g < nb % G ? g : nb % G);   // the group's first entry
     int32_t* so = soff + blockIdx.x * (M1_SLICES + 1);
     __shared__ int64_t len[1024];
     __shared__ int16_t order[1024];
@@ -628,7 +740,7 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
             const int s = (int)(k % M1_SLICES);
             const int64_t per = m / M1_SLICES, extra = m % M1_SLICES;
             const int64_t start = s * per + (s < extra ? s : extra);
-            plan[base + start + k / M1_SLICES] = (int32_t)(base + k);
+            plan[base + start + k / M1_SLICES] = uniq[base + k];
         }
         if (threadIdx.x <= M1_SLICES) {
             const int s = threadIdx.x;
@@ -639,7 +751,7 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
     }
     const int mm = (int)m;
     for (int k = threadIdx.x; k < mm; k += blockDim.x) {
-        const int64_t b = base + k;
+        const int64_t b = uniq[base + k];
         len[k] = seg_off[b + 1] - seg_off[b];
     }
     __syncthreads();
@@ -670,7 +782,7 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
         for (int s = 0; s < M1_SLICES; ++s) fill[s] = cnt[s];
         for (int r = 0; r < mm; ++r) {
             const int k = order[r];
-            plan[base + fill[slice_of[k]]++] = (int32_t)(base + k);
+            plan[base + fill[slice_of[k]]++] = uniq[base + k];
         }
     }
 }
@@ -724,7 +836,9 @@ __device__ __forceinline__ M1V<NP> m1_bundle(const MarchArgs& a, int64_t b, floa
     M1V<NP> kc, jc;
     kc = m1_rowload<NP, VEC>(kb, jb, (int64_t)a.seg_cell[s0] * ldb, dq, jc);
     M1V<NP> Kf = m1_sum(kc, kc), Jf = m1_sum(jc, jc);
-    const float hs = 0.5f * sc;
+    const float hs = -0.5f * sc;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) I.v[q] = make_float2(-I.v[q].x, -I.v[q].y);   // minus the intensity on the way
     // ring of loads in flight: values of the next cells of the following PF segments
     M1V<NP> rk[M1_PF], rj[M1_PF];
 #pragma unroll
@@ -738,7 +852,7 @@ __device__ __forceinline__ M1V<NP> m1_bundle(const MarchArgs& a, int64_t b, floa
         __syncwarp();
         const int64_t ahead = mine + M1_PF;   // the segment whose next cell this entry fetches
         const float shl = mine < s1 - 1 ? seg_len<float>(a, mine) * hs : 0.0f;
-        st[lane].sh = make_float2(shl, shl);
+        st[lane].nsh = make_float2(shl, shl);
         st[lane].off = ahead < s1 - 1 ? (int64_t)a.seg_cell[ahead + 1] * ldb : 0;
         __syncwarp();
         const int n = s1 - 1 - g < 32 ? (int)(s1 - 1 - g) : 32;
@@ -751,7 +865,7 @@ __device__ __forceinline__ M1V<NP> m1_bundle(const MarchArgs& a, int64_t b, floa
             rk[M1_PF - 1] = m1_rowload<NP, VEC>(kb, jb, e.off, dq, rj[M1_PF - 1]);
             const M1V<NP> Kn = m1_sum(kc, kx), Jn = m1_sum(jc, jx);
 #pragma unroll
-            for (int q = 0; q < NP; ++q) m1_step(I.v[q], Kf.v[q], Jf.v[q], Jn.v[q], e.sh);
+            for (int q = 0; q < NP; ++q) m1_step(I.v[q], Kf.v[q], Jf.v[q], Jn.v[q], e.nsh);
             Kf = Kn; Jf = Jn; kc = kx; jc = jx;
         }
     }
@@ -761,6 +875,8 @@ __device__ __forceinline__ M1V<NP> m1_bundle(const MarchArgs& a, int64_t b, floa
 #pragma unroll
         for (int q = 0; q < NP; ++q) m1_step(I.v[q], Kf.v[q], Jf.v[q], Jn.v[q], make_float2(hl, hl));
     }
+#pragma unroll
+    for (int q = 0; q < NP; ++q) I.v[q] = make_float2(-I.v[q].x, -I.v[q].y);
     return I;
 }
 
@@ -789,6 +905,7 @@ __device__ __forceinline__ void m1_store(float* __restrict__ p, const M1V<NP>& x
 template <int NP, bool VEC>
 __global__ void __launch_bounds__(256, RAPRAL_MARCH_MINB) k_march1(MarchArgs a, int lgG, const int32_t* __restrict__ plan,
                                                                    const int32_t* __restrict__ soff,
+                                                                   const int32_t* __restrict__ partner,
                                                                    float* __restrict__ part) {
     if (*a.status) return;
     constexpr int TW = 64 * NP, SLC = M1_SLICES, NC = 2 * NP;
@@ -824,7 +941,13 @@ __global__ void __launch_bounds__(256, RAPRAL_MARCH_MINB) k_march1(MarchArgs a, 
         if (a.wall_row && a.bundle_wall[b]) I0 = m1_load<NP, VEC>(reinterpret_cast<const float*>(a.wall_row) + c0, dq);
         const M1V<NP> I = m1_bundle<NP, VEC>(a, b, a.dir_scale_f[d0], st, lane, kb, jb, dq, a.ld * 4, I0);
         if (a.I_out) m1_store<NP, VEC>(reinterpret_cast<float*>(a.I_out) + d0 * a.nk + col, I, own);
-        const float w = a.dir_weight_f[d0];
+        float w = a.dir_weight_f[d0];
+        const int b2 = partner[b];
+        if (b2 >= 0) {   // the equal ray: its weight, and its intensities
+            const int64_t d2 = a.dir_off[b2];
+            w += a.dir_weight_f[d2];
+            if (a.I_out) m1_store<NP, VEC>(reinterpret_cast<float*>(a.I_out) + d2 * a.nk + col, I, own);
+        }
 #pragma unroll
         for (int q = 0; q < NP; ++q) {   // compensated sum over the slice's bundles
             const float2 y = make_float2(w * I.v[q].x - comp.v[q].x, w * I.v[q].y - comp.v[q].y);
@@ -1037,11 +1160,22 @@ static bool march1_vec(const MarchArgs& a, int64_t nk, const void* part) {
            ok(part) && (a.I_out == nullptr || ok(a.I_out));
 }
 
-static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, int G, void* part,
-                                 int32_t* plan, int32_t* soff) {
+// The march's plan: the equal rays and the slices of every (point, group).
+struct M1Plan {
+    unsigned long long* key;   // [n_bundles]
+    int32_t *partner, *uniq, *plan;   // [n_bundles]
+    int32_t* n_uniq;           // [n_points]
+    int32_t* soff;             // [n_points G (M1_SLICES + 1)]
+};
+
+static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t B, int64_t nk, int G,
+                                 void* part, const M1Plan& pl) {
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
-    k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, G, plan, soff);
+    if (B > 0) k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.key);
+    k_ray_pairs<<<(unsigned)P, 256, 0, ctx->stream>>>(a, pl.key, pl.partner, pl.uniq, pl.n_uniq);
+    k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, pl.uniq, pl.n_uniq, G, pl.plan,
+                                                             pl.soff, a.status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     MarchArgs b = a;
@@ -1054,9 +1188,11 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
     }
     dim3 g((unsigned)(P << lgG), div_up(nk, 64 * kM1NP));
     if (march1_vec(a, nk, part))
-        k_march1<kM1NP, true><<<g, 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, plan, soff, reinterpret_cast<float*>(part));
+        k_march1<kM1NP, true><<<g, 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner,
+                                                                          reinterpret_cast<float*>(part));
     else
-        k_march1<kM1NP, false><<<g, 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, plan, soff, reinterpret_cast<float*>(part));
+        k_march1<kM1NP, false><<<g, 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner,
+                                                                          reinterpret_cast<float*>(part));
     e = cudaGetLastError();
     if (e != cudaSuccess || G == 1) return e;
     k_group_sum<float><<<(unsigned)std::min<int64_t>(div_up(P * nk, 256), 152 * 16), 256, 0, ctx->stream>>>(
@@ -1091,14 +1227,6 @@ cudaError_t march_t(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, 
 
 }  // namespace
 
-cudaError_t launch_validate_rays(rapral_ctx* ctx, const rapral_rays* r, int64_t n_cells) {
-    const int64_t n = r->n_segments > r->n_dirs ? r->n_segments : r->n_dirs;
-    if (n == 0) return cudaSuccess;
-    k_validate_rays<<<div_up(n, 256), 256, 0, ctx->stream>>>(r->seg_cell, r->seg_ds, r->n_segments, n_cells,
-                                                            r->dir_scale, r->n_dirs, ctx->d_status);
-    return cudaGetLastError();
-}
-
 // Bundle groups per point where a point has eight or more bundles (a power of two):
 // enough blocks share a wavelength tile (points x groups >= 1536, about two
 // waves of resident blocks) that the tiles in flight, and so the kappa / j
@@ -1118,20 +1246,36 @@ static int march_groups(const rapral_rays* r) {
 
 static size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 
-// FP32 scratch: the FP32 copies, then k_march1's bundle plan and slice starts.
+// FP32 scratch: the FP32 copies of lengths, scales and weights (each from a
+// multiple of 64 floats), then k_march1's plan.
+static size_t march_copy_bytes(const rapral_rays* r) {
+    return round256((size_t)(r->n_segments + 2 * r->n_dirs + 128) * sizeof(float));
+}
 static size_t march_plan_bytes(const rapral_rays* r) {
-    return round256((size_t)(r->n_bundles + (int64_t)r->n_points * march_groups(r) * (M1_SLICES + 1) + 64) *
-                    sizeof(int32_t));
+    return round256((size_t)r->n_bundles * 8) + 3 * round256((size_t)r->n_bundles * 4) +
+           round256((size_t)r->n_points * 4) +
+           round256((size_t)r->n_points * march_groups(r) * (M1_SLICES + 1) * 4);
 }
 
 size_t march_scratch_bytes(const rapral_rays* r, int64_t nk, int precision) {
     size_t bytes = 0;
-    if (precision == RAPRAL_FP32)
-        bytes = round256((size_t)(r->n_segments + 2 * r->n_dirs + 128) * sizeof(float)) + march_plan_bytes(r);
+    if (precision == RAPRAL_FP32) bytes = march_copy_bytes(r) + march_plan_bytes(r);
     const int G = march_groups(r);
     const size_t el = precision == RAPRAL_FP64 ? sizeof(double) : sizeof(float);
     if (G > 1) bytes += (size_t)r->n_points * G * nk * el;
     return bytes + nk * el + 256;   // + the wall's Planck row
+}
+
+cudaError_t launch_validate_rays(rapral_ctx* ctx, const rapral_rays* r, int64_t n_cells, void* copies) {
+    const int64_t n = r->n_segments > r->n_dirs ? r->n_segments : r->n_dirs;
+    if (n == 0) return cudaSuccess;
+    float* f = reinterpret_cast<float*>(copies);
+    float* fd = f ? f + ((r->n_segments + 63) / 64) * 64 : nullptr;
+    float* fw = f ? fd + ((r->n_dirs + 63) / 64) * 64 : nullptr;
+    k_validate_rays<<<div_up(n, 256), 256, 0, ctx->stream>>>(r->seg_cell, r->seg_ds, r->n_segments, n_cells,
+                                                            r->dir_scale, r->dir_weight, r->n_dirs, f, fd, fw,
+                                                            ctx->d_status);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kappa, const void* emis, int64_t ld,
@@ -1149,26 +1293,23 @@ cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kapp
     if (precision == RAPRAL_FP64)
         return march_t<double>(ctx, a, r->n_points, nk, r->max_dirs, r->max_bundles_per_point, G, scratch,
                                r->node_values != 0);
-    // FP32 copies of the path lengths, direction scales and weights, then the group partials
-    float* f = reinterpret_cast<float*>(scratch);
-    const size_t copies = round256((size_t)(r->n_segments + 2 * r->n_dirs + 128) * sizeof(float));
-    int32_t* plan = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(scratch) + copies);
-    int32_t* soff = plan + ((r->n_bundles + 63) / 64) * 64;
-    void* part = reinterpret_cast<char*>(scratch) + copies + march_plan_bytes(r);
-    float* fd = f + ((r->n_segments + 63) / 64) * 64;
-    float* fw = fd + ((r->n_dirs + 63) / 64) * 64;
-    if (r->n_segments > 0)
-        k_to_float<<<(unsigned)std::min<int64_t>(div_up(r->n_segments, 256), 4096), 256, 0, ctx->stream>>>(
-            r->seg_ds, r->n_segments, f);
-    if (r->n_dirs > 0) {
-        k_to_float<<<(unsigned)std::min<int64_t>(div_up(r->n_dirs, 256), 4096), 256, 0, ctx->stream>>>(
-            r->dir_scale, r->n_dirs, fd);
-        k_to_float<<<(unsigned)std::min<int64_t>(div_up(r->n_dirs, 256), 4096), 256, 0, ctx->stream>>>(
-            r->dir_weight, r->n_dirs, fw);
-    }
-    a.seg_ds_f = f; a.dir_scale_f = fd; a.dir_weight_f = fw;
+    // the FP32 copies (written by launch_validate_rays), the plan, then the group partials
+    char* at = reinterpret_cast<char*>(scratch);
+    a.seg_ds_f = reinterpret_cast<float*>(at);
+    a.dir_scale_f = a.seg_ds_f + ((r->n_segments + 63) / 64) * 64;
+    a.dir_weight_f = a.dir_scale_f + ((r->n_dirs + 63) / 64) * 64;
+    at += march_copy_bytes(r);
+    void* part = at + march_plan_bytes(r);
+    M1Plan pl;
+    const auto take = [&at](size_t bytes) { char* p = at; at += round256(bytes); return p; };
+    pl.key = reinterpret_cast<unsigned long long*>(take((size_t)r->n_bundles * 8));
+    pl.partner = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
+    pl.uniq = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
+    pl.plan = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
+    pl.n_uniq = reinterpret_cast<int32_t*>(take((size_t)r->n_points * 4));
+    pl.soff = reinterpret_cast<int32_t*>(take((size_t)r->n_points * G * (M1_SLICES + 1) * 4));
     if (march1_applies(a, r->max_dirs, r->max_bundles_per_point, r->node_values != 0))
-        return march1_launch(ctx, a, r->n_points, nk, G, part, plan, soff);
+        return march1_launch(ctx, a, r->n_points, r->n_bundles, nk, G, part, pl);
     return march_t<float>(ctx, a, r->n_points, nk, r->max_dirs, r->max_bundles_per_point, G, part,
                           r->node_values != 0);
 }

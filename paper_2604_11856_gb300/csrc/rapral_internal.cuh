@@ -324,10 +324,13 @@ cudaError_t launch_line_sum_batch(rapral_ctx* ctx, int tile_w, int wpb, int pb, 
                                   int64_t total, unsigned long long* counter, int* blocks_out, bool launch, bool broad);
 
 // Rays
-cudaError_t launch_validate_rays(rapral_ctx* ctx, const rapral_rays* r, int64_t n_cells);
+// Checks a ray set; with `copies` (the start of an FP32 march's scratch) also
+// writes the FP32 copies that launch_march reads there.
+cudaError_t launch_validate_rays(rapral_ctx* ctx, const rapral_rays* r, int64_t n_cells, void* copies = nullptr);
 // The march needs march_scratch_bytes(r, nk, precision) of scratch (256-byte
 // aligned): FP32 copies of the ray lengths, direction scales and weights
-// (FP32 only), then per-group partial spectral fluxes where a point's
+// and the single-direction march's plan (FP32 only; the copies are written by
+// launch_validate_rays on the same scratch), then per-group partial spectral fluxes where a point's
 // bundles are split over several blocks.
 size_t march_scratch_bytes(const rapral_rays* r, int64_t nk, int precision);
 cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kappa, const void* emis,
