@@ -23,7 +23,10 @@
 // where P(lam) = 2 h c^2 / lam^5 in the Planck function's units.  The
 // exponent is <= 0 wherever sigma_i != 0 (lam below the edge), whereas the
 // Saha factor and the Planck function alone over- and underflow at low T.
+#include <algorithm>
+
 #include "rapral_internal.cuh"
+#include "exp_fix.cuh"
 
 namespace {
 
@@ -64,26 +67,35 @@ __device__ __forceinline__ double cont_exp(double x) { return exp(x); }
 __device__ __forceinline__ float cont_div(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double cont_div(double a, double b) { return a / b; }
 
-__global__ void k_cont_validate(ContModels M, int* status) {
+// a <= b of positive doubles by their bits: comparisons run on the FP64 pipe,
+// which has 1/64 of the FP32 rate, and the searches below are nothing else
+__device__ __forceinline__ bool pos_le(double a, double b) {
+    return __double_as_longlong(a) <= __double_as_longlong(b);
+}
+
+// One warp a level (blocks of eight), lanes along its nodes: one thread a level
+// walked its 120 nodes as a chain of loads (62 us).
+__global__ void __launch_bounds__(256) k_cont_validate(ContModels M, int* status) {
     const rapral_continuum& m = M.m[blockIdx.x];
-    for (int i = threadIdx.x; i < m.n_levels; i += blockDim.x) {
+    const int lane = threadIdx.x & 31, i = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (i < m.n_levels) {
         const int64_t a = m.node_off[i], b = m.node_off[i + 1];
         if ((i == 0 && a != 0) || (i == m.n_levels - 1 && b != m.n_nodes) || a < 0 || b < a + 2 ||
             b > m.n_nodes) {
-            fail(status, CHK_CONT_TABLE, i);
-            continue;
-        }
-        if (!(m.E[i] >= 0.0 && m.E[i] < m.E_ionize) || !(m.g[i] > 0.0) || !isfinite(m.g[i]))
-            fail(status, CHK_CONT_TABLE, i);
-        for (int64_t j = a; j < b; ++j) {
-            if (!(m.node_sigma[j] >= 0.0) || !isfinite(m.node_sigma[j]) || !(m.node_lam[j] > 0.0) ||
-                !isfinite(m.node_lam[j]) || (j + 1 < b && !(m.node_lam[j + 1] > m.node_lam[j]))) {
-                fail(status, CHK_CONT_TABLE, j);
-                break;
+            if (lane == 0) fail(status, CHK_CONT_TABLE, i);
+        } else {
+            if (lane == 0 && (!(m.E[i] >= 0.0 && m.E[i] < m.E_ionize) || !(m.g[i] > 0.0) || !isfinite(m.g[i])))
+                fail(status, CHK_CONT_TABLE, i);
+            for (int64_t j = a + lane; j < b; j += 32) {
+                if (!(m.node_sigma[j] >= 0.0) || !isfinite(m.node_sigma[j]) || !(m.node_lam[j] > 0.0) ||
+                    !isfinite(m.node_lam[j]) || (j + 1 < b && !(m.node_lam[j + 1] > m.node_lam[j]))) {
+                    fail(status, CHK_CONT_TABLE, j);
+                    break;
+                }
             }
         }
     }
-    if (threadIdx.x == 0) {
+    if (blockIdx.y == 0 && threadIdx.x == 0) {
         for (int k = 0; k < m.n_ion_terms; ++k)
             if (!(m.ion_g[k] >= 0.0) || !isfinite(m.ion_E[k])) fail(status, CHK_CONT_TABLE, k);
         if (m.D) {
@@ -99,7 +111,7 @@ __global__ void k_cont_validate(ContModels M, int* status) {
 __global__ void __launch_bounds__(1024) k_cont_levels(ContModels M, double lam_min, double h, ContLevel* out,
                                                       const int* status) {
     if (*status) return;
-    __shared__ double key[RAPRAL_MAX_CONT_LEVELS];
+    __shared__ unsigned long long key[RAPRAL_MAX_CONT_LEVELS];   // positive doubles order like their bits
     const int r = threadIdx.x;
     int m = 0, i = 0;
     double last = 0.0;
@@ -107,12 +119,13 @@ __global__ void __launch_bounds__(1024) k_cont_levels(ContModels M, double lam_m
         while (r >= M.lev0[m + 1]) ++m;
         i = r - M.lev0[m];
         last = M.m[m].node_lam[M.m[m].node_off[i + 1] - 1];
-        key[r] = last;
+        key[r] = (unsigned long long)__double_as_longlong(last);
     }
     __syncthreads();
     if (r < M.I) {
         int rank = 0;
-        for (int q = 0; q < M.I; ++q) rank += (key[q] > last || (key[q] == last && q < r)) ? 1 : 0;
+        const unsigned long long own = key[r];
+        for (int q = 0; q < M.I; ++q) rank += (key[q] > own || (key[q] == own && q < r)) ? 1 : 0;
         ContLevel L;
         L.last = last;
         L.v = (M.m[m].E_ionize - M.m[m].E[i]) * 1e-7;
@@ -179,7 +192,7 @@ __global__ void __launch_bounds__(128) k_cont_sigma(ContModels M, const ContLeve
         int64_t lo = a, hi = b;   // last node <= lam_first (or a)
         while (hi - lo > 1) {
             const int64_t mid = (lo + hi) >> 1;
-            if (x[mid] <= lam_first) lo = mid;
+            if (pos_le(x[mid], lam_first)) lo = mid;
             else hi = mid;
         }
         int64_t j = lo;
@@ -240,7 +253,7 @@ __global__ void __launch_bounds__(128) k_cont_sigma32(ContModels M, const ContLe
         int64_t lo = a, hi = b;
         while (hi - lo > 1) {
             const int64_t mid = (lo + hi) >> 1;
-            if (x[mid] <= lam_first) lo = mid;
+            if (pos_le(x[mid], lam_first)) lo = mid;
             else hi = mid;
         }
         int64_t j = lo;
@@ -273,12 +286,12 @@ __global__ void k_cont_points(ContModels M, int64_t n_pad, double lam_min, doubl
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n_pad) return;
     const double lam = grid_lam(lam_min, h, k0 + k);
-    const double lcm = lam * 1e-7;
-    const double ir = lam / LAM_H;   // 1 / sigma
-    pts[k * 4 + 0] = (Tp)(1.0 / lam);
-    pts[k * 4 + 1] = (Tp)(1e-7 * 2.0 * ph.h * ph.c * ph.c / (1e4 * lcm * lcm * lcm * lcm * lcm));
+    const double ul = 1.0 / lam, u2 = ul * ul;
+    const double ir = lam * (1.0 / LAM_H);   // 1 / sigma
+    pts[k * 4 + 0] = (Tp)ul;
+    pts[k * 4 + 1] = (Tp)(1e-7 * 2.0 * ph.h * ph.c * ph.c / (1e4 * 1e-35) * (u2 * u2 * ul));   // lam in cm: 1e-7 lam
     pts[k * 4 + 2] = (Tp)(ir * ir * ir);
-    pts[k * 4 + 3] = (Tp)(ir * ir * ir * ir);
+    pts[k * 4 + 3] = (Tp)(ir * ir * (ir * ir));
     for (int m = 0; m < M.M; ++m) {
         const rapral_continuum& md = M.m[m];
         int j = 0;
@@ -286,7 +299,7 @@ __global__ void k_cont_points(ContModels M, int64_t n_pad, double lam_min, doubl
         if (md.D) {
             const double* xs = md.D_sigma;
             const int nD = md.n_D_sigma;
-            const double sg = fmin(fmax(LAM_H / lam, xs[0]), xs[nD - 1]);
+            const double sg = fmin(fmax(LAM_H * ul, xs[0]), xs[nD - 1]);
             int lo = 0, hi = nD - 1;   // last node <= sg, at most nD - 2
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
@@ -309,6 +322,10 @@ __global__ void k_cont_coef(ContModels M, const ContLevel* lev, rapral_cells cel
                             double lim, Tp* coefN, Tp* coefA, Tp* coefA2, int* warm, Tp* theta, Tp* ff, Tp* Drow,
                             const int* status) {
     if (*status) return;
+    __shared__ uint64_t tab[EXPFIX_N];
+    __shared__ double sQ[RAPRAL_MAX_CONT_MODELS], sA[RAPRAL_MAX_CONT_MODELS];   // ln(2 Q_+), ln(N_+ N_e S / 2 Q_+)
+    expfix_load(tab);
+    __syncthreads();
     const int64_t c = blockIdx.x;
     const int64_t C = cells.n_cells;
     const double T = cells.Tve[c];
@@ -316,20 +333,28 @@ __global__ void k_cont_coef(ContModels M, const ContLevel* lev, rapral_cells cel
     const double ne = n[cells.ne_col];
     const double lnS = 1.5 * log(ph.h * ph.h / (2.0 * M_PI * ph.me * ph.kB * T));
     const double th = ph.c2 * 1e7 / T;
+    // the ion's partition function once a model, not once a level
+    for (int mi = threadIdx.x; mi < M.M; mi += blockDim.x) {
+        const rapral_continuum& m = M.m[mi];
+        double Qp = 0.0;
+        for (int k = 0; k < m.n_ion_terms; ++k) Qp += m.ion_g[k] * exp_fix(-ph.c2 * m.ion_E[k] / T, tab);
+        const double lnQ = log(2.0 * Qp);
+        sQ[mi] = lnQ;
+        sA[mi] = log(n[m.ion_col]) + log(ne) + lnS - lnQ;
+    }
+    __syncthreads();
     int hot = th * u_max > lim;
     for (int r = threadIdx.x; r < M.I; r += blockDim.x) {
         const ContLevel L = lev[r];
         const rapral_continuum& m = M.m[L.m];
-        double Qp = 0.0;
-        for (int k = 0; k < m.n_ion_terms; ++k) Qp += m.ion_g[k] * exp(-ph.c2 * m.ion_E[k] / T);
         const double lg = log(m.g[L.i]);
-        const double N = exp(cells.lnpref[c * S + m.species] + lg - ph.c2 * m.E[L.i] / T);
-        const double lnA = log(n[m.ion_col]) + log(ne) + lnS - log(2.0 * Qp) + lg;
+        const double N = exp_fix(cells.lnpref[c * S + m.species] + lg - ph.c2 * m.E[L.i] / T, tab);
+        const double lnA = sA[L.m] + lg;
         const double lnA2 = lnA + th * L.v;
         if (lnA2 > lim) hot = 1;
         coefN[r * C + c] = (Tp)N;
-        coefA[r * C + c] = (Tp)exp(lnA);
-        coefA2[r * C + c] = (Tp)exp(lnA2);
+        coefA[r * C + c] = (Tp)exp_fix(lnA, tab);
+        coefA2[r * C + c] = (Tp)exp_fix(lnA2, tab);
     }
     hot = __syncthreads_or(hot);
     if (threadIdx.x == 0) {
@@ -338,12 +363,10 @@ __global__ void k_cont_coef(ContModels M, const ContLevel* lev, rapral_cells cel
     }
     for (int mi = threadIdx.x; mi < M.M; mi += blockDim.x) {
         const rapral_continuum& m = M.m[mi];
-        double Qp = 0.0;
-        for (int k = 0; k < m.n_ion_terms; ++k) Qp += m.ion_g[k] * exp(-ph.c2 * m.ion_E[k] / T);
-        const double F = exp(cells.lnpref[c * S + m.species] + log(2.0 * Qp) - lnS - ph.c2 * m.E_ionize / T) * 1e-40;
+        const double F = exp_fix(cells.lnpref[c * S + m.species] + sQ[mi] - lnS - ph.c2 * m.E_ionize / T, tab) * 1e-40;
         const double* cc = m.ff_c;
-        const double A1 = cc[0] + cc[1] * exp(-cc[2] * T);
-        const double A2 = cc[3] + cc[4] * exp(-cc[5] * T) + cc[6] * exp(-cc[7] * T);
+        const double A1 = cc[0] + cc[1] * exp_fix(-cc[2] * T, tab);
+        const double A2 = cc[3] + cc[4] * exp_fix(-cc[5] * T, tab) + cc[6] * exp_fix(-cc[7] * T, tab);
         ff[(c * M.M + mi) * 2] = (Tp)(F * A1);
         ff[(c * M.M + mi) * 2 + 1] = (Tp)(F * A2);
         Tp* row = Drow + (c * M.M + mi) * CONT_DMAX;
@@ -767,7 +790,9 @@ static int cont_run(rapral_ctx* ctx, const ContModels& Mh, int S, const rapral_c
     cudaStream_t s = ctx->stream;
     cudaError_t e = launch_validate_cells(ctx, cells);
     if (e == cudaSuccess) {
-        k_cont_validate<<<M, 128, 0, s>>>(Mh, ctx->d_status);
+        int maxlev = 1;
+        for (int m = 0; m < M; ++m) maxlev = std::max(maxlev, Mh.m[m].n_levels);
+        k_cont_validate<<<dim3(M, div_up(maxlev, 8)), 256, 0, s>>>(Mh, ctx->d_status);
         k_cont_levels<<<1, RAPRAL_MAX_CONT_LEVELS, 0, s>>>(Mh, g->lam_min, h, lev, ctx->d_status);
         k_cont_tiles<<<div_up(T, 256), 256, 0, s>>>(lev, I, T, W, g->lam_min, h, k0, n_lev, tab_off, ctx->d_status);
         e = cudaGetLastError();
