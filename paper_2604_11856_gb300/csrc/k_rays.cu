@@ -143,31 +143,84 @@ __device__ __forceinline__ void seg_step2(float& I0, float& I1, float k0, float 
     }
 }
 
-// The nd directions of one column (nd <= MAXD, the same for the whole warp):
-// packed in pairs in FP32.  FP64 shares kappa s, s j_far and s (j_near -
-// j_far) of the common length s between the directions.
+// The nd directions of one column (nd <= MAXD, the same for the whole warp;
+// scmax: their largest scale).  With the common length s the step of a
+// direction of scale c is I + c B, A = s j_far - s kappa I, B = A +
+// p(c s kappa) (s (j_near - j_far) - c s kappa A), so s kappa, s j_far and
+// s (j_near - j_far) are shared.  FP32 runs two directions a packed
+// instruction, with t = -c s kappa carried so that no sign is flipped (FP32
+// and integer instructions share one pipe, which bounds the slab): the
+// largest scale decides once for all directions and, by a vote, for the warp
+// (lanes on two paths would take both) whether the short series (|t| below
+// 2^-5, four terms, truncation 3e-9: 8 packed instructions a pair) or the
+// seven-term one (11) holds; only where it does not is each pair tested.
+__device__ __forceinline__ float2 f2c(float c) { return make_float2(c, c); }
+template <bool SHORT>
+__device__ __forceinline__ void dir_pair(float& I0, float& I1, float2 t0, float2 jd, float2 dj, float2 sc) {
+    const float2 t = __fmul2_rn(t0, sc);
+    float2 p = f2c(1.0f / 120.0f);
+    if (!SHORT) {
+        p = __ffma2_rn(t, f2c(1.0f / 40320.0f), f2c(1.0f / 5040.0f));
+        p = __ffma2_rn(t, p, f2c(1.0f / 720.0f));
+        p = __ffma2_rn(t, p, f2c(1.0f / 120.0f));
+    }
+    p = __ffma2_rn(t, p, f2c(1.0f / 24.0f));
+    p = __ffma2_rn(t, p, f2c(1.0f / 6.0f));
+    p = __ffma2_rn(t, p, f2c(0.5f));
+    const float2 I = make_float2(I0, I1);
+    const float2 A = __ffma2_rn(t0, I, jd);
+    const float2 r = __ffma2_rn(sc, __ffma2_rn(p, __ffma2_rn(t, A, dj), A), I);
+    I0 = r.x;
+    I1 = r.y;
+}
 template <class T, int MAXD>
-__device__ __forceinline__ void dir_steps(T (&I)[MAXD], T kf, T ds, const T* sc, int nd, T jf, T jn) {
+__device__ __forceinline__ void dir_steps(T (&I)[MAXD], T kf, T ds, const T* sc, T scmax, int nd, T jf, T jn) {
     if constexpr (MAXD == 1) {
         seg_step(I[0], kf, ds, jf, jn);
     } else if constexpr (sizeof(T) == 4) {
+        const float t0 = -kf * ds;
+        const float2 t2 = f2c(t0), jd = f2c(ds * jf), dj = f2c(ds * (jn - jf));
+        const float tm = fabsf(t0) * scmax;
+        const auto pairs = [&](auto step) {
 #pragma unroll
-        for (int d = 0; d + 1 < MAXD; d += 2)
-            seg_step2(I[d], I[d + 1], kf, kf, ds * sc[d], ds * sc[d + 1], jf, jf, jn, jn);
-        if (MAXD & 1) seg_step(I[MAXD - 1], kf, ds * sc[MAXD - 1], jf, jn);
+            for (int d = 0; d < MAXD; d += 2) {
+                if (d % 4 == 0 && d >= nd) break;
+                if (d + 1 < MAXD) {
+                    step(I[d], I[d + 1], make_float2(sc[d], sc[d + 1]));
+                } else {   // the last of an odd number, with an idle half of scale 0
+                    float idle = 0.0f;
+                    step(I[d], idle, make_float2(sc[d], 0.0f));
+                }
+            }
+        };
+        if (!__any_sync(0xffffffffu, tm >= 0.03125f)) {
+            pairs([&](float& a, float& b, float2 s) { dir_pair<true>(a, b, t2, jd, dj, s); });
+        } else if (!__any_sync(0xffffffffu, tm >= (float)RAPRAL_THIN_F32)) {
+            pairs([&](float& a, float& b, float2 s) { dir_pair<false>(a, b, t2, jd, dj, s); });
+        } else {
+            pairs([&](float& a, float& b, float2 s) {
+                if (fabsf(t0) * fmaxf(s.x, s.y) < (float)RAPRAL_THIN_F32) {
+                    dir_pair<false>(a, b, t2, jd, dj, s);
+                } else {
+                    seg_step(a, kf, ds * s.x, jf, jn);
+                    seg_step(b, kf, ds * s.y, jf, jn);
+                }
+            });
+        }
     } else {
         const T t0 = kf * ds, jd = ds * jf, dj = ds * (jn - jf);
 #pragma unroll
         for (int d = 0; d < MAXD; ++d) {
-            if (d >= nd) break;
-            const T t = t0 * sc[d];
-            const int hi = abs_hi(t);
-            if (hi < T64_1) {
-                const T p = thin_series(t, hi);
-                const T A = fma(-t0, I[d], jd);
-                I[d] = fma(sc[d], fma(p, fma(-t, A, dj), A), I[d]);
-            } else {
-                I[d] = thick_step(I[d], kf, t, jf, jn);
+            if (d < nd) {
+                const T t = t0 * sc[d];
+                const int hi = abs_hi(t);
+                if (hi < T64_1) {
+                    const T p = thin_series(t, hi);
+                    const T A = fma(-t0, I[d], jd);
+                    I[d] = fma(sc[d], fma(p, fma(-t, A, dj), A), I[d]);
+                } else {
+                    I[d] = thick_step(I[d], kf, t, jf, jn);
+                }
             }
         }
     }
@@ -318,6 +371,9 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
     T sc[MAXD];
 #pragma unroll
     for (int d = 0; d < MAXD; ++d) sc[d] = d < nd ? dir_val<T>(a.dir_scale, a.dir_scale_f, d0 + d) : T(0);
+    T scmax = T(0);
+#pragma unroll
+    for (int d = 0; d < MAXD; ++d) scmax = sc[d] > scmax ? sc[d] : scmax;
     // one direction: its scale goes into the staged length
     const T stage_scale = MAXD == 1 ? sc[0] : T(1);
 #pragma unroll
@@ -380,7 +436,7 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
                 seg_step2(I[0][0], I[1][0], kf[0], kf[1], ds, ds, jf[0], jf[1], jn[0], jn[1]);
             } else {
 #pragma unroll
-                for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, nd, jf[v], jn[v]);
+                for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, scmax, nd, jf[v], jn[v]);
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -396,7 +452,7 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
             seg_step2(I[0][0], I[1][0], kf[0], kf[1], ds, ds, jf[0], jf[1], jc[0], jc[1]);
         } else {
 #pragma unroll
-            for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, nd, jf[v], jc[v]);
+            for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, scmax, nd, jf[v], jc[v]);
         }
     }
 }
