@@ -570,9 +570,10 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ?
 //
 // Same work and results contract as k_march<float, 2, 1, 8>, organised for
 // fewer instructions per segment-wavelength:
-//  * lane l owns two ADJACENT columns (base + 2l, base + 2l + 1): one 8-byte
-//    load fetches both, for kappa and for j (a warp reads 256 contiguous
-//    bytes of a row);
+//  * lane l owns four or two ADJACENT columns: one 16- or 8-byte load fetches
+//    them, for kappa and for j (a warp reads 512 or 256 contiguous bytes of a
+//    row); where rows are not aligned for it, two columns 32 apart with one
+//    coalesced 4-byte load each;
 //  * node values are carried doubled (K = kappa_a + kappa_b, the sum of the
 //    two cells at a face), with the segment length halved to match, which
 //    removes the averaging multiplies;
@@ -708,7 +709,7 @@ __global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t B, unsign
 // it, -1: none), and the marched bundles in index order (uniq, from the
 // point's first bundle) with their number (n_uniq).  A bundle of a key's odd
 // rank is the partner of the one before it, if the two are equal.
-__global__ void __launch_bounds__(256) k_ray_pairs(MarchArgs a, const unsigned long long* __restrict__ key,
+__global__ void __launch_bounds__(512) k_ray_pairs(MarchArgs a, const unsigned long long* __restrict__ key,
                                                    int32_t* __restrict__ partner, int32_t* __restrict__ uniq,
                                                    int32_t* __restrict__ n_uniq) {
     if (*a.status) return;
@@ -726,12 +727,18 @@ __global__ void __launch_bounds__(256) k_ray_pairs(MarchArgs a, const unsigned l
     const int n = (int)nb;
     for (int k = threadIdx.x; k < n; k += blockDim.x) ks[k] = key[pb0 + k];
     __syncthreads();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const unsigned long long x = ks[k];
+    for (int kb = 0; kb < n; kb += blockDim.x / 4) {   // four lanes a bundle, every fourth earlier one each
+        const int k = kb + (int)(threadIdx.x >> 2);
+        const unsigned long long x = k < n ? ks[k] : 0ULL;
         int rank = 0, prev = -1;
-        for (int q = 0; q < k; ++q)
-            if (ks[q] == x) { ++rank; prev = q; }
-        first[k] = (int16_t)(x != 0ULL && (rank & 1) ? prev : -1);
+        if (x != 0ULL)
+            for (int q = threadIdx.x & 3; q < k; q += 4)
+                if (ks[q] == x) { ++rank; prev = q; }
+        rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+        prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, 1));
+        rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+        prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, 2));
+        if (k < n && (threadIdx.x & 3) == 0) first[k] = (int16_t)((rank & 1) ? prev : -1);
     }
     __syncthreads();
     for (int k = warp; k < n; k += blockDim.x >> 5) {   // the full comparison, a warp a candidate
@@ -847,8 +854,9 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
 template <int NP> struct M1V { float2 v[NP]; };
 
 // The lane's columns of one row: one 8-byte (NP = 1) or 16-byte (NP = 2)
-// load when the columns are aligned (VEC), else one 4-byte load a column at
-// the offsets dq[] from the first (columns past the range repeat the last).
+// load of adjacent columns when they are aligned (VEC), else one coalesced
+// 4-byte load a column at the offsets dq[] from the first (32 apart; columns
+// past the range repeat the last).
 template <int NP, bool VEC>
 __device__ __forceinline__ M1V<NP> m1_load(const float* __restrict__ p, const int (&dq)[2 * NP]) {
     M1V<NP> r;
@@ -947,8 +955,8 @@ __device__ __forceinline__ void m1_store(float* __restrict__ p, const M1V<NP>& x
     } else {
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
-            if (own[2 * q]) p[2 * q] = x.v[q].x;
-            if (own[2 * q + 1]) p[2 * q + 1] = x.v[q].y;
+            if (own[2 * q]) p[64 * q] = x.v[q].x;
+            if (own[2 * q + 1]) p[64 * q + 32] = x.v[q].y;
         }
     }
 }
@@ -969,14 +977,16 @@ __global__ void __launch_bounds__(256, RAPRAL_MARCH_MINB) k_march1(MarchArgs a, 
     const int nk = (int)a.nk;
     const int tile0 = (int)blockIdx.y * TW;
     const int base = (tile0 + TW > nk && nk >= TW) ? nk - TW : tile0;
-    const int col = base + NC * lane;                 // the lane's columns: col .. col + NC - 1
+    // the lane's columns: col .. col + NC - 1 (VEC), or col, col + 32, ...
+    constexpr int CS = VEC ? 1 : 32;
+    const int col = base + (VEC ? NC * lane : lane);
     const int c0 = col < nk ? col : nk - 1;           // clamped reads (VEC: never clamped)
     int dq[NC];
     bool own[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
-        dq[q] = (col + q < nk ? col + q : nk - 1) - c0;
-        own[q] = col + q >= tile0 && col + q < nk;
+        dq[q] = (col + CS * q < nk ? col + CS * q : nk - 1) - c0;
+        own[q] = col + CS * q >= tile0 && col + CS * q < nk;
     }
     const char* kb = reinterpret_cast<const char*>(reinterpret_cast<const float*>(a.kappa) + c0);
     const char* jb = reinterpret_cast<const char*>(reinterpret_cast<const float*>(a.emis) + c0);
@@ -1193,26 +1203,20 @@ cudaError_t march_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t
 }
 
 // k_march1 applies: FP32 cell-valued single-direction bundles, eight or more
-// a point, and the 8-byte alignment and even sizes of its paired columns.
+// a point.
 static bool march1_applies(const MarchArgs& a, int maxd, int maxb, bool nodes) {
     return !nodes && maxd <= 1 && maxb >= 8 && a.ld <= 2147483647LL;
 }
 
-// Columns a lane owns in k_march1 (2 NP) and the tile width (64 NP).
-#ifndef RAPRAL_M1_NP
-#define RAPRAL_M1_NP 1
-#endif
-constexpr int kM1NP = RAPRAL_M1_NP;
-
-// Vector loads and stores of 2 NP floats: every row of kappa / emis,
-// q_lambda, I_out and the wall row starts aligned to 8 NP bytes, and the
-// range is whole tiles or ends on a multiple of 2 NP columns past the first
-// tile.
-static bool march1_vec(const MarchArgs& a, int64_t nk, const void* part) {
-    const unsigned al = 8u * kM1NP - 1u;
+// Whether a lane's 2 NP adjacent columns can be loaded and stored as one
+// vector: every row of kappa / emis, q_lambda, I_out and the wall row starts
+// aligned to 8 NP bytes, and the range is whole tiles or ends on a multiple of
+// 2 NP columns past the first tile.
+static bool march1_vec(const MarchArgs& a, int64_t nk, const void* part, int NP) {
+    const unsigned al = 8u * NP - 1u;
     const auto ok = [al](const void* q) { return (reinterpret_cast<uintptr_t>(q) & al) == 0; };
-    const int64_t nc = 2 * kM1NP;
-    return nk >= 64 * kM1NP && nk % nc == 0 && a.ld % nc == 0 && ok(a.kappa) && ok(a.emis) && ok(a.q_lambda) &&
+    const int64_t nc = 2 * NP;
+    return nk >= 64 * NP && nk % nc == 0 && a.ld % nc == 0 && ok(a.kappa) && ok(a.emis) && ok(a.q_lambda) &&
            ok(part) && (a.I_out == nullptr || ok(a.I_out));
 }
 
@@ -1229,7 +1233,7 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
     if (B > 0) k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.key);
-    k_ray_pairs<<<(unsigned)P, 256, 0, ctx->stream>>>(a, pl.key, pl.partner, pl.uniq, pl.n_uniq);
+    k_ray_pairs<<<(unsigned)P, 512, 0, ctx->stream>>>(a, pl.key, pl.partner, pl.uniq, pl.n_uniq);
     k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, pl.uniq, pl.n_uniq, G, pl.plan,
                                                              pl.soff, a.status);
     cudaError_t e = cudaGetLastError();
@@ -1242,13 +1246,18 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
             a.lam_min, a.h, a.k0, nk, a.T_wall, a.ph, row);
         b.wall_row = row;
     }
-    dim3 g((unsigned)(P << lgG), div_up(nk, 64 * kM1NP));
-    if (march1_vec(a, nk, part))
-        k_march1<kM1NP, true><<<g, 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner,
-                                                                          reinterpret_cast<float*>(part));
+    // four adjacent columns a lane where 16-byte loads are aligned (100 x 50
+    // cells, 20 points x 512 rays, 16,384 columns: 3.93 ms, two columns 4.16),
+    // two where 8-byte ones are (16,382: 4.24), else two columns 32 apart (16,383:
+    // 4.72, four of them 4.95)
+    float* pf = reinterpret_cast<float*>(part);
+    const auto grid = [&](int np) { return dim3((unsigned)(P << lgG), div_up(nk, 64 * np)); };
+    if (march1_vec(a, nk, part, 2))
+        k_march1<2, true><<<grid(2), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
+    else if (march1_vec(a, nk, part, 1))
+        k_march1<1, true><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
     else
-        k_march1<kM1NP, false><<<g, 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner,
-                                                                          reinterpret_cast<float*>(part));
+        k_march1<1, false><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
     e = cudaGetLastError();
     if (e != cudaSuccess || G == 1) return e;
     k_group_sum<float><<<(unsigned)std::min<int64_t>(div_up(P * nk, 256), 152 * 16), 256, 0, ctx->stream>>>(
