@@ -236,9 +236,7 @@ int rapral_populations(rapral_ctx* ctx, const rapral_species* sp, const rapral_c
         return set_error(ctx, RAPRAL_EINVAL, "null cell or species array");
     cudaSetDevice(ctx->device);
     const Phys ph = make_phys(ctx->codata);
-    cudaError_t e = launch_validate_cells(ctx, cells);
-    if (e == cudaSuccess) e = launch_populations(ctx, sp, cells, lnpref, ph);
-    return cuda_status(ctx, e, "populations");
+    return cuda_status(ctx, launch_populations(ctx, sp, cells, lnpref, ph), "populations");   // checks the cells too
 }
 
 static int check_grid(rapral_ctx* ctx, const rapral_grid* g, int64_t k0, int64_t nk) {

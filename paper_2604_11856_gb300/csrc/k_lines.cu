@@ -188,19 +188,42 @@ __global__ void __launch_bounds__(256) k_line_plan(rapral_lines ln, const double
     if (threadIdx.x == 0 && wblk) atomicMax(wmax, wblk);
 }
 
+// Entries of the sorted x[0, n) below v (UPPER: not above v), by one warp: 32
+// probes a round (four rounds for 320k lines; a thread's bisection is a chain
+// of 18 loads, twice, before a block could begin).
+template <bool UPPER>
+__device__ __forceinline__ int64_t warp_bound(const double* __restrict__ x, int64_t n, double v) {
+    const int lane = threadIdx.x & 31;
+    int64_t a = 0, b = n;
+    while (a < b) {
+        const int64_t step = (b - a + 31) / 32, p = a + lane * step;
+        bool in = false;
+        if (p < b) in = UPPER ? x[p] <= v : x[p] < v;
+        const int c = __popc(__ballot_sync(0xffffffffu, in));   // the probes that are below come first
+        if (c == 0) break;
+        b = min(b, a + c * step);
+        a += (c - 1) * step + 1;
+    }
+    return a;
+}
+
 // Lines whose centre can reach tile t: lam0 within the widest window of the
-// tile's wavelength span (binary search when lam0 is sorted, else all).
+// tile's wavelength span (searched by two warps when lam0 is sorted, else
+// all).  For the whole block; range: two shared words.
 __device__ void tile_candidates(const double* lam0, int64_t L, int sorted, double wmax, double lam_min, double h,
-                                int64_t kt0, int64_t kt1, int64_t* b0, int64_t* b1) {
+                                int64_t kt0, int64_t kt1, int64_t* range, int64_t* b0, int64_t* b1) {
     if (!sorted) { *b0 = 0; *b1 = L; return; }
-    const double lo = lam_min + ((double)kt0 - wmax - 2.0) * h;
-    const double hi = lam_min + ((double)kt1 + wmax + 2.0) * h;
-    int64_t a = 0, b = L;
-    while (a < b) { int64_t m = (a + b) >> 1; if (lam0[m] < lo) a = m + 1; else b = m; }
-    *b0 = a;
-    b = L;
-    while (a < b) { int64_t m = (a + b) >> 1; if (lam0[m] <= hi) a = m + 1; else b = m; }
-    *b1 = a;
+    const int warp = threadIdx.x >> 5;
+    if (warp == 0) {
+        const int64_t a = warp_bound<false>(lam0, L, lam_min + ((double)kt0 - wmax - 2.0) * h);
+        if ((threadIdx.x & 31) == 0) range[0] = a;
+    } else if (warp == 1) {
+        const int64_t a = warp_bound<true>(lam0, L, lam_min + ((double)kt1 + wmax + 2.0) * h);
+        if ((threadIdx.x & 31) == 0) range[1] = a;
+    }
+    __syncthreads();
+    *b0 = range[0];
+    *b1 = range[1];
 }
 
 __global__ void __launch_bounds__(256) k_bin_count(const double* __restrict__ lam0, int64_t L,
@@ -212,8 +235,10 @@ __global__ void __launch_bounds__(256) k_bin_count(const double* __restrict__ la
     const int t = blockIdx.x;
     const int64_t kt0 = k0 + (int64_t)t * tile_w;
     const int64_t kt1 = min(kt0 + tile_w, k0 + nk) - 1;
+    __shared__ int64_t range[2];
     int64_t b0, b1;
-    tile_candidates(lam0, L, !*unsorted, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, &b0, &b1);
+    tile_candidates(lam0, L, !*unsorted, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, range,
+                    &b0, &b1);
     int cnt = 0;
     for (int64_t l = b0 + threadIdx.x; l < b1; l += blockDim.x) {
         const int2 r = line_tiles[l];
@@ -242,8 +267,10 @@ __global__ void __launch_bounds__(256) k_bin_fill(const double* __restrict__ lam
     const int t = blockIdx.x;
     const int64_t kt0 = k0 + (int64_t)t * tile_w;
     const int64_t kt1 = min(kt0 + tile_w, k0 + nk) - 1;
+    __shared__ int64_t range[2];
     int64_t b0, b1;
-    tile_candidates(lam0, L, !*unsorted, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, &b0, &b1);
+    tile_candidates(lam0, L, !*unsorted, __longlong_as_double((long long)*wmaxp), lam_min, h, kt0, kt1, range,
+                    &b0, &b1);
     __shared__ int wsum[8];
     __shared__ int base_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;

@@ -47,7 +47,7 @@ template <int CC>
 __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const double* __restrict__ Ttr,
                                                      const double* __restrict__ Tve, const double* __restrict__ n,
                                                      int32_t ncol, int64_t C, double c2, double* __restrict__ lnpref,
-                                                     const int* status) {
+                                                     int* status) {
     if (*status) return;
     __shared__ uint64_t tab[EXPFIX_N];
     __shared__ double pv[CC][32];      // Boltzmann factors of 32 vibrational levels of a state, with its weight
@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const do
     const int S = sp.n_species, s = blockIdx.y;
     const int64_t c0 = (int64_t)blockIdx.x * CC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (s == 0 && tid < CC && c0 + tid < C) check_cell(Ttr, Tve, n, c0 + tid, ncol, status);
     double bve[CC], btr[CC], z[CC];
     ExpFixScale sc[CC];
 #pragma unroll

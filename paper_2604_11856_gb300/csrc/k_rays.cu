@@ -1060,13 +1060,24 @@ __global__ void k_group_sum(const T* __restrict__ part, int G, int64_t P, int64_
 }
 
 // Spectral integral in two deterministic stages: blocks (point, slice)
-// Neumaier-sum a slice of FLUX_SPAN grid points each, then one block per
-// point adds the slices in order.
-constexpr int FLUX_SPAN = 4096;
+// Neumaier-sum a slice of FLUX_SPAN grid points each, eight a thread, then one
+// warp per point adds the slices, each lane a strided part in order.  Weights
+// other than 1 (the grid's ends) are applied to their points, the spacing once
+// at the end: five FP64 operations a point.
+constexpr int FLUX_SPAN = 2048;
+
+// (s, c) += x, Neumaier; magnitudes are compared by their bits
+__device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
+    const double t = s + x;
+    const bool big = (__double_as_longlong(s) & 0x7fffffffffffffffll) >= (__double_as_longlong(x) & 0x7fffffffffffffffll);
+    const double hi = big ? s : x, lo = big ? x : s;
+    c += (hi - t) + lo;
+    s = t;
+}
 
 template <class T>
 __global__ void __launch_bounds__(256) k_wall_flux_part(const T* __restrict__ qlam, int64_t nk, int64_t k0,
-                                                        int64_t n, double h_um, double2* __restrict__ part,
+                                                        int64_t n, double* __restrict__ part,
                                                         const int* status) {
     if (*status) return;
     const int64_t p = blockIdx.x;
@@ -1074,36 +1085,35 @@ __global__ void __launch_bounds__(256) k_wall_flux_part(const T* __restrict__ ql
     double s = 0.0, c = 0.0;
     for (int64_t k = a + threadIdx.x; k < b; k += blockDim.x) {
         const int64_t kg = k0 + k;
-        const double w = (kg == 0 || kg == n - 1) ? 0.5 : 1.0;
-        const double x = w * (double)qlam[p * nk + k] * h_um;
-        const double t = s + x;
-        if (fabs(s) >= fabs(x)) c += (s - t) + x; else c += (x - t) + s;
-        s = t;
+        double x = (double)qlam[p * nk + k];
+        if (kg == 0 || kg == n - 1) x *= 0.5;
+        neumaier_add(s, c, x);
     }
-    __shared__ double red[256];
-    red[threadIdx.x] = s + c;
+    __shared__ double red[8];
+    double v = s + c;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) v += red[w];
+        part[p * gridDim.y + blockIdx.y] = v;
     }
-    if (threadIdx.x == 0) part[p * gridDim.y + blockIdx.y] = make_double2(red[0], 0.0);
 }
 
-__global__ void __launch_bounds__(32) k_wall_flux_sum(const double2* __restrict__ part, int nparts,
+__global__ void __launch_bounds__(32) k_wall_flux_sum(const double* __restrict__ part, int nparts, double h_um,
                                                       double* __restrict__ q, const int* status) {
     if (*status) return;
     const int64_t p = blockIdx.x;
-    if (threadIdx.x == 0) {
-        double s = 0.0, c = 0.0;
-        for (int i = 0; i < nparts; ++i) {
-            const double x = part[p * nparts + i].x;
-            const double t = s + x;
-            if (fabs(s) >= fabs(x)) c += (s - t) + x; else c += (x - t) + s;
-            s = t;
-        }
-        q[p] += s + c;
+    double s = 0.0, c = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += 32) neumaier_add(s, c, part[p * nparts + i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {   // lane l + o into lane l
+        const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+        neumaier_add(s, c, s2);
+        c += c2;
     }
+    if (threadIdx.x == 0) q[p] += (s + c) * h_um;
 }
 
 // Tangent slab: directions are split into bundles of at most SLAB_DIRS
@@ -1386,17 +1396,17 @@ cudaError_t launch_wall_flux(rapral_ctx* ctx, const void* q_lambda, int precisio
     if (n_points == 0) return cudaSuccess;
     const double h_um = h * 1e-3;
     const int64_t np = wall_flux_parts(nk);
-    double2* part = reinterpret_cast<double2*>(partials);
+    double* part = reinterpret_cast<double*>(partials);
     dim3 grid((unsigned)n_points, (unsigned)np);
     if (precision == RAPRAL_FP64)
         k_wall_flux_part<double><<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const double*>(q_lambda), nk, k0,
-                                                                g->n, h_um, part, ctx->d_status);
+                                                                g->n, part, ctx->d_status);
     else
         k_wall_flux_part<float><<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const float*>(q_lambda), nk, k0,
-                                                               g->n, h_um, part, ctx->d_status);
+                                                               g->n, part, ctx->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_wall_flux_sum<<<(unsigned)n_points, 32, 0, ctx->stream>>>(part, (int)np, q, ctx->d_status);
+    k_wall_flux_sum<<<(unsigned)n_points, 32, 0, ctx->stream>>>(part, (int)np, h_um, q, ctx->d_status);
     return cudaGetLastError();
 }
 
