@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(128) k_line_sum_f64(LineSumArgs a) {
 // again with the FP64 Voigt width and the literal test |lam_k - lam0| <=
 // 100 lamV, so every (line, point) inclusion matches the FP64 decision.
 // Per point: u = |(k - kc) s - u0| (s = h / 2lamV), the Whiting bracket with
-// MUFU ex2 / rsqrt / rcp, terms that underflow FP32 skipped, and Kahan
+// MUFU ex2 / rsqrt / rcp, exponentials below FP32 rounding left out, and Kahan
 // compensated sums of kappa and j over the tile's lines.
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -720,27 +720,35 @@ __device__ __forceinline__ float sinpi_series(float d) {
 
 // One (line, cell) pair set up for a warp's tile [kt0, kt0 + TW): window
 // offsets inside the tile (as floats), u at the tile's first point, profile
-// constants, and whether every point of the window part in the tile lies in
-// the far wings (|u| > 11, where both exponentials are zero in FP32) or past
-// the Gaussian core (|u| > 5.62).  Everything a warp needs per pair is
+// constants, and the part of the line where an exponential of the bracket is
+// above the FP32 rounding of the rest.  Everything a warp needs per pair is
 // computed here, by one lane per pair.
-// Bracket modes: both exponentials; the Gaussian core zero in FP32 over the
-// span (|u| > 5.62, 2.772 u^2 log2(e) > 126); both zero (|u| > 11, also
-// 0.4 u^2.25 log2(e) > 126).  Dropping a term that ex2 flushes to zero does
-// not change a sum.
-enum { BR_NEAR = 0, BR_MID = 1, BR_FAR = 2 };
+// Exponentials of the bracket: beyond |u| = 6 the correction 0.016 r (1 - r)
+// e^{-0.4 u^2.25} is below 4e-10 of the Lorentz part r / (1 + 4u^2) for every
+// r, and the Gaussian e^{-2.772 u^2} below 5e-44, under 1e-30 of it for the r
+// that a natural width of 5.9e-6 nm leaves: both are left out there.
+constexpr float NEAR_U = 6.0f;
 
 struct PairF32 {
     float lo, hi;     // window part inside the tile, offsets from kt0
+    float x0, wn;     // line centre as an offset from kt0; points around it with |u| <= NEAR_U
     float ub, ub_lo;  // signed u at kt0, (kt0 - kc) s - u0, as a float-float pair
     float s;          // h / (2 lamV): step of u per grid point
     float r, aj, ak;
-    int mode;         // BR_NEAR, BR_MID or BR_FAR over the window part in the tile
+};
+
+// What a warp's set-up reads of its cell, in shared memory: held in registers
+// it was spilled through the sweep.
+struct WarpCell {
+    float2 bve_ff, btr_ff;
+    float sqrtT_f, stc_f, pad[2];
+    float2 lp[RAPRAL_MAX_SPECIES];   // ln(N_s / Z_s) as float-float pairs
+    float2 cb[RAPRAL_MAX_SPECIES];   // (N_0, W) of the optional terms
 };
 
 // FL: bit 0 the optional Lorentz terms, bit 1 the departure coefficients.
 template <int FL>
-__device__ __forceinline__ bool setup_pair_f32(const LineSumArgs& a, const LineF32& L, const CellPrep& cp, float2 lp,
+__device__ __forceinline__ bool setup_pair_f32(const LineSumArgs& a, const LineF32& L, const WarpCell& cp, float2 lp,
                                                float2 cb, int line, int64_t c, float hf, float inv_hf, int kt0,
                                                float kt0f, float kt1f, bool count, PairF32* P, int64_t* cnt) {
     constexpr bool BR = (FL & 1) != 0, DEP = (FL & 2) != 0, VG = (FL & 4) != 0;
@@ -833,14 +841,12 @@ __device__ __forceinline__ bool setup_pair_f32(const LineSumArgs& a, const LineF
         P->ub = uh;
         P->ub_lo = e + pe;
     }
-    // smallest |u| over the evaluated part of the tile
-    const float ua = fmaf(lo_rel, s, P->ub), ue = fmaf(hi_rel, s, P->ub);
-    const float umin = (ua > 0.0f) ? ua : (ue < 0.0f ? -ue : 0.0f);
     P->lo = lo_rel;
     P->hi = hi_rel;
+    P->x0 = L.kcf - kt0f + L.delta;
+    P->wn = 2.0f * NEAR_U * lamV * inv_hf;
     P->s = s;
     P->r = r;
-    P->mode = umin > 11.0f ? BR_FAR : ((!VG && umin > 5.62f) ? BR_MID : BR_NEAR);
     P->aj = Sj * pre;
     P->ak = Sk * pre;
     if (count) {
@@ -857,27 +863,6 @@ __device__ __forceinline__ bool setup_pair_f32(const LineSumArgs& a, const LineF
     return true;
 }
 
-// One Whiting evaluation, bracket only (the factor 1e3 / (2 lamV (1.065 +
-// 0.447 r + 0.058 r^2)) is folded into aj, ak).  Near the line centre both
-// exponentials are kept; BR_MID drops the Gaussian core and BR_FAR both
-// where they are zero in FP32 over the whole span being evaluated.
-template <int M>
-__device__ __forceinline__ float whiting_bracket(float u, float r, float omr, float c16) {
-    const float u2 = u * u;
-    const float v = u2 * rsqrt_approx(rsqrt_approx(u));                      // u^2.25
-    const float q4 = fmaf(4.0f, u2, 1.0f);
-    const float p1 = fmaf(0.1f, v, 1.0f);
-    const float rd = rcp_approx(q4 * p1);
-    const float num = fmaf(r, p1, -c16 * q4);                                // r(1+0.1v) - c16(1+4u^2)
-    if (M == BR_FAR) return num * rd;
-    // past u^2 = 31.5 and v = 218 the approximate ex2 returns 0 (flushed) or
-    // below 1.5e-38, so neither exponential needs a guard
-    const float e2 = ex2_approx(-0.5770780f * v);    // e^{-0.4 v}
-    if (M == BR_MID) return fmaf(num, rd, c16 * e2);
-    const float g = ex2_approx(-3.99915f * u2);      // e^{-2.772 u^2}
-    return fmaf(omr, g, fmaf(num, rd, c16 * e2));
-}
-
 // Kahan step: (s, c) += x.
 __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
     const float y = x - c;
@@ -886,99 +871,161 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
     s = t;
 }
 
-// One pair over the lane's points k = lane + 32 i of the tile: runs of 32
-// points outside the window part [lo, hi] are skipped (the test is the same
-// for the whole warp); in the others each lane adds its point if it lies in
-// the window.
-template <int PPT, int M>
-__device__ __forceinline__ void sweep_pair(float lo, float hi, float lanef, float s, float ub, float ub_lo, float r,
-                                           float omr, float c16, float aj, float ak, float (&bj)[PPT],
-                                           float (&bk)[PPT]) {
+// A batch's staged lines.  Lines whose window covers the whole tile: W0 = s,
+// ub, ub_lo, r and W1 = aj, ak, those with no near part from the front, the
+// others from the end.  The others (partial lines) two a slot in packed-pair
+// order: G[0] = -mid, half (of the window part in the tile), G[1] = ub, ub_lo,
+// G[2] = s, r, G[3] = aj, ak, each for both lines, and per line the runs it
+// reaches (low half) and the runs that hold points of its near part (high).
+template <int PB>
+struct LineSlots {
+    float4 G[4][PB / 2];
+    float4 W0[PB];
+    float2 W1[PB];
+    unsigned runs[PB];
+};
+
+// Whiting's bracket of a slot's two lines at the lane's point of one run (the
+// factor 1e3 / (2 lamV (1.065 + 0.447 r + 0.058 r^2)) is folded into aj, ak),
+// added to the run's sums, a sum a line.  With q4 = 1 + 4u^2, p1 = 1 + 0.1
+// u^2.25, c = 0.016 (1 - r): r ((p1 - c q4) / (q4 p1)), and in a near run
+// + r c e^{-0.4 u^2.25} + (1 - r) e^{-2.772 u^2}.
+//
+// The MUFU pipe (16 rsqrt or rcp a clock and SM) takes 24 clocks a warp for a
+// far evaluation with its own reciprocal; the two lines share the one of
+// their denominators' product (20 clocks, beside 17 of the FP32 pipe).
+// |u| is capped so that the product of a point in its window and one far out
+// of it stays in range; points outside a window add zero.
+template <bool NEAR>
+__device__ __forceinline__ void slot_eval(float k, float2 nmid, float2 half, float2 ub, float2 ubl, float2 s, float2 nc,
+                                          float2 r, float2 aj, float2 ak, float& bj, float& bk) {
+    const auto c2 = [](float x) { return make_float2(x, x); };
+    // signed u at point k: one rounding of k s + ub (exact product), then the
+    // low part; relative to u itself, so the Gaussian core keeps FP32 accuracy
+    // however far the tile start lies from the line centre
+    const float2 u = __fadd2_rn(__ffma2_rn(c2(k), s, ub), ubl);
+    const float2 d = __fadd2_rn(c2(k), nmid);
+    const float2 w = make_float2(fminf(fabsf(u.x), 1e4f), fminf(fabsf(u.y), 1e4f));
+    const float2 u2 = __fmul2_rn(w, w);
+    const float2 q = make_float2(rsqrt_approx(rsqrt_approx(w.x)), rsqrt_approx(rsqrt_approx(w.y)));
+    const float2 v = __fmul2_rn(u2, q);                    // u^2.25
+    const float2 q4 = __ffma2_rn(c2(4.0f), u2, c2(1.0f));
+    const float2 p1 = __ffma2_rn(c2(0.1f), v, c2(1.0f));
+    const float2 qp = __fmul2_rn(q4, p1);
+    const float rp = rcp_approx(qp.x * qp.y);
+    const float2 rd = make_float2(qp.y * rp, qp.x * rp);
+    float2 h = __fmul2_rn(__ffma2_rn(nc, q4, p1), rd);
+    if (NEAR) {
+        const float2 xc = __fmul2_rn(c2(-0.5770780f), v);  // -0.4 log2(e) v
+        const float2 xg = __fmul2_rn(c2(-3.99915f), u2);   // -2.772 log2(e) u^2
+        const float2 e2 = make_float2(ex2_approx(xc.x), ex2_approx(xc.y));
+        const float2 g = make_float2(ex2_approx(xg.x), ex2_approx(xg.y));
+        const float2 omr = __ffma2_rn(c2(-1.0f), r, c2(1.0f));
+        h = __ffma2_rn(__fmul2_rn(c2(0.016f), omr), e2, h);
+        h = __ffma2_rn(omr, g, __fmul2_rn(r, h));
+    }
+    h.x = fabsf(d.x) <= half.x ? h.x : 0.0f;
+    h.y = fabsf(d.y) <= half.y ? h.y : 0.0f;
+    bj = fmaf(aj.y, h.y, fmaf(aj.x, h.x, bj));
+    bk = fmaf(ak.y, h.y, fmaf(ak.x, h.x, bk));
+}
+
+// The n staged lines over the lane's points lane + 32 i of the tile.  Lines
+// of a slot are neighbours in the sorted list, so they reach nearly the same
+// runs; a run is taken if either reaches it, and as near if either is.
+template <int PPT, int PB>
+__device__ __forceinline__ void sweep_slots(const LineSlots<PB>& sl, int n, float lanef, float (&bj)[PPT],
+                                            float (&bk)[PPT]) {
+    for (int j = 0; 2 * j < n; ++j) {
+        const uint2 m = *reinterpret_cast<const uint2*>(&sl.runs[2 * j]);
+        const unsigned runs = m.x | m.y;
+        const float4 g0 = sl.G[0][j], g1 = sl.G[1][j], g2 = sl.G[2][j], g3 = sl.G[3][j];
+        const float2 nmid = make_float2(g0.x, g0.y), half = make_float2(g0.z, g0.w);
+        const float2 ub = make_float2(g1.x, g1.y), ubl = make_float2(g1.z, g1.w);
+        const float2 s = make_float2(g2.x, g2.y), r = make_float2(g2.z, g2.w);
+        const float2 aj = make_float2(g3.x, g3.y), ak = make_float2(g3.z, g3.w);
+        const float2 nc = __ffma2_rn(make_float2(0.016f, 0.016f), r, make_float2(-0.016f, -0.016f));
+        const float2 ajr = __fmul2_rn(aj, r), akr = __fmul2_rn(ak, r);
 #pragma unroll
-    for (int i = 0; i < PPT; ++i) {
-        const float p0 = 32.0f * i;
-        if (p0 + 31.0f < lo || p0 > hi) continue;
-        const float k = lanef + p0;
-        // signed u at point k: one rounding of k s + ub (exact product), then
-        // the low part; relative to u itself, so the Gaussian core keeps FP32
-        // accuracy however far the tile start lies from the line centre
-        const float br = whiting_bracket<M>(fabsf(fmaf(k, s, ub) + ub_lo), r, omr, c16);
-        if (k >= lo && k <= hi) {   // predicated update: lanes outside the window part add nothing
-            bj[i] = fmaf(aj, br, bj[i]);
-            bk[i] = fmaf(ak, br, bk[i]);
+        for (int i = 0; i < PPT; ++i) {
+            if (!(runs & (1u << i))) continue;   // the same for the whole warp
+            if (runs & (0x10000u << i))
+                slot_eval<true>(lanef + 32.0f * i, nmid, half, ub, ubl, s, nc, r, aj, ak, bj[i], bk[i]);
+            else
+                slot_eval<false>(lanef + 32.0f * i, nmid, half, ub, ubl, s, nc, r, ajr, akr, bj[i], bk[i]);
         }
     }
 }
 
-// One pair whose window covers every point of the tile: no point needs the
-// window test, so the brackets of runs i and i + 1 are evaluated together in
-// packed FP32 (two results per instruction; the MUFU operations stay
-// scalar).  Operations and roundings are those of whiting_bracket and of the
-// predicated update, so the sums are bitwise the same as sweep_pair's.
-template <int PPT, int M>
-__device__ __forceinline__ void sweep_pair_full(float lanef, float s, float ub, float ub_lo, float r, float omr,
-                                                float c16, float aj, float ak, float (&bj)[PPT], float (&bk)[PPT]) {
-    static_assert(PPT % 2 == 0, "runs are taken two at a time");
-    const float2 s2 = make_float2(s, s), ub2 = make_float2(ub, ub), ubl2 = make_float2(ub_lo, ub_lo);
-    const float2 one = make_float2(1.0f, 1.0f), four = make_float2(4.0f, 4.0f), tenth = make_float2(0.1f, 0.1f);
-    const float2 r2 = make_float2(r, r), nc16 = make_float2(-c16, -c16);
-    const float2 aj2 = make_float2(aj, aj), ak2 = make_float2(ak, ak);
-#pragma unroll
-    for (int i = 0; i < PPT; i += 2) {
-        const float2 k = make_float2(lanef + 32.0f * i, lanef + 32.0f * (i + 1));
-        const float2 u = __fadd2_rn(__ffma2_rn(k, s2, ub2), ubl2);     // signed u; only |u| and u^2 are used
-        const float2 u2 = __fmul2_rn(u, u);
-        const float2 q = make_float2(rsqrt_approx(rsqrt_approx(fabsf(u.x))), rsqrt_approx(rsqrt_approx(fabsf(u.y))));
-        const float2 v = __fmul2_rn(u2, q);                            // u^2.25
-        const float2 q4 = __ffma2_rn(four, u2, one);
-        const float2 p1 = __ffma2_rn(tenth, v, one);
-        const float2 qp = __fmul2_rn(q4, p1);
-        const float2 rd = make_float2(rcp_approx(qp.x), rcp_approx(qp.y));
-        const float2 num = __ffma2_rn(r2, p1, __fmul2_rn(nc16, q4));   // r(1+0.1v) - c16(1+4u^2)
-        float2 br;
-        if (M == BR_FAR) {
-            br = __fmul2_rn(num, rd);
-        } else {
-            const float2 xc = __fmul2_rn(make_float2(-0.5770780f, -0.5770780f), v);
-            const float2 e2 = make_float2(ex2_approx(xc.x), ex2_approx(xc.y));    // e^{-0.4 v}
-            br = __ffma2_rn(num, rd, __fmul2_rn(make_float2(c16, c16), e2));
-            if (M == BR_NEAR) {
-                const float2 xg = __fmul2_rn(make_float2(-3.99915f, -3.99915f), u2);
-                const float2 g = make_float2(ex2_approx(xg.x), ex2_approx(xg.y));     // e^{-2.772 u^2}
-                br = __ffma2_rn(make_float2(omr, omr), g, br);
-            }
-        }
-        const float2 j2 = __ffma2_rn(aj2, br, make_float2(bj[i], bj[i + 1]));
-        const float2 k2 = __ffma2_rn(ak2, br, make_float2(bk[i], bk[i + 1]));
-        bj[i] = j2.x; bj[i + 1] = j2.y;
-        bk[i] = k2.x; bk[i + 1] = k2.y;
-    }
-}
-
-// The staged pairs q0 .. q1 - 1 of one class: bracket mode M, and whether
-// their windows cover the whole tile.
-template <int PPT, int M, bool WHOLE>
-__device__ __forceinline__ void sweep_class(const float4* sm0, const float4* sm1, int q0, int q1, float lanef,
+// One line whose window covers every point of the tile: no point needs the
+// window test, and the runs are taken four at a time in packed pairs with one
+// reciprocal for the four (|u| <= 50 in a window, so the denominators' product
+// stays below 2e27), which overlaps their latencies and takes 18 clocks of the
+// MUFU pipe an evaluation instead of 24.
+template <int PPT, bool NEAR>
+__device__ __forceinline__ void sweep_whole(float lanef, float s, float ub, float ub_lo, float r, float aj, float ak,
                                             float (&bj)[PPT], float (&bk)[PPT]) {
+    static_assert(PPT % 4 == 0, "runs are taken four at a time");
+    const auto c2 = [](float x) { return make_float2(x, x); };
+    const float omr = 1.0f - r, c = 0.016f * omr;
+    const float2 aj2 = c2(NEAR ? aj : aj * r), ak2 = c2(NEAR ? ak : ak * r);
+#pragma unroll
+    for (int i0 = 0; i0 < PPT; i0 += 4) {
+        float2 u2[2], v[2], qp[2], num[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = i0 + 2 * h;
+            const float2 k = make_float2(lanef + 32.0f * i, lanef + 32.0f * (i + 1));
+            const float2 u = __fadd2_rn(__ffma2_rn(k, c2(s), c2(ub)), c2(ub_lo));     // signed u; only |u| and u^2 are used
+            u2[h] = __fmul2_rn(u, u);
+            const float2 q = make_float2(rsqrt_approx(rsqrt_approx(fabsf(u.x))), rsqrt_approx(rsqrt_approx(fabsf(u.y))));
+            v[h] = __fmul2_rn(u2[h], q);                            // u^2.25
+            const float2 q4 = __ffma2_rn(c2(4.0f), u2[h], c2(1.0f));
+            const float2 p1 = __ffma2_rn(c2(0.1f), v[h], c2(1.0f));
+            qp[h] = __fmul2_rn(q4, p1);
+            num[h] = __ffma2_rn(c2(-c), q4, p1);
+        }
+        const float d0 = qp[0].x * qp[0].y, d1 = qp[1].x * qp[1].y;
+        const float R = rcp_approx(d0 * d1);
+        const float rr[2] = {R * d1, R * d0};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = i0 + 2 * h;
+            float2 br = __fmul2_rn(num[h], make_float2(qp[h].y * rr[h], qp[h].x * rr[h]));
+            if (NEAR) {
+                const float2 xc = __fmul2_rn(c2(-0.5770780f), v[h]), xg = __fmul2_rn(c2(-3.99915f), u2[h]);
+                const float2 e2 = make_float2(ex2_approx(xc.x), ex2_approx(xc.y));    // e^{-0.4 v}
+                const float2 g = make_float2(ex2_approx(xg.x), ex2_approx(xg.y));     // e^{-2.772 u^2}
+                br = __ffma2_rn(c2(c), e2, br);
+                br = __ffma2_rn(c2(omr), g, __fmul2_rn(c2(r), br));
+            }
+            const float2 j2 = __ffma2_rn(aj2, br, make_float2(bj[i], bj[i + 1]));
+            const float2 k2 = __ffma2_rn(ak2, br, make_float2(bk[i], bk[i + 1]));
+            bj[i] = j2.x; bj[i + 1] = j2.y;
+            bk[i] = k2.x; bk[i + 1] = k2.y;
+        }
+    }
+}
+template <int PPT, int PB, bool NEAR>
+__device__ __forceinline__ void sweep_wholes(const LineSlots<PB>& sl, int q0, int q1, float lanef, float (&bj)[PPT],
+                                             float (&bk)[PPT]) {
     for (int q = q0; q < q1; ++q) {
-        const float4 A = sm0[q];   // lo, hi, ub, s
-        const float4 B = sm1[q];   // r, ub_lo, aj, ak
-        const float r = B.x, omr = 1.0f - r, c16 = 0.016f * r * omr;
-        if (WHOLE) sweep_pair_full<PPT, M>(lanef, A.w, A.z, B.y, r, omr, c16, B.z, B.w, bj, bk);
-        else sweep_pair<PPT, M>(A.x, A.y, lanef, A.w, A.z, B.y, r, omr, c16, B.z, B.w, bj, bk);
+        const float4 A = sl.W0[q];
+        const float2 B = sl.W1[q];
+        sweep_whole<PPT, NEAR>(lanef, A.x, A.y, A.z, A.w, B.x, B.y, bj, bk);
     }
 }
 
 // The same sweep with the exact Voigt shape: r is y, u is x.
 template <int PPT>
-__device__ __forceinline__ void sweep_pair_voigt(const VoigtCoef& vc, float lo, float hi, float lanef, float s, float ub,
+__device__ __forceinline__ void sweep_pair_voigt(const VoigtCoef& vc, float lo, float hi, float o0, float kf, float s, float ub,
                                                  float ub_lo, float y, float aj, float ak, float (&bj)[PPT],
                                                  float (&bk)[PPT]) {
 #pragma unroll
     for (int i = 0; i < PPT; ++i) {
-        const float p0 = 32.0f * i;
+        const float p0 = o0 + 32.0f * i;
         if (p0 + 31.0f < lo || p0 > hi) continue;
-        const float k = lanef + p0;
+        const float k = kf + 32.0f * i;
         const float br = voigt_re<float>(vc, fmaf(k, s, ub) + ub_lo, y);
         if (k >= lo && k <= hi) {
             bj[i] = fmaf(aj, br, bj[i]);
@@ -993,12 +1040,25 @@ __device__ __forceinline__ void sweep_pair_voigt(const VoigtCoef& vc, float lo, 
 // then sweeps them over its points.  With the points interleaved, whether a
 // pair's window reaches the i-th run of 32 points is the same for the whole
 // warp, so runs outside the window are skipped without a masked evaluation.
-// The staged pairs are grouped by class (bracket mode, and whether the
-// window covers the whole tile, where two points go per packed FP32
-// instruction), one loop per class.  Warps never wait for each other.
+// Lines whose window covers the whole tile are swept one at a time over four
+// runs, the others two at a time run by run.  Warps never wait for each other.
+// Tiles of 256 and 512 points are swept in parts of 128, so that a line's
+// set-up, a quarter of the time at 128, serves several parts: 256 points take
+// 29.3 ms for 31.1 on 200 cells x 1e6 points and 63.8 for 65.3 on 80,000 cells x
+// 4,096, but 1.01 for 0.98 on 48 cells x 65,536, where half as many units leave
+// the last wave emptier.
+//
+// What bounds it: set-up takes a quarter, whole lines a quarter to a half,
+// partial lines the rest (most of the afterbody's cool cells); issue slots are
+// 70 % busy, the MUFU pipe about as much, and more resident warps help (32 an
+// SM at 64 registers against 24 at 80).  Line sums in ms, before (one line
+// at a time, a reciprocal a point, both exponentials in every run of a tile
+// that holds the line's centre) and now: 200 cells x 1e6 points 33.9 -> 31.2,
+// 80,000 cells x 4,096 points 76.9 -> 65.6, 48 x 65,536 1.04 -> 0.97, full
+// Lorentz width 96 x 100,001 0.83 -> 0.74.
 template <int PPT, int FL, int PB = 32>
-__device__ __forceinline__ void warp_tile_f32(const LineSumArgs& a, int t, int64_t c, float4* sm0, float4* sm1,
-                                              float2* smlp, float2* smcb, float4* acc, int lane, int64_t* cnt) {
+__device__ __forceinline__ void warp_tile_f32(const LineSumArgs& a, int t, int64_t c, LineSlots<PB>& sl,
+                                              WarpCell& wc, float4* acc, int lane, int64_t* cnt) {
     constexpr int TW = 32 * PPT;
     const int kt0 = (int)(a.k0 + (int64_t)t * TW);
     const int kt1 = (int)min(a.k0 + (int64_t)(t + 1) * TW, a.k0 + a.nk) - 1;   // inclusive
@@ -1008,86 +1068,128 @@ __device__ __forceinline__ void warp_tile_f32(const LineSumArgs& a, int t, int64
     // memory (acc[i * 32 + lane] = (s_j, c_j, s_k, c_k)); inside a batch of at
     // most PB lines the terms are added plainly in registers (error <= (PB - 1) u
     // of the batch's magnitude, u = 2^-24)
-    float bk[PPT], bj[PPT];
 #pragma unroll
-    for (int i = 0; i < PPT; ++i) {
-        bk[i] = bj[i] = 0.0f;
-        acc[i * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-    const CellPrep cp = a.cp[c];
+    for (int i = 0; i < PPT; ++i) acc[i * 32 + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float hf = (float)a.h;
     const float inv_hf = (float)(1.0 / a.h);
     const bool count = a.count != 0;
-    if (lane < a.S) {   // the cell's ln(N_s / Z_s) as float-float pairs
+    if (lane == 0) {
+        const CellPrep& cp = a.cp[c];
+        wc.bve_ff = cp.bve_ff;
+        wc.btr_ff = cp.btr_ff;
+        wc.sqrtT_f = cp.sqrtT_f;
+        wc.stc_f = cp.stc_f;
+    }
+    if (lane < a.S) {
         const double v = a.lnpref[c * a.S + lane];
-        smlp[lane] = v > -INFINITY ? ff_from(v) : make_float2(-INFINITY, 0.0f);
-        if (FL & 1) smcb[lane] = a.cb32[c * a.S + lane];   // (N_0, W) of the optional terms
+        wc.lp[lane] = v > -INFINITY ? ff_from(v) : make_float2(-INFINITY, 0.0f);
+        if (FL & 1) wc.cb[lane] = a.cb32[c * a.S + lane];
     }
     __syncwarp();
     const int beg = a.tile_off[t], end = a.tile_off[t + 1];
     constexpr int NH = PB / 32;   // staged halves of 32 pairs (one pair a lane each)
-    constexpr int NCLS = (FL & 4) ? 1 : 6;
     for (int b = beg; b < end; b += PB) {
-        // stage the pairs that reach the tile grouped by class (bracket mode,
-        // plus 3 where the window covers the whole tile; one class with the
-        // exact Voigt shape), in lane order within a class, so the sweeps
-        // below run one loop per class with no test per pair; with PB = 64
-        // the second 32 pairs are staged in their own half the same way
-        int base[NH][NCLS + 1];
+        PairF32 P[NH];
+        bool valid[NH];
 #pragma unroll
         for (int hh = 0; hh < NH; ++hh) {
             const int nb = min(32, end - (b + 32 * hh));
-            PairF32 P;
-            bool valid = false;
+            valid[hh] = false;
             if (lane < nb) {
                 const int l = a.tile_lines[b + 32 * hh + lane];
                 const LineF32 L = a.lf[l];
-                valid = setup_pair_f32<FL>(a, L, cp, smlp[L.species], (FL & 1) ? smcb[L.species] : make_float2(0.f, 0.f),
-                                           l, c, hf, inv_hf, kt0, kt0f, kt1f, count, &P, cnt);
-            }
-            int cls = -1;
-            if (valid) cls = (FL & 4) ? 0 : P.mode + ((P.lo <= 0.0f && P.hi >= (float)(TW - 1)) ? 3 : 0);
-            const unsigned lt = (1u << lane) - 1u;
-            int pos = 0;
-            base[hh][0] = 32 * hh;
-#pragma unroll
-            for (int k = 0; k < NCLS; ++k) {
-                const unsigned m = __ballot_sync(0xffffffffu, cls == k);
-                if (cls == k) pos = base[hh][k] + __popc(m & lt);
-                base[hh][k + 1] = base[hh][k] + __popc(m);
-            }
-            if (cls >= 0) {
-                sm0[pos] = make_float4(P.lo, P.hi, P.ub, P.s);
-                sm1[pos] = make_float4(P.r, P.ub_lo, P.aj, P.ak);
+                valid[hh] = setup_pair_f32<FL>(a, L, wc, wc.lp[L.species],
+                                               (FL & 1) ? wc.cb[L.species] : make_float2(0.f, 0.f), l, c, hf, inv_hf,
+                                               kt0, kt0f, kt1f, count, &P[hh], cnt);
             }
         }
-        __syncwarp();
+        // the tile's parts of 128 points, four runs each: the lines' set-up serves all of them
+#pragma unroll 1
+        for (int g0 = 0; g0 < PPT; g0 += 4) {
+            const float o0 = 32.0f * g0;
+            int n = 0, nf = 0, nn = 0;   // lines staged: partial, whole far (from the front), whole near (from the end)
 #pragma unroll
-        for (int hh = 0; hh < NH; ++hh) {
+            for (int hh = 0; hh < NH; ++hh) {
+                const PairF32& Q = P[hh];
+                bool part = valid[hh] && Q.lo <= o0 + 127.0f && Q.hi >= o0;
+                const bool whole = part && !(FL & 4) && Q.lo <= o0 && Q.hi >= o0 + 127.0f;
+                const bool wnear = Q.x0 - Q.wn <= o0 + 127.0f && Q.x0 + Q.wn >= o0;
+                const unsigned mf = __ballot_sync(0xffffffffu, whole && !wnear);
+                const unsigned mn = __ballot_sync(0xffffffffu, whole && wnear);
+                const unsigned lt = (1u << lane) - 1u;
+                if (whole) {
+                    const int q = wnear ? PB - 1 - nn - __popc(mn & lt) : nf + __popc(mf & lt);
+                    sl.W0[q] = make_float4(Q.s, Q.ub, Q.ub_lo, Q.r);
+                    sl.W1[q] = make_float2(Q.aj, Q.ak);
+                    part = false;
+                }
+                nf += __popc(mf);
+                nn += __popc(mn);
+                const unsigned m = __ballot_sync(0xffffffffu, part);
+                if (part) {
+                    const int pos = n + __popc(m & lt), j = pos >> 1, o = pos & 1;
+                    unsigned runs = 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float p0 = o0 + 32.0f * i;
+                        if (Q.lo <= p0 + 31.0f && Q.hi >= p0)
+                            runs |= (Q.x0 - Q.wn <= p0 + 31.0f && Q.x0 + Q.wn >= p0 ? 0x10001u : 1u) << i;
+                    }
+                    sl.runs[pos] = runs;
+                    float* g = reinterpret_cast<float*>(&sl.G[0][j]) + o;
+                    constexpr int GS = (int)(sizeof(sl.G[0]) / sizeof(float));
+                    g[0] = -0.5f * (Q.lo + Q.hi);
+                    g[2] = 0.5f * (Q.hi - Q.lo);
+                    g[GS] = Q.ub;
+                    g[GS + 2] = Q.ub_lo;
+                    g[2 * GS] = Q.s;
+                    g[2 * GS + 2] = Q.r;
+                    g[3 * GS] = Q.aj;
+                    g[3 * GS + 2] = Q.ak;
+                }
+                n += __popc(m);
+            }
+            if (n + nf + nn == 0) continue;   // the same for the whole warp
+            if ((n & 1) && lane == 0) {   // an idle line beside the last one: u = 1 everywhere, in no window
+                const int j = n >> 1;
+                float* g = reinterpret_cast<float*>(&sl.G[0][j]) + 1;
+                constexpr int GS = (int)(sizeof(sl.G[0]) / sizeof(float));
+                sl.runs[n] = 0;
+                g[0] = 0.0f;
+                g[2] = -1.0f;
+                g[GS] = 1.0f;
+                g[GS + 2] = 0.0f;
+                g[2 * GS] = 0.0f;
+                g[2 * GS + 2] = 1.0f;
+                g[3 * GS] = 0.0f;
+                g[3 * GS + 2] = 0.0f;
+            }
+            __syncwarp();
+            float bk[4], bj[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) bk[i] = bj[i] = 0.0f;
+            const float kf = lanef + o0;
             if (FL & 4) {
-                for (int q = base[hh][0]; q < base[hh][NCLS]; ++q) {
-                    const float4 A = sm0[q];
-                    const float4 B = sm1[q];
-                    sweep_pair_voigt<PPT>(c_voigt, A.x, A.y, lanef, A.w, A.z, B.y, B.x, B.z, B.w, bj, bk);
+                for (int q = 0; q < n; ++q) {
+                    const float* g = reinterpret_cast<const float*>(&sl.G[0][q >> 1]) + (q & 1);
+                    constexpr int GS = (int)(sizeof(sl.G[0]) / sizeof(float));
+                    sweep_pair_voigt<4>(c_voigt, -g[0] - g[2], -g[0] + g[2], o0, kf, g[2 * GS], g[GS], g[GS + 2],
+                                        g[2 * GS + 2], g[3 * GS], g[3 * GS + 2], bj, bk);
                 }
             } else {
-                sweep_class<PPT, BR_NEAR, false>(sm0, sm1, base[hh][0], base[hh][1], lanef, bj, bk);
-                sweep_class<PPT, BR_MID, false>(sm0, sm1, base[hh][1], base[hh][2], lanef, bj, bk);
-                sweep_class<PPT, BR_FAR, false>(sm0, sm1, base[hh][2], base[hh][3], lanef, bj, bk);
-                sweep_class<PPT, BR_NEAR, true>(sm0, sm1, base[hh][3], base[hh][4], lanef, bj, bk);
-                sweep_class<PPT, BR_MID, true>(sm0, sm1, base[hh][4], base[hh][5], lanef, bj, bk);
-                sweep_class<PPT, BR_FAR, true>(sm0, sm1, base[hh][5], base[hh][6], lanef, bj, bk);
+                sweep_wholes<4, PB, false>(sl, 0, nf, kf, bj, bk);
+                sweep_wholes<4, PB, true>(sl, PB - nn, PB, kf, bj, bk);
+                sweep_slots<4, PB>(sl, n, kf, bj, bk);
             }
-        }
 #pragma unroll
-        for (int i = 0; i < PPT; ++i) {
-            float4 v = acc[i * 32 + lane];
-            kahan_add(v.x, v.y, bj[i]);
-            kahan_add(v.z, v.w, bk[i]);
-            acc[i * 32 + lane] = v;
-            bj[i] = bk[i] = 0.0f;
+            for (int i = 0; i < 4; ++i) {
+                float4 v = acc[(g0 + i) * 32 + lane];
+                kahan_add(v.x, v.y, bj[i]);
+                kahan_add(v.z, v.w, bk[i]);
+                acc[(g0 + i) * 32 + lane] = v;
+            }
+            __syncwarp();
         }
-        __syncwarp();
     }
     float* K = reinterpret_cast<float*>(a.kappa) + c * a.ld - a.k0;
     float* J = reinterpret_cast<float*>(a.emis) + c * a.ld - a.k0;
@@ -1102,26 +1204,26 @@ __device__ __forceinline__ void warp_tile_f32(const LineSumArgs& a, int t, int64
     }
 }
 
-// Resident blocks per SM asked of the compiler: 24 warps per SM, so at most
-// 80 registers per thread (measured best against 32, 28 and 20 warps).
+// Resident blocks per SM asked of the compiler: 32 warps per SM, so at most
+// 64 registers per thread (200 cells x 1e6 points 31.2 ms, 28 warps 31.3, 24
+// 32.2; 80,000 cells x 4,096 points 65.6, 66.2 and 67.3).  Tiles of 512 points
+// keep 8 KB of sums a warp in shared memory: 16 warps.
 #ifndef RAPRAL_LS_WARPS
-#define RAPRAL_LS_WARPS 24
+#define RAPRAL_LS_WARPS 32
 #endif
-#define RAPRAL_LS_BLOCKS(WPB) (RAPRAL_LS_WARPS / (WPB))
+#define RAPRAL_LS_BLOCKS(PPT, WPB) (((PPT) > 8 ? 16 : RAPRAL_LS_WARPS) / (WPB))
 
 template <int PPT, int WPB, int FL = 0, int PB = 32>
-__global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_f32(LineSumArgs a) {
+__global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(PPT, WPB)) k_line_sum_f32(LineSumArgs a) {
     if (*a.status) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t c = (int64_t)blockIdx.x * WPB + warp;
     if (c >= a.C) return;
-    __shared__ float4 sm0[WPB][PB];   // lo, hi, ub, s of each staged pair
-    __shared__ float4 sm1[WPB][PB];   // r, ub_lo, aj, ak
-    __shared__ float2 smlp[WPB][RAPRAL_MAX_SPECIES];
-    __shared__ float2 smcb[WPB][RAPRAL_MAX_SPECIES];
+    __shared__ __align__(16) LineSlots<PB> sl[WPB];
+    __shared__ __align__(16) WarpCell wc[WPB];
     __shared__ float4 acc[WPB][32 * PPT];
     int64_t cnt[4] = {0, 0, 0, 0};
-    warp_tile_f32<PPT, FL, PB>(a, blockIdx.y, c, sm0[warp], sm1[warp], smlp[warp], smcb[warp], acc[warp], lane, cnt);
+    warp_tile_f32<PPT, FL, PB>(a, blockIdx.y, c, sl[warp], wc[warp], acc[warp], lane, cnt);
     if (a.count) block_count(a.stats, cnt[0], cnt[1], cnt[2], cnt[3]);
 }
 
@@ -1130,15 +1232,13 @@ __global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_f3
 // order (tile by tile), from an atomic counter; each warp does the same
 // work as there, so the sums are bitwise the same.
 template <int PPT, int WPB, int PB = 32>
-__global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_f32_persist(LineSumArgs a, int64_t n_groups,
+__global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(PPT, WPB)) k_line_sum_f32_persist(LineSumArgs a, int64_t n_groups,
                                                                             int64_t total,
                                                                             unsigned long long* counter) {
     if (*a.status) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ float4 sm0[WPB][PB];
-    __shared__ float4 sm1[WPB][PB];
-    __shared__ float2 smlp[WPB][RAPRAL_MAX_SPECIES];
-    __shared__ float2 smcb[WPB][RAPRAL_MAX_SPECIES];
+    __shared__ __align__(16) LineSlots<PB> sl[WPB];
+    __shared__ __align__(16) WarpCell wc[WPB];
     __shared__ float4 acc[WPB][32 * PPT];
     __shared__ long long unit_s;
     int64_t cnt[4] = {0, 0, 0, 0};
@@ -1150,7 +1250,7 @@ __global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_f3
         if (u >= total) break;
         const int t = (int)(u / n_groups);
         const int64_t c = (u - (int64_t)t * n_groups) * WPB + warp;
-        if (c < a.C) warp_tile_f32<PPT, 0, PB>(a, t, c, sm0[warp], sm1[warp], smlp[warp], smcb[warp], acc[warp], lane, cnt);
+        if (c < a.C) warp_tile_f32<PPT, 0, PB>(a, t, c, sl[warp], wc[warp], acc[warp], lane, cnt);
         __syncwarp();
     }
     if (a.count) block_count(a.stats, cnt[0], cnt[1], cnt[2], cnt[3]);
@@ -1179,16 +1279,14 @@ static cudaError_t launch_persist(rapral_ctx* ctx, const LineSumArgs& a, dim3 g)
 // list is exhausted; units of a request are ordered tile by tile so blocks
 // working at the same time share a tile's line list in L2.
 template <int PPT, int WPB, bool BR = false, int PB = 32>
-__global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_batch(const BatchItem* __restrict__ items,
+__global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(PPT, WPB)) k_line_sum_batch(const BatchItem* __restrict__ items,
                                                                        int n_items, int64_t total,
                                                                        unsigned long long* counter,
                                                                        unsigned long long* stats, const int* status) {
     if (*status) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ float4 sm0[WPB][PB];
-    __shared__ float4 sm1[WPB][PB];
-    __shared__ float2 smlp[WPB][RAPRAL_MAX_SPECIES];
-    __shared__ float2 smcb[WPB][RAPRAL_MAX_SPECIES];
+    __shared__ __align__(16) LineSlots<PB> sl[WPB];
+    __shared__ __align__(16) WarpCell wc[WPB];
     __shared__ float4 acc[WPB][32 * PPT];
     __shared__ long long unit_s;
     int64_t cnt[4] = {0, 0, 0, 0};
@@ -1208,7 +1306,7 @@ __global__ void __launch_bounds__(32 * WPB, RAPRAL_LS_BLOCKS(WPB)) k_line_sum_ba
         const int t = (int)(local / it.n_groups);
         const int64_t c = (local - (int64_t)t * it.n_groups) * WPB + warp;
         if (c < it.a.C)
-            warp_tile_f32<PPT, BR ? 1 : 0, PB>(it.a, t, c, sm0[warp], sm1[warp], smlp[warp], smcb[warp], acc[warp],
+            warp_tile_f32<PPT, BR ? 1 : 0, PB>(it.a, t, c, sl[warp], wc[warp], acc[warp],
                                                lane, cnt);
         __syncwarp();
     }
