@@ -35,36 +35,45 @@ __device__ __forceinline__ float recip(float x) {
 
 // FP64.  The FP64 pipe has 1/64 of the FP32 rate here, so a step costs its
 // count of FP64 operations.  The series is entered at the length |t| needs
-// (truncation below 1e-17 relative: 3 terms below 2^-17, 5 below 2^-10, 9
-// below 2^-4, 14 below 1/2; the lanes of a warp share the tail), and |t| is
+// (truncation below 2e-17 relative: 3, 4, 5, 6, 9, 14 terms below 2^-17, 2^-13,
+// 2^-10, 2^-7, 2^-4, 1/2; the lanes of a warp share the tail), and |t| is
 // compared by its high word on the integer pipe.  A thin step is 8 to 20 FP64
 // operations; with an expm1 and two divisions whatever its t it took the
-// time of 75 (61 cells x 25 directions x 100,001 points: 18.6 -> 5.6 ms).
-constexpr int T64_17 = 0x3EE00000, T64_10 = 0x3F500000, T64_4 = 0x3FB00000, T64_1 = 0x3FE00000;   // 2^-k
+// time of 75 (61 cells x 25 directions x 100,001 points: 18.8 -> 5.5 ms).
+constexpr int hi_2m(int k) { return (1023 - k) << 20; }   // high word of 2^-k
+constexpr int T64_1 = hi_2m(1);
 __device__ __forceinline__ int abs_hi(double t) { return __double2hiint(t) & 0x7fffffff; }
 __device__ __forceinline__ double thin_series(double t, int hi) {
     double p;
-    if (hi < T64_17) {
+    if (hi < hi_2m(17)) {
         p = 1.0 / 24.0;
     } else {
-        if (hi < T64_10) {
-            p = 1.0 / 720.0;
+        if (hi < hi_2m(13)) {
+            p = -1.0 / 120.0;
         } else {
-            if (hi < T64_4) {
-                p = 1.0 / 3628800.0;
+            if (hi < hi_2m(10)) {
+                p = 1.0 / 720.0;
             } else {
-                p = fma(t, -1.0 / 1307674368000.0, 1.0 / 87178291200.0);
-                p = fma(t, p, -1.0 / 6227020800.0);
-                p = fma(t, p, 1.0 / 479001600.0);
-                p = fma(t, p, -1.0 / 39916800.0);
-                p = fma(t, p, 1.0 / 3628800.0);
+                if (hi < hi_2m(7)) {
+                    p = -1.0 / 5040.0;
+                } else {
+                    if (hi < hi_2m(4)) {
+                        p = 1.0 / 3628800.0;
+                    } else {
+                        p = fma(t, -1.0 / 1307674368000.0, 1.0 / 87178291200.0);
+                        p = fma(t, p, -1.0 / 6227020800.0);
+                        p = fma(t, p, 1.0 / 479001600.0);
+                        p = fma(t, p, -1.0 / 39916800.0);
+                        p = fma(t, p, 1.0 / 3628800.0);
+                    }
+                    p = fma(t, p, -1.0 / 362880.0);
+                    p = fma(t, p, 1.0 / 40320.0);
+                    p = fma(t, p, -1.0 / 5040.0);
+                }
+                p = fma(t, p, 1.0 / 720.0);
             }
-            p = fma(t, p, -1.0 / 362880.0);
-            p = fma(t, p, 1.0 / 40320.0);
-            p = fma(t, p, -1.0 / 5040.0);
-            p = fma(t, p, 1.0 / 720.0);
+            p = fma(t, p, -1.0 / 120.0);
         }
-        p = fma(t, p, -1.0 / 120.0);
         p = fma(t, p, 1.0 / 24.0);
     }
     p = fma(t, p, -1.0 / 6.0);
@@ -175,9 +184,7 @@ __device__ __forceinline__ void dir_pair(float& I0, float& I1, float2 t0, float2
 }
 template <class T, int MAXD>
 __device__ __forceinline__ void dir_steps(T (&I)[MAXD], T kf, T ds, const T* sc, T scmax, int nd, T jf, T jn) {
-    if constexpr (MAXD == 1) {
-        seg_step(I[0], kf, ds, jf, jn);
-    } else if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 4) {
         const float t0 = -kf * ds;
         const float2 t2 = f2c(t0), jd = f2c(ds * jf), dj = f2c(ds * (jn - jf));
         const float tm = fabsf(t0) * scmax;
@@ -364,23 +371,71 @@ __device__ __forceinline__ void march_nodes(const MarchArgs& a, int64_t b, T sc,
     }
 }
 
-template <class T, int V, int MAXD>
-__device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int64_t d0, int nd, SegStage<T>* stage,
+// The march of a bundle of several directions over the lane's column: a step
+// of 17 directions is about 150 FP32 instructions a warp.  The next MPF cells
+// are in flight, across the staging seams: entry j of the stage holds the
+// length of segment j and the row of the cell that step j + MPF needs (two,
+// three, four and six ahead take the same time).
+template <class T, int MAXD>
+__device__ __forceinline__ void march_multi(const MarchArgs& a, int64_t b, int64_t d0, int nd, SegStage<T>* stage,
+                                            int lane, const char* kbase, int64_t ldb, int64_t offK, int64_t offJ,
+                                            int col0, T (&I)[1][MAXD]) {
+    constexpr int MPF = 2;
+    T sc[MAXD], scmax = T(0);
+#pragma unroll
+    for (int d = 0; d < MAXD; ++d) {
+        sc[d] = d < nd ? dir_val<T>(a.dir_scale, a.dir_scale_f, d0 + d) : T(0);
+        scmax = sc[d] > scmax ? sc[d] : scmax;
+    }
+    const T I0 = (a.wall_row && a.bundle_wall[b]) ? reinterpret_cast<const T*>(a.wall_row)[col0] : T(0);
+#pragma unroll
+    for (int d = 0; d < MAXD; ++d) I[0][d] = I0;
+    const int64_t s0 = a.seg_off[b], s1 = a.seg_off[b + 1];
+    if (s1 <= s0) return;
+    const auto row_of = [&](int64_t i) { return i < s1 ? kbase + (int64_t)a.seg_cell[i] * ldb : kbase; };   // past the end: a valid row
+    const char* r0 = row_of(s0);
+    T kc = *reinterpret_cast<const T*>(r0 + offK), jc = *reinterpret_cast<const T*>(r0 + offJ);
+    T kf = kc, jf = jc, rk[MPF], rj[MPF];
+#pragma unroll
+    for (int q = 0; q < MPF; ++q) {
+        const char* r = row_of(s0 + 1 + q);
+        rk[q] = *reinterpret_cast<const T*>(r + offK);
+        rj[q] = *reinterpret_cast<const T*>(r + offJ);
+    }
+    for (int64_t g = s0; g < s1 - 1; g += 32) {
+        const int64_t mine = g + lane;
+        __syncwarp();
+        stage[lane].row = row_of(mine + 1 + MPF);
+        stage[lane].ds = mine < s1 - 1 ? seg_len<T>(a, mine) : T(0);
+        __syncwarp();
+        const int n = s1 - 1 - g < 32 ? (int)(s1 - 1 - g) : 32;
+        for (int j = 0; j < n; ++j) {
+            const T ds = stage[j].ds;
+            const char* r = stage[j].row;
+            const T kx = rk[0], jx = rj[0];
+#pragma unroll
+            for (int q = 0; q + 1 < MPF; ++q) { rk[q] = rk[q + 1]; rj[q] = rj[q + 1]; }
+            rk[MPF - 1] = *reinterpret_cast<const T*>(r + offK);
+            rj[MPF - 1] = *reinterpret_cast<const T*>(r + offJ);
+            const T kn = T(0.5) * (kc + kx), jn = T(0.5) * (jc + jx);
+            dir_steps<T, MAXD>(I[0], kf, ds, sc, scmax, nd, jf, jn);
+            kf = kn; jf = jn; kc = kx; jc = jx;
+        }
+    }
+    // last segment: its near node is the cell's own value
+    dir_steps<T, MAXD>(I[0], kf, seg_len<T>(a, s1 - 1), sc, scmax, nd, jf, jc);
+}
+
+template <class T, int V>
+__device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int64_t d0, SegStage<T>* stage,
                                              int lane, const char* kbase, int64_t ldb, int64_t offK, int64_t offJ,
-                                             int col0, T (&I)[V][MAXD]) {
-    T sc[MAXD];
-#pragma unroll
-    for (int d = 0; d < MAXD; ++d) sc[d] = d < nd ? dir_val<T>(a.dir_scale, a.dir_scale_f, d0 + d) : T(0);
-    T scmax = T(0);
-#pragma unroll
-    for (int d = 0; d < MAXD; ++d) scmax = sc[d] > scmax ? sc[d] : scmax;
-    // one direction: its scale goes into the staged length
-    const T stage_scale = MAXD == 1 ? sc[0] : T(1);
+                                             int col0, T (&I)[V][1]) {
+    // the direction's scale goes into the staged length
+    const T stage_scale = dir_val<T>(a.dir_scale, a.dir_scale_f, d0);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         const T I0 = (a.wall_row && a.bundle_wall[b]) ? reinterpret_cast<const T*>(a.wall_row)[col0 + 32 * v] : T(0);
-#pragma unroll
-        for (int d = 0; d < MAXD; ++d) I[v][d] = I0;
+        I[v][0] = I0;
     }
     const int64_t s0 = a.seg_off[b], s1 = a.seg_off[b + 1];
     if (s1 <= s0) return;
@@ -415,8 +470,7 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
                 jx[v] = *reinterpret_cast<const T*>(r0 + offJ + 32 * v * sizeof(T));
             }
         }
-        constexpr int U = MAXD == 1 ? kUnroll : 1;   // bundles of many directions: registers go to I
-#pragma unroll U
+#pragma unroll kUnroll
         for (int j = 0; j < n; ++j) {
             const T ds = stage[j].ds;
             const char* rn = stage[j + 1].row;
@@ -432,11 +486,11 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
                 kn[v] = T(0.5) * (kc[v] + kx[v]);
                 jn[v] = T(0.5) * (jc[v] + jx[v]);
             }
-            if constexpr (V == 2 && MAXD == 1 && sizeof(T) == 4) {
+            if constexpr (V == 2 && sizeof(T) == 4) {
                 seg_step2(I[0][0], I[1][0], kf[0], kf[1], ds, ds, jf[0], jf[1], jn[0], jn[1]);
             } else {
 #pragma unroll
-                for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, scmax, nd, jf[v], jn[v]);
+                for (int v = 0; v < V; ++v) seg_step(I[v][0], kf[v], ds, jf[v], jn[v]);
             }
 #pragma unroll
             for (int v = 0; v < V; ++v) {
@@ -448,11 +502,11 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
     }
     {   // last segment: its near node is the cell's own value
         const T ds = seg_len<T>(a, s1 - 1) * stage_scale;
-        if constexpr (V == 2 && MAXD == 1 && sizeof(T) == 4) {
+        if constexpr (V == 2 && sizeof(T) == 4) {
             seg_step2(I[0][0], I[1][0], kf[0], kf[1], ds, ds, jf[0], jf[1], jc[0], jc[1]);
         } else {
 #pragma unroll
-            for (int v = 0; v < V; ++v) dir_steps<T, MAXD>(I[v], kf[v], ds, sc, scmax, nd, jf[v], jc[v]);
+            for (int v = 0; v < V; ++v) seg_step(I[v][0], kf[v], ds, jf[v], jc[v]);
         }
     }
 }
@@ -483,17 +537,28 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
 #ifndef RAPRAL_MARCH_MINB
 #define RAPRAL_MARCH_MINB 4
 #endif
-#ifndef RAPRAL_MARCH_MINB17
-#define RAPRAL_MARCH_MINB17 3
-#endif
+// Warps a block: eight where they share a point's bundles; one for the slab,
+// whose warps are independent and all take the same time, so that the last
+// wave is spread over the chip.  FP32 slab, 200 cells x 17 directions x 262,144
+// columns: blocks of 8 warps 669 us, 2 warps 632, 1 warp 619 at 24 resident
+// warps an SM, 578 at 32 (28: 589, 40: 582); FP64, 61 cells x 25 directions x
+// 100,001: 5.94, 5.74 and 5.58 ms.
+constexpr int march_warps(int MAXD, int SL) { return SL == 1 && MAXD > 1 ? 1 : 8; }
+// Resident blocks asked of the compiler.
+template <class T>
+constexpr int march_minb(int V, int MAXD, int SL) {
+    return MAXD == 1 ? (sizeof(T) == 4 && V > 1 ? RAPRAL_MARCH_MINB : 1)
+           : MAXD > 17 ? 1
+           : SL > 1 ? (sizeof(T) == 4 ? 3 : 1)
+                    : (sizeof(T) == 4 ? 32 : 12);
+}
 template <class T, int V, int MAXD, int SL, bool NODES = false>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ? RAPRAL_MARCH_MINB
-                                       : (sizeof(T) == 4 && MAXD == 17) ? RAPRAL_MARCH_MINB17
-                                                                        : 1)
+__global__ void __launch_bounds__(32 * march_warps(MAXD, SL), march_minb<T>(V, MAXD, SL))
     k_march(MarchArgs a, int lgG, T* __restrict__ part) {
     static_assert(!NODES || MAXD == 1, "node-valued rays have one direction a bundle");
+    static_assert(MAXD == 1 || V == 1, "bundles of several directions take one column a lane");
     if (*a.status) return;
-    constexpr int W = 8, CW = W / SL, TW = CW * 32 * V;
+    constexpr int W = march_warps(MAXD, SL), CW = W / SL, TW = CW * 32 * V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slice = warp / CW, cgrp = warp % CW;
     // columns fit in int: nk <= 32 x 65535 (checked by the caller)
@@ -529,7 +594,8 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ?
             march_nodes<T, V>(a, b, dir_val<T>(a.dir_scale, a.dir_scale_f, d0), stage, lane, kbase, ldb, offK, offJ,
                               I);
         } else {
-            march_bundle<T, V, MAXD>(a, b, d0, nd, stage, lane, kbase, ldb, offK, offJ, col0, I);
+            if constexpr (MAXD == 1) march_bundle<T, V>(a, b, d0, stage, lane, kbase, ldb, offK, offJ, col0, I);
+            else march_multi<T, MAXD>(a, b, d0, nd, stage, lane, kbase, ldb, offK, offJ, col0, I);
         }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -555,7 +621,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ?
     for (int v = 0; v < V; ++v) red[slice][cgrp * 32 * V + lane + 32 * v] = acc[v];
     __syncthreads();
     T* dst = (lgG == 0 ? reinterpret_cast<T*>(a.q_lambda) : part) + (int64_t)blockIdx.x * a.nk;
-    for (int i = threadIdx.x; i < TW; i += 256) {
+    for (int i = threadIdx.x; i < TW; i += blockDim.x) {
         const int kk = base + i;
         if (kk < tile0 || kk >= nk) continue;
         T s = red[0][i];
@@ -579,7 +645,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ?
 //    removes the averaging multiplies;
 //  * the step (m1_step) carries minus the intensity and minus the half length
 //    and takes the series as long as the depth needs;
-//  * equal rays of a point are marched once (k_ray_pairs);
+//  * equal rays of a point are marched once (k_ray_match, k_ray_verify);
 //  * the staged list holds, for step j, the segment's halved length (as the
 //    packed pair the step multiplies by) and the byte offset of the row of the
 //    cell PF steps ahead (row x ld, computed once by the staging lane), so a
@@ -590,8 +656,6 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && MAXD == 1 && V > 1)  ?
 //    (k_march_plan), so the warps finish together at the block's reduction.
 // Every slice still Kahan-sums its bundles in a fixed order and the slices
 // and groups are added in fixed order: results do not depend on timing.
-// Conditions (checked by the launcher): kappa, emis and the wall row 8-byte
-// aligned, ld and nk even, nk >= 64.
 
 #ifndef RAPRAL_M1_PF
 #define RAPRAL_M1_PF 2
@@ -705,29 +769,24 @@ __global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t B, unsign
     }
 }
 
-// Per point: partner[b] of every marched bundle (the equal bundle marched with
-// it, -1: none), and the marched bundles in index order (uniq, from the
-// point's first bundle) with their number (n_uniq).  A bundle of a key's odd
-// rank is the partner of the one before it, if the two are equal.
-__global__ void __launch_bounds__(512) k_ray_pairs(MarchArgs a, const unsigned long long* __restrict__ key,
-                                                   int32_t* __restrict__ partner, int32_t* __restrict__ uniq,
-                                                   int32_t* __restrict__ n_uniq) {
+// cand[b]: the earlier bundle of the point that bundle b may be the partner of
+// (a key's odd ranks go to the one before them), -1 for the others; partner[]
+// cleared.  One block a point, four lanes a bundle.
+__global__ void __launch_bounds__(512) k_ray_match(MarchArgs a, const unsigned long long* __restrict__ key,
+                                                   int32_t* __restrict__ cand, int32_t* __restrict__ partner) {
     if (*a.status) return;
     __shared__ unsigned long long ks[M1_PAIR_MAX];
-    __shared__ int16_t first[M1_PAIR_MAX];   // the bundle this one is a partner of, or -1
     const int64_t pb0 = a.point_off[blockIdx.x];
     const int64_t nb = a.point_off[blockIdx.x + 1] - pb0;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) partner[pb0 + k] = -1;
-    if (nb > M1_PAIR_MAX) {
-        for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) uniq[pb0 + k] = (int32_t)(pb0 + k);
-        if (threadIdx.x == 0) n_uniq[blockIdx.x] = (int32_t)nb;
-        return;
+    for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) {
+        partner[pb0 + k] = -1;
+        if (nb > M1_PAIR_MAX) cand[pb0 + k] = -1;
     }
+    if (nb > M1_PAIR_MAX) return;
     const int n = (int)nb;
     for (int k = threadIdx.x; k < n; k += blockDim.x) ks[k] = key[pb0 + k];
     __syncthreads();
-    for (int kb = 0; kb < n; kb += blockDim.x / 4) {   // four lanes a bundle, every fourth earlier one each
+    for (int kb = 0; kb < n; kb += blockDim.x / 4) {
         const int k = kb + (int)(threadIdx.x >> 2);
         const unsigned long long x = k < n ? ks[k] : 0ULL;
         int rank = 0, prev = -1;
@@ -738,37 +797,32 @@ __global__ void __launch_bounds__(512) k_ray_pairs(MarchArgs a, const unsigned l
         prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, 1));
         rank += __shfl_xor_sync(0xffffffffu, rank, 2);
         prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, 2));
-        if (k < n && (threadIdx.x & 3) == 0) first[k] = (int16_t)((rank & 1) ? prev : -1);
+        if (k < n && (threadIdx.x & 3) == 0) cand[pb0 + k] = (rank & 1) ? (int32_t)(pb0 + prev) : -1;
     }
-    __syncthreads();
-    for (int k = warp; k < n; k += blockDim.x >> 5) {   // the full comparison, a warp a candidate
-        const int q = first[k];
-        if (q < 0) continue;
-        const int64_t x0 = a.seg_off[pb0 + q], y0 = a.seg_off[pb0 + k];
-        const int64_t m = a.seg_off[pb0 + q + 1] - x0;
-        const int64_t dx = a.dir_off[pb0 + q], dy = a.dir_off[pb0 + k];
-        bool eq = m == a.seg_off[pb0 + k + 1] - y0 &&
-                  __float_as_uint(a.dir_scale_f[dx]) == __float_as_uint(a.dir_scale_f[dy]) &&
-                  (a.bundle_wall[pb0 + q] != 0) == (a.bundle_wall[pb0 + k] != 0);
-        for (int64_t i = lane; eq && i < m; i += 32)
-            eq = a.seg_cell[x0 + i] == a.seg_cell[y0 + i] &&
-                 __float_as_uint(a.seg_ds_f[x0 + i]) == __float_as_uint(a.seg_ds_f[y0 + i]);
-        eq = __all_sync(0xffffffffu, eq);
-        if (lane == 0) {
-            if (eq) partner[pb0 + q] = (int32_t)(pb0 + k);
-            else first[k] = -1;
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-        int out = 0;
-        for (int k0 = 0; k0 < n; k0 += 32) {
-            const bool keep = k0 + lane < n && first[k0 + lane] < 0;
-            const unsigned mk = __ballot_sync(0xffffffffu, keep);
-            if (keep) uniq[pb0 + out + __popc(mk & ((1u << lane) - 1u))] = (int32_t)(pb0 + k0 + lane);
-            out += __popc(mk);
-        }
-        if (lane == 0) n_uniq[blockIdx.x] = out;
+}
+
+// The full comparison, a warp a candidate: equal bundles become partners, the
+// others march on their own (cand back to -1).
+__global__ void __launch_bounds__(256) k_ray_verify(MarchArgs a, int64_t B, int32_t* __restrict__ cand,
+                                                    int32_t* __restrict__ partner) {
+    if (*a.status) return;
+    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (k >= B) return;
+    const int64_t q = cand[k];
+    if (q < 0) return;
+    const int64_t x0 = a.seg_off[q], y0 = a.seg_off[k], m = a.seg_off[q + 1] - x0;
+    const int64_t dx = a.dir_off[q], dy = a.dir_off[k];
+    bool eq = m == a.seg_off[k + 1] - y0 &&
+              __float_as_uint(a.dir_scale_f[dx]) == __float_as_uint(a.dir_scale_f[dy]) &&
+              (a.bundle_wall[q] != 0) == (a.bundle_wall[k] != 0);
+    for (int64_t i = lane; eq && i < m; i += 32)
+        eq = a.seg_cell[x0 + i] == a.seg_cell[y0 + i] &&
+             __float_as_uint(a.seg_ds_f[x0 + i]) == __float_as_uint(a.seg_ds_f[y0 + i]);
+    eq = __all_sync(0xffffffffu, eq);
+    if (lane == 0) {
+        if (eq) partner[q] = (int32_t)k;
+        else cand[k] = -1;
     }
 }
 
@@ -782,15 +836,34 @@ __global__ void __launch_bounds__(512) k_ray_pairs(MarchArgs a, const unsigned l
 // more than 1024 bundles are dealt round-robin in index order.
 __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ point_off,
                                                     const int64_t* __restrict__ seg_off,
-                                                    const int32_t* __restrict__ uniq,
-                                                    const int32_t* __restrict__ n_uniq, int G,
+                                                    const int32_t* __restrict__ cand, int G,
                                                     int32_t* __restrict__ plan, int32_t* __restrict__ soff,
                                                     const int* status) {
     if (*status) return;
     const int64_t p = blockIdx.x / G;
     const int g = (int)(blockIdx.x % G);
     const int64_t pb0 = point_off[p];
-    const int64_t nb = n_uniq[p];
+    int64_t nb = point_off[p + 1] - pb0;
+    // the point's marched bundles (those that are no one's partner), in index order
+    __shared__ int16_t us[M1_PAIR_MAX];
+    __shared__ int nu;
+    const bool all = nb > M1_PAIR_MAX;
+    if (!all) {
+        if (threadIdx.x < 32) {
+            const int lane = threadIdx.x, n = (int)nb;
+            int out = 0;
+            for (int k0 = 0; k0 < n; k0 += 32) {
+                const bool keep = k0 + lane < n && cand[pb0 + k0 + lane] < 0;
+                const unsigned mk = __ballot_sync(0xffffffffu, keep);
+                if (keep) us[out + __popc(mk & ((1u << lane) - 1u))] = (int16_t)(k0 + lane);
+                out += __popc(mk);
+            }
+            if (lane == 0) nu = out;
+        }
+        __syncthreads();
+        nb = nu;
+    }
+    const auto uniq = [&](int64_t i) { return (int32_t)(all ? i : pb0 + us[i - pb0]); };
     const int64_t m = nb > g ? (nb - g + G - 1) / G : 0;                     // bundles of this group
     const int64_t base = pb0 + (int64_t)g * (nb / G) + (g < nb % G ? g : nb % G);   // the group's first entry
     int32_t* so = soff + blockIdx.x * (M1_SLICES + 1);
@@ -803,7 +876,7 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
             const int s = (int)(k % M1_SLICES);
             const int64_t per = m / M1_SLICES, extra = m % M1_SLICES;
             const int64_t start = s * per + (s < extra ? s : extra);
-            plan[base + start + k / M1_SLICES] = uniq[base + k];
+            plan[base + start + k / M1_SLICES] = uniq(base + k);
         }
         if (threadIdx.x <= M1_SLICES) {
             const int s = threadIdx.x;
@@ -814,7 +887,7 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
     }
     const int mm = (int)m;
     for (int k = threadIdx.x; k < mm; k += blockDim.x) {
-        const int64_t b = uniq[base + k];
+        const int64_t b = uniq(base + k);
         len[k] = seg_off[b + 1] - seg_off[b];
     }
     __syncthreads();
@@ -845,7 +918,7 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
         for (int s = 0; s < M1_SLICES; ++s) fill[s] = cnt[s];
         for (int r = 0; r < mm; ++r) {
             const int k = order[r];
-            plan[base + fill[slice_of[k]]++] = uniq[base + k];
+            plan[base + fill[slice_of[k]]++] = uniq(base + k);
         }
     }
 }
@@ -1064,7 +1137,7 @@ __global__ void k_group_sum(const T* __restrict__ part, int G, int64_t P, int64_
 // warp per point adds the slices, each lane a strided part in order.  Weights
 // other than 1 (the grid's ends) are applied to their points, the spacing once
 // at the end: five FP64 operations a point.
-constexpr int FLUX_SPAN = 2048;
+constexpr int FLUX_SPAN = 1024;
 
 // (s, c) += x, Neumaier; magnitudes are compared by their bits
 __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
@@ -1076,7 +1149,7 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
 }
 
 template <class T>
-__global__ void __launch_bounds__(256) k_wall_flux_part(const T* __restrict__ qlam, int64_t nk, int64_t k0,
+__global__ void __launch_bounds__(128) k_wall_flux_part(const T* __restrict__ qlam, int64_t nk, int64_t k0,
                                                         int64_t n, double* __restrict__ part,
                                                         const int* status) {
     if (*status) return;
@@ -1089,14 +1162,14 @@ __global__ void __launch_bounds__(256) k_wall_flux_part(const T* __restrict__ ql
         if (kg == 0 || kg == n - 1) x *= 0.5;
         neumaier_add(s, c, x);
     }
-    __shared__ double red[8];
+    __shared__ double red[4];
     double v = s + c;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) v += red[w];
+        for (int w = 1; w < 4; ++w) v += red[w];
         part[p * gridDim.y + blockIdx.y] = v;
     }
 }
@@ -1192,7 +1265,7 @@ __global__ void k_axisym_fill(const double* xf, int32_t nx, const double* rf, in
 
 template <class T, int V, int MAXD, int SL, bool NODES = false>
 cudaError_t march_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, int G, void* part) {
-    constexpr int TW = (8 / SL) * 32 * V;
+    constexpr int W = march_warps(MAXD, SL), TW = (W / SL) * 32 * V;
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
     MarchArgs b = a;
@@ -1204,7 +1277,7 @@ cudaError_t march_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t
         b.wall_row = row;
     }
     dim3 g((unsigned)(P << lgG), div_up(nk, TW));
-    k_march<T, V, MAXD, SL, NODES><<<g, 256, 0, ctx->stream>>>(b, lgG, reinterpret_cast<T*>(part));
+    k_march<T, V, MAXD, SL, NODES><<<g, 32 * W, 0, ctx->stream>>>(b, lgG, reinterpret_cast<T*>(part));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || G == 1) return e;
     k_group_sum<T><<<(unsigned)std::min<int64_t>(div_up(P * nk, 256), 152 * 16), 256, 0, ctx->stream>>>(
@@ -1233,8 +1306,7 @@ static bool march1_vec(const MarchArgs& a, int64_t nk, const void* part, int NP)
 // The march's plan: the equal rays and the slices of every (point, group).
 struct M1Plan {
     unsigned long long* key;   // [n_bundles]
-    int32_t *partner, *uniq, *plan;   // [n_bundles]
-    int32_t* n_uniq;           // [n_points]
+    int32_t *partner, *cand, *plan;   // [n_bundles]
     int32_t* soff;             // [n_points G (M1_SLICES + 1)]
 };
 
@@ -1243,9 +1315,10 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
     if (B > 0) k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.key);
-    k_ray_pairs<<<(unsigned)P, 512, 0, ctx->stream>>>(a, pl.key, pl.partner, pl.uniq, pl.n_uniq);
-    k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, pl.uniq, pl.n_uniq, G, pl.plan,
-                                                             pl.soff, a.status);
+    k_ray_match<<<(unsigned)P, 512, 0, ctx->stream>>>(a, pl.key, pl.cand, pl.partner);
+    if (B > 0) k_ray_verify<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.cand, pl.partner);
+    k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, pl.cand, G, pl.plan, pl.soff,
+                                                             a.status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     MarchArgs b = a;
@@ -1328,7 +1401,6 @@ static size_t march_copy_bytes(const rapral_rays* r) {
 }
 static size_t march_plan_bytes(const rapral_rays* r) {
     return round256((size_t)r->n_bundles * 8) + 3 * round256((size_t)r->n_bundles * 4) +
-           round256((size_t)r->n_points * 4) +
            round256((size_t)r->n_points * march_groups(r) * (M1_SLICES + 1) * 4);
 }
 
@@ -1379,9 +1451,8 @@ cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kapp
     const auto take = [&at](size_t bytes) { char* p = at; at += round256(bytes); return p; };
     pl.key = reinterpret_cast<unsigned long long*>(take((size_t)r->n_bundles * 8));
     pl.partner = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
-    pl.uniq = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
+    pl.cand = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
     pl.plan = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
-    pl.n_uniq = reinterpret_cast<int32_t*>(take((size_t)r->n_points * 4));
     pl.soff = reinterpret_cast<int32_t*>(take((size_t)r->n_points * G * (M1_SLICES + 1) * 4));
     if (march1_applies(a, r->max_dirs, r->max_bundles_per_point, r->node_values != 0))
         return march1_launch(ctx, a, r->n_points, r->n_bundles, nk, G, part, pl);
@@ -1399,10 +1470,10 @@ cudaError_t launch_wall_flux(rapral_ctx* ctx, const void* q_lambda, int precisio
     double* part = reinterpret_cast<double*>(partials);
     dim3 grid((unsigned)n_points, (unsigned)np);
     if (precision == RAPRAL_FP64)
-        k_wall_flux_part<double><<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const double*>(q_lambda), nk, k0,
+        k_wall_flux_part<double><<<grid, 128, 0, ctx->stream>>>(reinterpret_cast<const double*>(q_lambda), nk, k0,
                                                                 g->n, part, ctx->d_status);
     else
-        k_wall_flux_part<float><<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const float*>(q_lambda), nk, k0,
+        k_wall_flux_part<float><<<grid, 128, 0, ctx->stream>>>(reinterpret_cast<const float*>(q_lambda), nk, k0,
                                                                g->n, part, ctx->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
