@@ -88,12 +88,14 @@ __device__ __forceinline__ double expfix_double(uint64_t v, int n) {
 // log2(e) 2^63
 constexpr uint64_t EXPFIX_LOG2E = 0xb8aa3b295c17f0bcull;
 
+// out of line: the rare path's FP64 operations stay out of the callers' loops
+static __device__ __noinline__ double expfix_slow(double x) { return exp(x); }
 // e^x for any x: the fixed-point form for |x| < 690, exp(x) otherwise.
 __device__ __forceinline__ double exp_fix(double x, const uint64_t* tab) {
     const uint64_t bits = (uint64_t)__double_as_longlong(x);
     const int ex = (int)(bits >> 52) & 0x7ff;
     const int hi = __double2hiint(x) & 0x7fffffff;
-    if (hi >= 0x40859000) return exp(x);   // |x| >= 690, inf or NaN
+    if (hi >= 0x40859000) return expfix_slow(x);   // |x| >= 690, inf or NaN
     const uint64_t B = ((bits << 11) | (uint64_t(1) << 63));   // |x| = B 2^(ex - 1086)
     const uint64_t P = __umul64hi(B, EXPFIX_LOG2E);            // |x| log2(e) = P 2^(ex - 1085)
     const int sh = 1032 - ex;                                   // to 53 fraction bits; > 0 for |x| < 2^9.. 690
@@ -136,12 +138,15 @@ __device__ __forceinline__ ExpFixScale expfix_scale(double b) {
     r.F = 44 + s;
     return r;
 }
+// (out of line, so that its product is not formed ahead of the test: an FP64
+// operation a term)
+static __device__ __noinline__ double expfix_far(double E, double b) { return exp(-b * E); }
 // e^{-b E}: Ef from expfix_energy(E), sc from expfix_scale(b)
 __device__ __forceinline__ double expfix_boltzmann(uint64_t Ef, const ExpFixScale& sc, double E, double b,
                                                    const uint64_t* tab) {
     const uint64_t P = __umul64hi(Ef, sc.m);
     const int n = (int)(P >> sc.F);
-    if (sc.F == 0 || Ef == EXPFIX_BAD || n > 1000 || (P >> sc.F) > 1000) return exp(-b * E);
+    if (sc.F == 0 || Ef == EXPFIX_BAD || (P >> sc.F) > 1000) return expfix_far(E, b);
     return expfix_double(expfix_frac(P << (64 - sc.F), tab), n);
 }
 

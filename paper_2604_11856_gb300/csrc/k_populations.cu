@@ -40,7 +40,7 @@ __global__ void k_validate_cells(const double* Ttr, const double* Tve, const dou
 // the rotational ladders (diatomics).  What a term costs is its exponential;
 // with expfix_boltzmann it is 95 integer operations and one FP64 multiply-add
 // beside them (exp(double) kept the FP64 pipe busy at 21 operation times a
-// term: 5000 cells, 53,000 terms a cell, 9.7 -> 1.2 ms).  A level is read and
+// term: 5000 cells, 53,000 terms a cell, 9.7 -> 0.96 ms).  A level is read and
 // turned into fixed point once for its CC cells.
 // The order of a cell's sum does not depend on CC.
 template <int CC>
@@ -57,16 +57,21 @@ __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const do
     const int64_t c0 = (int64_t)blockIdx.x * CC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (s == 0 && tid < CC && c0 + tid < C) check_cell(Ttr, Tve, n, c0 + tid, ncol, status);
+    __shared__ double sb[2][CC];       // c2 / T_ve, c2 / T_tr: a division a block and cell, not one a thread
+    if (tid < 2 * CC) {
+        const int q = tid >> 1;
+        const int64_t c = c0 + q < C ? c0 + q : C - 1;
+        sb[tid & 1][q] = c2 / ((tid & 1) ? Ttr : Tve)[c];
+    }
+    __syncthreads();
     double bve[CC], btr[CC], z[CC];
     ExpFixScale sc[CC];
 #pragma unroll
     for (int q = 0; q < CC; ++q) {
-        const int64_t c = c0 + q < C ? c0 + q : C - 1;
-        bve[q] = c2 / Tve[c];
-        btr[q] = c2 / Ttr[c];
+        bve[q] = sb[0][q];
+        btr[q] = sb[1][q];
         z[q] = 0.0;
     }
-    __syncthreads();
     if (sp.kind[s] == RAPRAL_ATOM) {
         const int64_t b = sp.atom_off[s + 1];
 #pragma unroll
@@ -90,8 +95,7 @@ __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const do
                 __syncthreads();
                 for (int x = tid; x < CC * nvc; x += 256) {   // a (cell, level) a thread
                     const int q = x / nvc, v = x - q * nvc;
-                    const int64_t c = c0 + q < C ? c0 + q : C - 1;
-                    const double b = c2 / Tve[c];
+                    const double b = sb[0][q];
                     pv[q][v] = sp.st_g[i] * exp_fix(-b * sp.st_E[i], tab) / sp.st_sigma[i] *
                                exp_fix(-b * vib[v0 + v], tab);
                 }
