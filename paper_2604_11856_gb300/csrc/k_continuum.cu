@@ -171,8 +171,23 @@ __device__ __forceinline__ double cont_sigma_walk(const double* x, const double*
     return slope * (lam - x[j]) + y[j];
 }
 
-// one warp per (tile, level): a binary search for the lane's first point,
-// then a forward walk over its later points
+// The last of the nodes x[a, b) at or below lam (or a), by one warp, 32 probes
+// a round: 120 nodes take two rounds of loads where a bisection takes seven.
+__device__ __forceinline__ int64_t node_below(const double* x, int64_t a, int64_t b, double lam) {
+    const int lane = threadIdx.x & 31;
+    int64_t lo = a, hi = b;   // x[lo - 1] <= lam < x[hi]
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) / 32, p = lo + lane * step;
+        const int c = __popc(__ballot_sync(0xffffffffu, p < hi && pos_le(x[p < hi ? p : lo], lam)));
+        if (c == 0) break;
+        hi = min(hi, lo + c * step);
+        lo += (c - 1) * step + 1;
+    }
+    return lo > a ? lo - 1 : a;
+}
+
+// one warp per (tile, level): a search for the tile's first point, then a
+// forward walk over the lane's points (a tile spans few nodes)
 template <typename Tp>
 __global__ void __launch_bounds__(128) k_cont_sigma(ContModels M, const ContLevel* lev, const int* n_lev,
                                                      const int64_t* tab_off, int W, double lam_min, double h,
@@ -188,14 +203,7 @@ __global__ void __launch_bounds__(128) k_cont_sigma(ContModels M, const ContLeve
         const int64_t a = m.node_off[L.i], b = m.node_off[L.i + 1] - 1;
         const double* x = m.node_lam;
         const double* y = m.node_sigma;
-        const double lam_first = grid_lam(lam_min, h, k0 + t * W + lane);
-        int64_t lo = a, hi = b;   // last node <= lam_first (or a)
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (pos_le(x[mid], lam_first)) lo = mid;
-            else hi = mid;
-        }
-        int64_t j = lo;
+        int64_t j = node_below(x, a, b, grid_lam(lam_min, h, k0 + t * W));
         for (int p = lane; p < W; p += 32) {
             const int64_t k = t * W + p;
             double sg = 0.0;
@@ -248,15 +256,7 @@ __global__ void __launch_bounds__(128) k_cont_sigma32(ContModels M, const ContLe
         const double* x = m.node_lam;
         const int64_t nb = M.node0[L.m];
         const int64_t klo = L.klo, khi = L.khi;
-        // the lane's first point: last node <= its wavelength (or a)
-        const double lam_first = grid_lam(lam_min, h, kt + lane);
-        int64_t lo = a, hi = b;
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (pos_le(x[mid], lam_first)) lo = mid;
-            else hi = mid;
-        }
-        int64_t j = lo;
+        int64_t j = node_below(x, a, b, lam_t);   // last node <= the tile's first wavelength (or a)
         float base = (float)(lam_t - x[j]);
         for (int p = lane; p < W; p += 32) {
             const int64_t k = kt + p;
