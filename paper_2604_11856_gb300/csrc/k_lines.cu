@@ -447,14 +447,14 @@ __device__ __forceinline__ double widen(float x) {
 }
 // u^(1/4) for u in [2^-60, 2^60]: w = u^(-1/4) to FP32 accuracy, e = 1 - u w^4
 // (below 2^-19), u^(1/4) = u w^3 (1 - e)^(-3/4) with the series through e^2
-// (e^3 < 2^-57): 8 FP64 operations, two square roots take 18 operation times.
+// (e^3 < 2^-57): 7 FP64 operations, two square roots take 18 operation times.
 __device__ __forceinline__ double root4(double u) {
     float r, wf;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(trunc_float(u)));
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(wf) : "f"(r));
-    const double w = widen(wf), w2 = w * w;
-    const double e = fma(-u, w2 * w2, 1.0);
-    const double y = u * w2 * w;
+    const double w = widen(wf), w2 = w * w, x = u * w2;
+    const double e = fma(-x, w2, 1.0);
+    const double y = x * w;
     return fma(y, e * fma(e, 0.65625, 0.75), y);
 }
 // n / d for d in [1, 2^100]: an FP32 reciprocal and one step of third order
@@ -475,10 +475,10 @@ __device__ __forceinline__ bool le_bits(double a, double b) {
 // whatever lanes are in the window: thread i owns points i, i + 128, ..., so
 // that a warp's points are runs of 32 in a row and a run outside the window
 // is skipped by the whole warp (with 128 points in a row a warp, a window of
-// 70 points kept 37 % of the lanes busy), and an evaluation is 23 FP64
+// 70 points kept 37 % of the lanes busy), and an evaluation is 22 FP64
 // operations: wavelengths formed once a tile, comparisons on the integer
 // pipe, u^2.25 and the quotient by Newton steps from FP32 seeds, exponentials
-// in fixed point.  24 cells x 50,001 points, 64,000 lines: 20.3 -> 5.2 ms.
+// in fixed point.  24 cells x 50,001 points, 64,000 lines: 20.3 -> 4.9 ms.
 template <int PPT, bool VG = false>
 __global__ void __launch_bounds__(128) k_line_sum_f64(LineSumArgs a) {
     if (*a.status) return;
@@ -1328,7 +1328,10 @@ cudaError_t launch_line_plan(rapral_ctx* ctx, const rapral_species* sp, const ra
     if (ln->n_lines == 0) return cudaSuccess;
     BroadArgs b = br ? *br : BroadArgs{};
     if (!broad_terms(br)) lb = nullptr, lb32 = nullptr;
-    k_line_plan<<<div_up(ln->n_lines, 256), 256, 0, ctx->stream>>>(
+    // a block's warps share one SM's FP64 pipe: a short list goes out a warp a
+    // block (1,500 lines: 22 us as 6 blocks of eight warps)
+    const int nt = ln->n_lines < 152 * 256 ? 32 : 256;
+    k_line_plan<<<div_up(ln->n_lines, nt), nt, 0, ctx->stream>>>(
         *ln, sp->mass, sp->kind, sp->n_species, lam_min, h, ph, plan->k0, plan->nk, plan->tile_w, d_max, out, out32,
         plan->line_tiles, plan->wmax, plan->unsorted, b, lb, lb32, ctx->d_status);
     return cudaGetLastError();
