@@ -375,12 +375,16 @@ __device__ __forceinline__ void march_nodes(const MarchArgs& a, int64_t b, T sc,
 // of 17 directions is about 150 FP32 instructions a warp.  The next MPF cells
 // are in flight, across the staging seams: entry j of the stage holds the
 // length of segment j and the row of the cell that step j + MPF needs (two,
-// three, four and six ahead take the same time).
+// three, four and six ahead take the same time).  In FP32 two steps are
+// unrolled: the ring's shift is then a renaming, where a copy of a value still
+// in flight waits for it (200 cells x 17 directions x 262,144 columns: 573 ->
+// 528 us; rings of three and four, unrolled by as many: 599 and 629).  In FP64
+// the loads are far ahead in time and the longer body costs 2 %.
 template <class T, int MAXD>
 __device__ __forceinline__ void march_multi(const MarchArgs& a, int64_t b, int64_t d0, int nd, SegStage<T>* stage,
                                             int lane, const char* kbase, int64_t ldb, int64_t offK, int64_t offJ,
                                             int col0, T (&I)[1][MAXD]) {
-    constexpr int MPF = 2;
+    constexpr int MPF = 2, UNROLL = sizeof(T) == 4 ? MPF : 1;
     T sc[MAXD], scmax = T(0);
 #pragma unroll
     for (int d = 0; d < MAXD; ++d) {
@@ -409,6 +413,7 @@ __device__ __forceinline__ void march_multi(const MarchArgs& a, int64_t b, int64
         stage[lane].ds = mine < s1 - 1 ? seg_len<T>(a, mine) : T(0);
         __syncwarp();
         const int n = s1 - 1 - g < 32 ? (int)(s1 - 1 - g) : 32;
+#pragma unroll UNROLL
         for (int j = 0; j < n; ++j) {
             const T ds = stage[j].ds;
             const char* r = stage[j].row;
