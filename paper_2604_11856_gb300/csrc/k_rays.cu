@@ -39,7 +39,8 @@ __device__ __forceinline__ float recip(float x) {
 // 2^-10, 2^-7, 2^-4, 1/2; the lanes of a warp share the tail), and |t| is
 // compared by its high word on the integer pipe.  A thin step is 8 to 20 FP64
 // operations; with an expm1 and two divisions whatever its t it took the
-// time of 75 (61 cells x 25 directions x 100,001 points: 18.8 -> 5.5 ms).
+// time of 75 (61 cells x 25 directions x 100,001 points: 18.8 -> 5.5 ms, 4.3
+// with the directions split over warps).
 constexpr int hi_2m(int k) { return (1023 - k) << 20; }   // high word of 2^-k
 constexpr int T64_1 = hi_2m(1);
 __device__ __forceinline__ int abs_hi(double t) { return __double2hiint(t) & 0x7fffffff; }
@@ -546,8 +547,7 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
 // whose warps are independent and all take the same time, so that the last
 // wave is spread over the chip.  FP32 slab, 200 cells x 17 directions x 262,144
 // columns: blocks of 8 warps 669 us, 2 warps 632, 1 warp 619 at 24 resident
-// warps an SM, 578 at 32 (28: 589, 40: 582); FP64, 61 cells x 25 directions x
-// 100,001: 5.94, 5.74 and 5.58 ms.
+// warps an SM, 578 at 32 (28: 589, 40: 582).
 constexpr int march_warps(int MAXD, int SL) { return SL == 1 && MAXD > 1 ? 1 : 8; }
 // Resident blocks asked of the compiler.
 template <class T>
@@ -557,15 +557,23 @@ constexpr int march_minb(int V, int MAXD, int SL) {
            : SL > 1 ? (sizeof(T) == 4 ? 3 : 1)
                     : (sizeof(T) == 4 ? 32 : 12);
 }
-template <class T, int V, int MAXD, int SL, bool NODES = false>
-__global__ void __launch_bounds__(32 * march_warps(MAXD, SL), march_minb<T>(V, MAXD, SL))
+// A split bundle's blocks: 30 resident warps an SM asked in FP32, 18 in FP64
+// (3 directions a warp) or 15 (7).
+template <class T>
+constexpr int march_minb_split(int MAXD, int DS) { return (sizeof(T) == 4 ? 32 : MAXD <= 3 ? 18 : 16) / DS; }
+// DS > 0: the directions of each bundle are dealt to the block's warps (at most
+// DS of them), MAXD or fewer each, all on the same 32 columns.
+template <class T, int V, int MAXD, int SL, bool NODES = false, int DS = 0>
+__global__ void __launch_bounds__(32 * (DS ? DS : march_warps(MAXD, SL)),
+                                  DS ? march_minb_split<T>(MAXD, DS) : march_minb<T>(V, MAXD, SL))
     k_march(MarchArgs a, int lgG, T* __restrict__ part) {
     static_assert(!NODES || MAXD == 1, "node-valued rays have one direction a bundle");
     static_assert(MAXD == 1 || V == 1, "bundles of several directions take one column a lane");
+    static_assert(DS == 0 || (SL == 1 && MAXD > 1), "a split of the directions has no bundle slices");
     if (*a.status) return;
-    constexpr int W = march_warps(MAXD, SL), CW = W / SL, TW = CW * 32 * V;
+    constexpr int W = DS ? DS : march_warps(MAXD, SL), CW = DS ? 1 : W / SL, TW = CW * 32 * V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int slice = warp / CW, cgrp = warp % CW;
+    const int slice = DS ? 0 : warp / CW, cgrp = DS ? 0 : warp % CW;
     // columns fit in int: nk <= 32 x 65535 (checked by the caller)
     const int nk = (int)a.nk;
     const int tile0 = (int)blockIdx.y * TW;
@@ -588,9 +596,14 @@ __global__ void __launch_bounds__(32 * march_warps(MAXD, SL), march_minb<T>(V, M
     const unsigned p = blockIdx.x >> lgG, grp = blockIdx.x & ((1u << lgG) - 1u);
     const int64_t b1 = a.point_off[p + 1];
     for (int64_t b = a.point_off[p] + (int64_t)grp * SL + slice; b < b1; b += (int64_t)SL << lgG) {
-        const int64_t d0 = a.dir_off[b];
-        const int nd = (int)(a.dir_off[b + 1] - d0);
-        if (nd == 0) continue;
+        int64_t d0 = a.dir_off[b];
+        int nd = (int)(a.dir_off[b + 1] - d0);
+        if (DS) {
+            const int q = min((nd + (int)(blockDim.x >> 5) - 1) / (int)(blockDim.x >> 5), MAXD);
+            d0 += warp * q;
+            nd = min(nd - warp * q, q);
+        }
+        if (nd <= 0) continue;
         T I[V][MAXD];
         if constexpr (NODES) {
             const bool wall = a.wall_row && a.bundle_wall[b];
@@ -621,16 +634,18 @@ __global__ void __launch_bounds__(32 * march_warps(MAXD, SL), march_minb<T>(V, M
             acc[v] = tt;
         }
     }
-    __shared__ T red[SL][TW];
+    constexpr int NR = DS ? DS : SL;
+    const int nr = DS ? (int)(blockDim.x >> 5) : SL;
+    __shared__ T red[NR][TW];
 #pragma unroll
-    for (int v = 0; v < V; ++v) red[slice][cgrp * 32 * V + lane + 32 * v] = acc[v];
+    for (int v = 0; v < V; ++v) red[DS ? warp : slice][cgrp * 32 * V + lane + 32 * v] = acc[v];
     __syncthreads();
     T* dst = (lgG == 0 ? reinterpret_cast<T*>(a.q_lambda) : part) + (int64_t)blockIdx.x * a.nk;
     for (int i = threadIdx.x; i < TW; i += blockDim.x) {
         const int kk = base + i;
         if (kk < tile0 || kk >= nk) continue;
         T s = red[0][i];
-        for (int q = 1; q < SL; ++q) s += red[q][i];
+        for (int q = 1; q < nr; ++q) s += red[q][i];
         dst[kk] = s;
     }
 }
@@ -1268,9 +1283,11 @@ __global__ void k_axisym_fill(const double* xf, int32_t nx, const double* rf, in
 #define RAPRAL_MARCH_V 2
 #endif
 
-template <class T, int V, int MAXD, int SL, bool NODES = false>
-cudaError_t march_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, int G, void* part) {
-    constexpr int W = march_warps(MAXD, SL), TW = (W / SL) * 32 * V;
+template <class T, int V, int MAXD, int SL, bool NODES = false, int DS = 0>
+cudaError_t march_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, int G, void* part,
+                         int n_split = 0) {
+    const int W = DS ? n_split : march_warps(MAXD, SL);
+    constexpr int TW = DS ? 32 * V : (march_warps(MAXD, SL) / SL) * 32 * V;
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
     MarchArgs b = a;
@@ -1282,7 +1299,7 @@ cudaError_t march_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t
         b.wall_row = row;
     }
     dim3 g((unsigned)(P << lgG), div_up(nk, TW));
-    k_march<T, V, MAXD, SL, NODES><<<g, 32 * W, 0, ctx->stream>>>(b, lgG, reinterpret_cast<T*>(part));
+    k_march<T, V, MAXD, SL, NODES, DS><<<g, 32 * W, 0, ctx->stream>>>(b, lgG, reinterpret_cast<T*>(part));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || G == 1) return e;
     k_group_sum<T><<<(unsigned)std::min<int64_t>(div_up(P * nk, 256), 152 * 16), 256, 0, ctx->stream>>>(
@@ -1374,7 +1391,25 @@ cudaError_t march_t(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, 
         return march_launch<T, 1, RAPRAL_MAX_DIRS, 8>(ctx, a, P, nk, G, part);
     }
     if (maxd <= 1) return march_launch<T, 1, 1, 1>(ctx, a, P, nk, G, part);
-    if (maxd <= 17) return march_launch<T, 1, 17, 1>(ctx, a, P, nk, G, part);
+    // A warp takes a bundle's directions one after the other, 1,400 cycles a
+    // step of 17 in FP32 however idle the chip is.  Up to 11 column tiles an SM
+    // they are split over warps of three: FP32, 200 cells x 17 directions x
+    // 5,000 / 20,000 / 45,000 / 55,000 / 65,000 columns 183 / 201 / 234 / 248 /
+    // 268 us in one warp, 76 / 105 / 160 / 237 / 301 split (five each: 104 / 127
+    // / 173 / 199 / 242; 8 directions, 100 cells, 55,000: 89, 71 split by threes,
+    // 70 by fives).  In FP64 the pipe is what bounds the march and the split
+    // keeps it fed at every size: 60 cells x 17 directions x 5,000 / 20,000 /
+    // 60,000 / 100,001 columns 1,160 / 1,405 / 2,762 / 3,240 us in one warp, 465 /
+    // 840 / 1,820 / 2,820 by threes, 680 / 1,048 / 1,864 / 2,680 by sevens, which
+    // are taken above the line.
+    if (maxd <= 17 && P * div_up(nk, 32) <= 152 * 11)
+        return march_launch<T, 1, 3, 1, false, 6>(ctx, a, P, nk, G, part, std::max(1, (int)div_up(maxd, 3)));
+    if constexpr (sizeof(T) == 8) {
+        if (maxd <= 17)
+            return march_launch<T, 1, 7, 1, false, 3>(ctx, a, P, nk, G, part, std::max(1, (int)div_up(maxd, 7)));
+    } else {
+        if (maxd <= 17) return march_launch<T, 1, 17, 1>(ctx, a, P, nk, G, part);
+    }
     return march_launch<T, 1, RAPRAL_MAX_DIRS, 1>(ctx, a, P, nk, G, part);
 }
 

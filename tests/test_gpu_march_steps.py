@@ -76,3 +76,37 @@ def test_slab_steps(precision, tol, n_mu, depth):
     ref, big = _march(tk.double().cpu().numpy(), tj.double().cpu().numpy(), dx, np.concatenate([[1.0], 1.0 / mu]))
     err = np.max(np.abs(I.double().cpu().numpy().astype(LD) - ref) / np.maximum(big, LD(1e-300)))
     assert err <= tol, float(err)
+
+
+@pytest.mark.parametrize("precision,tol", [(R.FP64, 7e-14), (R.FP32, 3.8e-5)])
+@pytest.mark.parametrize("n_mu", [1, 2, 3, 6, 13, 16, 17, 24])
+@pytest.mark.parametrize("nk", [1, 31, 33, 152 * 11 * 32, 152 * 11 * 32 + 1])
+def test_split_directions(precision, tol, n_mu, nk):
+    """The directions of a bundle in one warp or dealt to several: counts around the multiples of a warp's
+    share, ranges at and past the line between the two forms, intensities and their weighted sum."""
+    ctx = R.Context(0)
+    rng = np.random.default_rng(11)
+    C, dx, w = 12, 0.5, min(nk, 97)
+    kap = np.tile(2.0 ** rng.uniform(-20, 2, (C, w)), (1, -(-nk // w)))[:, :nk]
+    em = np.tile(2.0 ** rng.uniform(-3, 3, (C, w)), (1, -(-nk // w)))[:, :nk]
+    dt = torch.float64 if precision == R.FP64 else torch.float32
+    tk = torch.as_tensor(kap, device=ctx.device).to(dt)
+    tj = torch.as_tensor(em, device=ctx.device).to(dt)
+    mu = np.linspace(0.1, 0.9, n_mu)
+    wmu = rng.uniform(0.5, 1.5, n_mu)
+    geo = synth.SlabGeometry(cell_order=np.arange(C, dtype=np.int64), dx=np.full(C, dx), mu=mu, wmu=wmu)
+    rays = R.slab_rays(ctx, geo, ctx.device)
+    q = torch.empty((1, nk), dtype=dt, device=ctx.device)
+    I = torch.full((rays.n_dirs, nk), float("nan"), dtype=dt, device=ctx.device)
+    R.trace_rays(ctx, rays, C, tk, tj, synth.Grid(100.0, 200.0, max(nk, 2)), 0, nk, precision, q, I)
+    ctx.sync()
+    ref, big = _march(tk[:, :w].double().cpu().numpy(), tj[:, :w].double().cpu().numpy(), dx,
+                      np.concatenate([[1.0], 1.0 / mu]))
+    got = I.double().cpu().numpy()
+    reps = -(-nk // w)
+    tile = lambda x: np.tile(x.astype(float), (1, reps))[:, :nk]
+    assert np.max(np.abs(got - tile(ref)) / np.maximum(tile(big), 1e-300)) <= tol
+    weight = rays.t["dir_weight"].cpu().numpy()[:, None]
+    flux = np.abs(weight) * tile(big)
+    assert np.max(np.abs(q[0].double().cpu().numpy() - (weight * tile(ref)).sum(0)) /
+                  np.maximum(flux.sum(0), 1e-300)) <= tol
