@@ -180,25 +180,34 @@ __global__ void __launch_bounds__(256) k_cell_prep(const double* __restrict__ Tt
 }
 
 // Ground-level weight of each atomic species: the summed g of its levels at
-// E = 0 (0 for molecules).  A warp a species, lanes along its levels (one
-// thread walking 10,000 levels was a chain of load latencies: 1.2 ms).
-__global__ void k_ground_weights(rapral_species sp, double* g0) {
-    const int s = blockIdx.x, lane = threadIdx.x;
+// E = 0 (0 for molecules).  A block a species, threads along its levels: what
+// it takes is load latency (20,000 levels on two atoms, cold: one thread 1.2 ms,
+// a warp 57 us, 512 threads 10 us).
+constexpr int GROUND_THREADS = 512;
+__global__ void __launch_bounds__(GROUND_THREADS) k_ground_weights(rapral_species sp, double* g0) {
+    __shared__ double part[GROUND_THREADS / 32];
+    const int s = blockIdx.x, lane = threadIdx.x & 31;
     double g = 0.0;
     if (sp.kind[s] == RAPRAL_ATOM) {
         const int64_t b = sp.atom_off[s + 1];
 #pragma unroll 4
-        for (int64_t k = sp.atom_off[s] + lane; k < b; k += 32)
+        for (int64_t k = sp.atom_off[s] + threadIdx.x; k < b; k += GROUND_THREADS)
             if (sp.atom_E[k] == 0.0) g += sp.atom_g[k];
     }
     g = warp_sum(g);
+    if (lane == 0) part[threadIdx.x >> 5] = g;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    g = warp_sum(lane < GROUND_THREADS / 32 ? part[lane] : 0.0);
     if (lane == 0) g0[s] = g;
 }
 
 // Per (cell, atomic species): ground-level density N_0 = n_s g_0 / Z_s and
 // the van der Waals factor W = 6.65e-29 N (2T/M)^0.5 + 2.925e-29 N_o (2T/M_o)^0.5
 // (the other heavy particles in column order); zeros for molecules or for
-// terms that are off.  Largest values over the cells per species in dmax.
+// terms that are off.  Largest values over the cells per species in dmax.  A
+// thread a (cell, species): a few cells are a chain of FP64 exp, log and square
+// roots (96 cells x 8 species: 28 us with the species in turn, 11 so).
 __global__ void k_cell_broad(rapral_species sp, rapral_cells cells, BroadArgs br, const double* __restrict__ g0,
                              double2* __restrict__ cb, float2* __restrict__ cb32, unsigned long long* dmax,
                              const int* status) {
@@ -206,33 +215,30 @@ __global__ void k_cell_broad(rapral_species sp, rapral_cells cells, BroadArgs br
     __shared__ unsigned long long blk;
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool in = c < cells.n_cells;
-    const int S = sp.n_species, nc = cells.n_cols;
-    const double T = in ? cells.Ttr[c] : 1.0;
-    const double* n = cells.n + (in ? c : 0) * nc;
-    for (int s = 0; s < S; ++s) {
-        double N0 = 0.0, W = 0.0;
-        if (in && sp.kind[s] == RAPRAL_ATOM) {
-            if ((br.flags & RAPRAL_BROAD_RESONANCE) && g0[s] > 0.0)
-                N0 = exp(cells.lnpref[c * S + s] + log(g0[s]));
-            if (br.flags & RAPRAL_BROAD_VDW) {
-                const int col = sp.density_col[s];
-                double No = 0.0, NoM = 0.0;
-                for (int k = 0; k < nc && k < br.ncol; ++k) {
-                    if (k == col || !(br.colmass[k] > 0.0)) continue;
-                    No += n[k];
-                    NoM += n[k] * br.colmass[k];
-                }
-                W = 6.65e-29 * n[col] * sqrt(2.0 * T / sp.mass[s]);
-                if (No > 0.0) W += 2.925e-29 * No * sqrt(2.0 * T / (NoM / No));
+    const int S = sp.n_species, nc = cells.n_cols, s = blockIdx.y;
+    double N0 = 0.0, W = 0.0;
+    if (in && sp.kind[s] == RAPRAL_ATOM) {
+        const double* n = cells.n + c * nc;
+        if ((br.flags & RAPRAL_BROAD_RESONANCE) && g0[s] > 0.0) N0 = exp(cells.lnpref[c * S + s] + log(g0[s]));
+        if (br.flags & RAPRAL_BROAD_VDW) {
+            const double T = cells.Ttr[c];
+            const int col = sp.density_col[s];
+            double No = 0.0, NoM = 0.0;
+            for (int k = 0; k < nc && k < br.ncol; ++k) {
+                if (k == col || !(br.colmass[k] > 0.0)) continue;
+                No += n[k];
+                NoM += n[k] * br.colmass[k];
             }
+            W = 6.65e-29 * n[col] * sqrt(2.0 * T / sp.mass[s]);
+            if (No > 0.0) W += 2.925e-29 * No * sqrt(2.0 * T / (NoM / No));
         }
-        if (in) {
-            cb[c * S + s] = make_double2(N0, W);
-            cb32[c * S + s] = make_float2((float)N0, (float)W);
-        }
-        block_max((unsigned long long)__double_as_longlong(N0), &blk, &dmax[2 + 2 * s]);
-        block_max((unsigned long long)__double_as_longlong(W), &blk, &dmax[3 + 2 * s]);
     }
+    if (in) {
+        cb[c * S + s] = make_double2(N0, W);
+        cb32[c * S + s] = make_float2((float)N0, (float)W);
+    }
+    block_max((unsigned long long)__double_as_longlong(N0), &blk, &dmax[2 + 2 * s]);
+    block_max((unsigned long long)__double_as_longlong(W), &blk, &dmax[3 + 2 * s]);
 }
 
 }  // namespace
@@ -240,10 +246,10 @@ __global__ void k_cell_broad(rapral_species sp, rapral_cells cells, BroadArgs br
 cudaError_t launch_broad_cells(rapral_ctx* ctx, const rapral_species* sp, const rapral_cells* cells,
                                const BroadArgs& br, double* g0, double2* cb, float2* cb32, unsigned long long* d_max) {
     const int S = sp->n_species;
-    k_ground_weights<<<S, 32, 0, ctx->stream>>>(*sp, g0);   // d_max was cleared by launch_plan_reset
+    k_ground_weights<<<S, GROUND_THREADS, 0, ctx->stream>>>(*sp, g0);   // d_max was cleared by launch_plan_reset
     if (cells->n_cells == 0) return cudaGetLastError();
-    k_cell_broad<<<div_up(cells->n_cells, 128), 128, 0, ctx->stream>>>(*sp, *cells, br, g0, cb, cb32, d_max,
-                                                                       ctx->d_status);
+    k_cell_broad<<<dim3(div_up(cells->n_cells, 128), (unsigned)S), 128, 0, ctx->stream>>>(*sp, *cells, br, g0, cb,
+                                                                                          cb32, d_max, ctx->d_status);
     return cudaGetLastError();
 }
 
