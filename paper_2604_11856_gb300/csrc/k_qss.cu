@@ -1,21 +1,22 @@
 // Quasi-steady-state collisional-radiative populations (Sec. 2.1): per cell
 // and atomic radiator, the rate matrix R and source b of the QSS master
 // equation, solved by LU with partial pivoting.  One warp per cell: lanes
-// compute the transitions' up / down rates into shared memory, lane r
-// assembles row r from its own transitions (losses on the diagonal, gains off
-// it, in transition order), pivots and eliminates its row, and the warp
-// substitutes back column by column.  FP64 throughout: the systems span many
-// orders of magnitude in their rates.
+// compute the transitions' up / down rates and store them in the rows that gain
+// by them (added in order where a pair of levels has several transitions);
+// lane r sums column r, what its level loses, for the diagonal, pivots and
+// eliminates its row, and the warp substitutes back column by column.  FP64
+// throughout: the systems span many orders of magnitude in their rates.
 //
 // The FP64 pipe bounds it (a warp instruction of it takes 17 clocks of an SM,
-// whatever lanes are on), so the count of FP64 warp instructions a cell is
-// what the layout keeps down: rows are assembled from per-row lists, built
-// once a block (two instructions a row entry instead of four a transition
-// with two lanes on, 1,984 for 496 transitions), exponentials and pivot
-// comparisons run on the integer pipe, divisions are one Newton reciprocal a
-// level or pivot, and the back substitution is one instruction a column
-// instead of one lane's 496.  20,000 cells of 32 + 4 levels, 496 transitions:
-// 6.57 -> 2.25 ms.
+// whatever lanes are on; by count it is busy 75 % of the time), so the count
+// of FP64 warp instructions a cell is what the layout keeps down: 32 sums for
+// the diagonals of 32 rows (from lists of each row's transitions two a list
+// entry, by transitions four with two lanes on, 1,984 for 496), exponentials
+// and pivot comparisons on the integer pipe, divisions one Newton reciprocal a
+// level or pivot, back substitution one instruction a column instead of one
+// lane's 496.  The rates need no store of their own, so 16 warps an SM fit
+// (eight with one).  20,000 cells of 32 + 4 levels, 496 transitions: 6.57 ->
+// 2.25 ms, then 2.09 without the lists and the rates' store.
 #include <algorithm>
 
 #include "rapral_internal.cuh"
@@ -23,7 +24,7 @@
 
 namespace {
 
-constexpr int QW = 2;          // warps (cells) per block
+constexpr int QW = 4;          // warps (cells) per block
 constexpr int QMAXL = 32;      // levels solved
 constexpr int QMAXT = QMAXL * (QMAXL - 1) / 2;
 constexpr double N_AVOGADRO = 6.022e23;
@@ -51,19 +52,21 @@ __device__ __forceinline__ double recip64(double x) {
     return fma(y, fma(e, e, e), y);
 }
 
-__global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells cells, Phys ph, double* n_out,
-                                                 int* status) {
+__global__ void __launch_bounds__(32 * QW, 4)
+    k_qss(rapral_cr_model m, rapral_cells cells, Phys ph, double* n_out, int* status) {
     if (*status) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     __shared__ uint64_t tab[EXPFIX_N];
     __shared__ double Rs[QW][QMAXL][QMAXL + 1];
     __shared__ double bs[QW][QMAXL];
-    __shared__ double rate_up[QW][QMAXT], rate_dn[QW][QMAXT];
     __shared__ double Qh[QW][QMAXL], Qv[QW][QMAXL], iQh[QW][QMAXL], iQv[QW][QMAXL];
     __shared__ unsigned char slo[QMAXT], sup[QMAXT];
-    __shared__ unsigned short ent[2 * QMAXT], roff[QMAXL + 1];   // row r: ent[roff[r]] .. (transition, 1 << 15 if r is upper)
+    __shared__ unsigned pairs[QMAXL], twice;   // level i: a bit per j > i with a transition; any pair has several
     const int l = m.n_levels, T = m.n_trans, nc = cells.n_cols;
     expfix_load(tab);
+    if (threadIdx.x < QMAXL) pairs[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) twice = 0u;
+    __syncthreads();
     // every transition is checked before any indexed use
     bool bad = false;
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
@@ -77,27 +80,12 @@ __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells
         sup[t] = (unsigned char)j;
     }
     if (__syncthreads_or(bad)) return;
-    if (w == 0) {   // the rows' lists, in transition order
-        int n = 0;
-        for (int t = 0; t < T; ++t) n += (slo[t] == lane) + (sup[t] == lane);
-        int off = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int x = __shfl_up_sync(0xffffffffu, off, o);
-            if (lane >= o) off += x;
-        }
-        roff[lane + 1] = (unsigned short)off;
-        if (lane == 0) roff[0] = 0;
-        int at = off - n;
-        for (int t = 0; t < T; ++t) {
-            if (slo[t] == lane) ent[at++] = (unsigned short)t;
-            if (sup[t] == lane) ent[at++] = (unsigned short)(t | 0x8000);
-        }
-    }
+    for (int t = threadIdx.x; t < T; t += blockDim.x)
+        if (atomicOr(&pairs[slo[t]], 1u << sup[t]) >> sup[t] & 1u) twice = 1u;
     __syncthreads();
     double (*R)[QMAXL + 1] = Rs[w];
     double* b = bs[w];
-    for (int64_t c = (int64_t)blockIdx.x * QW + w; c < cells.n_cells; c += (int64_t)gridDim.x * QW) {
+    for (int64_t c = (int64_t)w * gridDim.x + blockIdx.x; c < cells.n_cells; c += (int64_t)gridDim.x * QW) {
         const double Ttr = cells.Ttr[c], Tve = cells.Tve[c];
         const double* dens = cells.n + c * nc;
         double nM = 0.0;
@@ -108,6 +96,8 @@ __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells
         const double lnTtr = log(Ttr), lnTve = log(Tve), iTtr = 1.0 / Ttr, iTve = 1.0 / Tve;
         const double nMa = nM * (1.0 / N_AVOGADRO), nea = ne * (1.0 / N_AVOGADRO);
         __syncwarp();
+        if (lane < l)
+            for (int j = 0; j < l; ++j) R[j][lane] = 0.0;
         // level weights Q_i = g_i e^{-c2 E_i / T} at both temperatures
         if (lane < l) {
             const double g = m.g[lane], x = -ph.c2 * m.E[lane];
@@ -118,8 +108,10 @@ __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells
             iQv[w][lane] = recip64(qv);
         }
         __syncwarp();
-        // transition rates per particle of the lower (up) / upper (down) level
-        for (int t = lane; t < T; t += 32) {
+        // transition rates per particle of the lower (up) / upper (down) level,
+        // straight to the rows that gain by them: R[upper][lower], R[lower][upper]
+        for (int t0 = 0; t0 < T; t0 += 32) {
+            const int t = min(t0 + lane, T - 1);
             const int i = slo[t], j = sup[t];
             // C T^n e^{-theta/T} as C e^{n ln T - theta/T}: one exp a rate
             const double theta = ph.c2 * (m.E[j] - m.E[i]);
@@ -132,26 +124,35 @@ __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells
                 ke_dn = ke_up * Qv[w][i] / Qv[w][j];
             }
             const double rad = m.lam[t] >= 200.0 ? m.A[t] : 0.0;
-            rate_up[w][t] = kh_up * nMa + ke_up * nea;
-            rate_dn[w][t] = kh_dn * nMa + ke_dn * nea + rad;
+            const double up = kh_up * nMa + ke_up * nea, dn = kh_dn * nMa + ke_dn * nea + rad;
+            if (!twice) {
+                R[j][i] = up;
+                R[i][j] = dn;
+            } else {   // pairs of levels with several transitions: added in their order
+                for (int q = 0; q < 32 && t0 + q < T; ++q) {
+                    if (lane == q) {
+                        R[j][i] += up;
+                        R[i][j] += dn;
+                    }
+                    __syncwarp();
+                }
+            }
         }
-        // row assembly: lane r owns row r
-        if (lane < l)
-            for (int j = 0; j < l; ++j) R[lane][j] = lane > 0 ? 0.0 : 1.0;
+        // lane r completes row r; what level r loses is what the others gain, column r
+        double diag = 0.0;
+        __syncwarp();
+        if (lane < l) {
+            double d[4] = {0.0, 0.0, 0.0, 0.0};
+            int j = 0;
+            for (; j + 3 < l; j += 4)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) d[q] -= R[j + q][lane];
+            for (; j < l; ++j) d[0] -= R[j][lane];
+            diag = (d[0] + d[1]) + (d[2] + d[3]);
+        }
         __syncwarp();
         if (lane < l) {
             if (lane > 0) {
-                double diag = 0.0;
-                for (int k = roff[lane]; k < roff[lane + 1]; ++k) {
-                    const int t = ent[k] & 0x7fff;
-                    const bool upper = ent[k] & 0x8000;
-                    const int j = upper ? slo[t] : sup[t];
-                    const double ru = rate_up[w][t], rd = rate_dn[w][t];
-                    diag -= upper ? rd : ru;
-                    const double gain = upper ? ru : rd;
-                    const double old = R[lane][j];   // nonzero only where a pair of levels has several transitions
-                    R[lane][j] = __double_as_longlong(old) == 0 ? gain : old + gain;
-                }
                 // electron-impact ionisation and three-body recombination
                 const double Qp = m.g_ion * exp_fix(-ph.c2 * m.E_ionize * iTve, tab);
                 const double x = 2.0 * M_PI * ph.me * ph.kB * Tve / (ph.h * ph.h);
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells
                 R[lane][lane] = diag - kf * nea;
                 b[lane] = -kr * nion * ne * nea;
             } else {   // closure: the levels and the lumped ones above sum to the density
+                for (int j = 0; j < l; ++j) R[0][j] = 1.0;
                 if (m.n_levels_all > l) {
                     double s = 0.0;
                     for (int p = l; p < m.n_levels_all; ++p) s += m.g[p] * exp_fix(-ph.c2 * m.E[p] * iTve, tab);
@@ -199,7 +201,15 @@ __global__ void __launch_bounds__(32 * QW) k_qss(rapral_cr_model m, rapral_cells
                 f = fma(fma(-f, piv, r), inv, f);   // the quotient, rounded once
                 if (nonfinite(f)) f = r / piv;      // pivots below 2^-1022
                 R[lane][k] = f;
-                for (int j = k + 1; j < l; ++j) R[lane][j] = fma(-f, R[k][j], R[lane][j]);
+                int j = k + 1;
+                for (; j + 3 < l; j += 4) {   // loads ahead of the stores, which the compiler has to keep in order
+                    double x[4], y[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) x[q] = R[k][j + q], y[q] = R[lane][j + q];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) R[lane][j + q] = fma(-f, x[q], y[q]);
+                }
+                for (; j < l; ++j) R[lane][j] = fma(-f, R[k][j], R[lane][j]);
                 b[lane] = fma(-f, b[k], b[lane]);
             }
             __syncwarp();
@@ -262,8 +272,9 @@ cudaError_t launch_qss(rapral_ctx* ctx, const rapral_cr_model* m, const rapral_c
                        const Phys& ph) {
     if (cells->n_cells == 0) return cudaSuccess;
     if (m->n_trans > QMAXT || m->n_levels > QMAXL) return cudaErrorInvalidValue;
-    // four blocks an SM fit (shared memory); each takes cells until none is left
-    const int64_t blocks = std::min<int64_t>((cells->n_cells + QW - 1) / QW, 152 * 4);
+    // four blocks an SM fit (shared memory); each takes cells until none is
+    // left, and the first cells go to a warp of every block
+    const int64_t blocks = std::min<int64_t>(cells->n_cells, 152 * 4);
     k_qss<<<(unsigned)blocks, 32 * QW, 0, ctx->stream>>>(*m, *cells, ph, n_out, ctx->d_status);
     return cudaGetLastError();
 }
