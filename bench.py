@@ -291,6 +291,36 @@ def march_traffic(cells, segments, grid_points):
     return t["bytes"] * (grid_points / t["grid_points"])
 
 
+def marched_segments(rays):
+    """Segments the march gathers for: of equal rays of a point (the same cells
+    and lengths: mirror images in an axisymmetric field), each pair's once.
+    Rays are told apart by a 64-bit hash here, by comparison in the march."""
+    import torch
+    t, n = rays.t, int(rays.struct.n_segments)
+    off, dev = t["seg_off"], t["seg_off"].device
+    length = off[1:] - off[:-1]
+    B = length.numel()
+    b = torch.repeat_interleave(torch.arange(B, device=dev), length)
+    pos = torch.arange(n, device=dev) - off[b]
+    ds = t["seg_ds"][:n].float().view(torch.int32).long()   # the lengths as the FP32 march holds them
+    h = (ds ^ (t["seg_cell"][:n].long() * 0x9E3779B97F4A7C1)) * 0x2545F4914F6CDD1D
+    h = ((h >> 29) ^ h) * (2 * pos + 0x5851F42D)
+    c = torch.cat([torch.zeros(1, dtype=torch.int64, device=dev), torch.cumsum(h, 0)])
+    point = torch.bucketize(torch.arange(B, device=dev), t["point_off"][1:], right=True)
+    key = (c[off[1:]] - c[off[:-1]]) * 0x1B873593 + point * 0x632BE59BD9B4E019 + length
+    _u, inv, count = torch.unique(key, return_inverse=True, return_counts=True)
+    one = torch.zeros_like(count).scatter_reduce(0, inv, length, "amax")
+    return int((((count + 1) // 2) * one).sum())
+
+
+def xu_operations(st):
+    """MUFU operations of the FP32 line sum, from the work counters: two rsqrt
+    and at least a quarter of a reciprocal an evaluation (four points of a line
+    that covers its tile share one, two lines elsewhere), two ex2 where the
+    Gaussian term counts (at least: whole runs of 32 points take both)."""
+    return 2.25 * st["evaluations"] + 2 * st["gauss_terms"]
+
+
 def cpu_baseline(problem, seconds, precision_note="f64"):
     """The oracle as it stands, on the host cores, on a bounded sample of the
     workload: every line, the whole grid, a few cells (one per thread), for
@@ -791,16 +821,16 @@ def run_headline(args):
         j = s % len(mine)
         if j == 0:
             pipe.begin()
-            launches[0] += 2                    # cell validation + populations
+            launches[0] += 1                    # populations (they check the cells)
         k0, nk = mine[j]
         if kev is not None:
             ctx.set_profile_events(*kev)
         pipe.step(k0, nk, march_events=mev)
         if kev is not None:
             ctx.set_profile_events(None, None)
-        # coefficients: cell and line validation, line prep, cell prep, bin bounds, count, scan, fill,
-        # line sum; march: ray validation, three FP32 copies, march, group sum; flux: part + sum
-        launches[0] += 9 + 6 + 2
+        # coefficients: cell records, line plan, count, scan, fill, line sum; march: ray checks with the FP32
+        # copies, hash, match and verify of equal rays, bundle plan, march, group sum; flux: part + sum
+        launches[0] += 6 + 7 + 2
         if j == len(mine) - 1:
             pipe.end()
             with torch.cuda.stream(sa):
@@ -865,14 +895,16 @@ def run_headline(args):
     nk_mean = float(np.mean(steps_nk))
     uniq = C * nk_mean * 8 + P * nk_mean * 4
     seglam_launch = nseg * nk_mean
-    gather = seglam_launch * 8 / (march_mean * 1e-3) / 1e9
+    n_marched = marched_segments(dp.rays)
+    gather_bytes = n_marched * nk_mean * 8
+    gather = gather_bytes / (march_mean * 1e-3) / 1e9
     l2 = l2_gather_peak(local)
     l2_peak = max(l2["GBps_48MB_table"], l2["GBps_96MB_table"])
-    march = {"kernel": "k_march1 (single-direction rays, FP32; + ray validation, FP32 copies, bundle plan, "
-                       "group sum)",
-             "kernel_ms": march_mean, "segments": nseg, "segment_lambda_per_launch": seglam_launch,
+    march = {"kernel": "k_march1 (single-direction rays, FP32; + ray checks and FP32 copies, the search for equal "
+                       "rays, bundle plan, group sum)",
+             "kernel_ms": march_mean, "segments": nseg, "segments_marched": n_marched, "segment_lambda_per_launch": seglam_launch,
              "ray_lambda_segments_per_s": seglam_launch / (march_mean * 1e-3),
-             "gather_bytes_per_launch": seglam_launch * 8, "gather_GBps": gather,
+             "gather_bytes_per_launch": gather_bytes, "gather_GBps": gather,
              "l2_gather_peak": l2, "frac_of_l2_gather_peak": gather / l2_peak,
              "dram_unique_bytes_per_launch": uniq,
              "dram_traffic_bytes_per_launch": march_traffic(C, nseg, nk_mean),
@@ -882,13 +914,14 @@ def run_headline(args):
     roof = {"bound": "hbm", "achieved": gather, "peak": hbm, "unit": "GB/s", "frac": gather / hbm,
             "traffic": march_traffic(C, nseg, nk_mean),
             "kernel": "k_march1 (single-direction rays, FP32)", "kernel_ms": march_mean,
-            "algorithmic_bytes": seglam_launch * 8,
+            "algorithmic_bytes": gather_bytes,
             "algorithmic_unit": "8 B (FP32 kappa + j of the next cell) gathered per segment-wavelength, x the "
-                                "launch's segments x columns",
+                                "segments of the launch's distinct rays (equal rays of a point, mirror images "
+                                "here, are marched once) x columns",
             "peak_source": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in peaks else "fallback",
             "served_from": "L2: the gathers hit L2, whose measured gather bandwidth is in march.l2_gather_peak; "
                            "DRAM (traffic) sees the chunk's kappa / j once and the segment lists once per "
-                           "64-column wavelength tile",
+                           "128-column wavelength tile",
             "frac_of_l2_gather_peak": gather / l2_peak}
     out = {"metric": METRIC, "value": value, "unit": "cell·λ points/s", "n_gpus": world, "steps": K,
            "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
@@ -913,7 +946,7 @@ def run_headline(args):
         ctx.reset_stats()
         R.spectral_coeffs(ctx, dp.species, dp.lines, dp.cells, p.grid, k0, nk, R.FP32, kap, em)
         st = ctx.get_stats()
-        per_chunk[j] = (3 * st["evaluations"] + st["gauss_terms"] + st["correction_terms"], st["evaluations"])
+        per_chunk[j] = (xu_operations(st), st["evaluations"])
     ctx.set_counters(False)
     xu = sum(per_chunk[s % len(mine)][0] for s in range(K))
     ev_total = sum(per_chunk[s % len(mine)][1] for s in range(K))
@@ -927,7 +960,7 @@ def run_headline(args):
                        "timed_inside": march["timed_inside"].replace("(the kernel alone on the GPU)", "(alone)"),
                        "note": "time: the line-sum kernel of each timed step (CUDA events the library records "
                                "around the launch, on its stream); XU "
-                               "operations: 3 per evaluation + one per Gaussian and correction term, from the "
+                               "operations: 2.25 per evaluation + two per Gaussian term, from the "
                                "library's work counters in an untimed pass over the same chunks"}
 
     if not args.no_e2e:
@@ -1031,7 +1064,7 @@ def stagnation_block(args, local, world, rank, fp64=True):
     peaks = measured_peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0)) * 1e6
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    xu_ops = 3 * stats["evaluations"] + stats["gauss_terms"] + stats["correction_terms"]
+    xu_ops = xu_operations(stats)
     peak = n_sm * 16 * sm_max / 1e9
     out = {"workload": STAG_WORKLOAD, "precision": "fp32-chosen", "steps": steps, "warmup": 3, "ms_per_step": ms,
            "value": C * K / (ms * 1e-3), "unit": "cell·λ points/s", "tiling": tuned,

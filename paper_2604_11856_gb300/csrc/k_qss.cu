@@ -8,7 +8,7 @@
 // throughout: the systems span many orders of magnitude in their rates.
 //
 // The FP64 pipe bounds it (a warp instruction of it takes 17 clocks of an SM,
-// whatever lanes are on; by count it is busy 75 % of the time), so the count
+// whatever lanes are on; it is 89 % busy), so the count
 // of FP64 warp instructions a cell is what the layout keeps down: 32 sums for
 // the diagonals of 32 rows (from lists of each row's transitions two a list
 // entry, by transitions four with two lanes on, 1,984 for 496), exponentials
