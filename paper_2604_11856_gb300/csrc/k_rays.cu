@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(32 * (DS ? DS : march_warps(MAXD, SL)),
     constexpr int W = DS ? DS : march_warps(MAXD, SL), CW = DS ? 1 : W / SL, TW = CW * 32 * V;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slice = DS ? 0 : warp / CW, cgrp = DS ? 0 : warp % CW;
+    const int nr = DS ? (int)(blockDim.x >> 5) : SL;   // partial sums a column
     // columns fit in int: nk <= 32 x 65535 (checked by the caller)
     const int nk = (int)a.nk;
     const int tile0 = (int)blockIdx.y * TW;
@@ -596,46 +597,46 @@ __global__ void __launch_bounds__(32 * (DS ? DS : march_warps(MAXD, SL)),
     const unsigned p = blockIdx.x >> lgG, grp = blockIdx.x & ((1u << lgG) - 1u);
     const int64_t b1 = a.point_off[p + 1];
     for (int64_t b = a.point_off[p] + (int64_t)grp * SL + slice; b < b1; b += (int64_t)SL << lgG) {
-        int64_t d0 = a.dir_off[b];
-        int nd = (int)(a.dir_off[b + 1] - d0);
-        if (DS) {
-            const int q = min((nd + (int)(blockDim.x >> 5) - 1) / (int)(blockDim.x >> 5), MAXD);
-            d0 += warp * q;
-            nd = min(nd - warp * q, q);
-        }
-        if (nd <= 0) continue;
-        T I[V][MAXD];
-        if constexpr (NODES) {
-            const bool wall = a.wall_row && a.bundle_wall[b];
+        const int64_t db = a.dir_off[b];
+        const int nb = (int)(a.dir_off[b + 1] - db);
+        // a warp's share and where its next one starts (a second share only if
+        // max_dirs understates the bundle)
+        const int q = DS ? min((nb + nr - 1) / nr, MAXD) : nb;
+        for (int first = DS ? warp * q : 0; first < nb; first += DS ? nr * q : nb) {
+            const int64_t d0 = db + first;
+            const int nd = DS ? min(nb - first, q) : nb;
+            T I[V][MAXD];
+            if constexpr (NODES) {
+                const bool wall = a.wall_row && a.bundle_wall[b];
 #pragma unroll
-            for (int v = 0; v < V; ++v) I[v][0] = wall ? reinterpret_cast<const T*>(a.wall_row)[col0 + 32 * v] : T(0);
-            march_nodes<T, V>(a, b, dir_val<T>(a.dir_scale, a.dir_scale_f, d0), stage, lane, kbase, ldb, offK, offJ,
-                              I);
-        } else {
-            if constexpr (MAXD == 1) march_bundle<T, V>(a, b, d0, stage, lane, kbase, ldb, offK, offJ, col0, I);
-            else march_multi<T, MAXD>(a, b, d0, nd, stage, lane, kbase, ldb, offK, offJ, col0, I);
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const int kk = colu + 32 * v;
-            const bool own = kk >= tile0 && kk < nk;
-            T part_v = T(0);
-#pragma unroll
-            for (int d = 0; d < MAXD; ++d) {
-                if (d < nd) {
-                    part_v += dir_val<T>(a.dir_weight, a.dir_weight_f, d0 + d) * I[v][d];
-                    if (a.I_out && own) reinterpret_cast<T*>(a.I_out)[(d0 + d) * a.nk + kk] = I[v][d];
-                }
+                for (int v = 0; v < V; ++v) I[v][0] = wall ? reinterpret_cast<const T*>(a.wall_row)[col0 + 32 * v] : T(0);
+                march_nodes<T, V>(a, b, dir_val<T>(a.dir_scale, a.dir_scale_f, d0), stage, lane, kbase, ldb, offK,
+                                  offJ, I);
+            } else {
+                if constexpr (MAXD == 1) march_bundle<T, V>(a, b, d0, stage, lane, kbase, ldb, offK, offJ, col0, I);
+                else march_multi<T, MAXD>(a, b, d0, nd, stage, lane, kbase, ldb, offK, offJ, col0, I);
             }
-            // compensated sum over the slice's bundles
-            const T y = part_v - comp[v];
-            const T tt = acc[v] + y;
-            comp[v] = (tt - acc[v]) - y;
-            acc[v] = tt;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int kk = colu + 32 * v;
+                const bool own = kk >= tile0 && kk < nk;
+                T part_v = T(0);
+#pragma unroll
+                for (int d = 0; d < MAXD; ++d) {
+                    if (d < nd) {
+                        part_v += dir_val<T>(a.dir_weight, a.dir_weight_f, d0 + d) * I[v][d];
+                        if (a.I_out && own) reinterpret_cast<T*>(a.I_out)[(d0 + d) * a.nk + kk] = I[v][d];
+                    }
+                }
+                // compensated sum over the slice's bundles
+                const T y = part_v - comp[v];
+                const T tt = acc[v] + y;
+                comp[v] = (tt - acc[v]) - y;
+                acc[v] = tt;
+            }
         }
     }
     constexpr int NR = DS ? DS : SL;
-    const int nr = DS ? (int)(blockDim.x >> 5) : SL;
     __shared__ T red[NR][TW];
 #pragma unroll
     for (int v = 0; v < V; ++v) red[DS ? warp : slice][cgrp * 32 * V + lane + 32 * v] = acc[v];

@@ -110,3 +110,28 @@ def test_split_directions(precision, tol, n_mu, nk):
     flux = np.abs(weight) * tile(big)
     assert np.max(np.abs(q[0].double().cpu().numpy() - (weight * tile(ref)).sum(0)) /
                   np.maximum(flux.sum(0), 1e-300)) <= tol
+
+
+@pytest.mark.parametrize("precision", [R.FP64, R.FP32])
+@pytest.mark.parametrize("claimed", [2, 5, 17])
+def test_bundle_longer_than_claimed(precision, claimed):
+    """A bundle of 17 directions in a ray set that claims fewer is marched whole (within the march's rounding, as above)."""
+    ctx = R.Context(0)
+    rng = np.random.default_rng(3)
+    C, nk = 9, 70
+    dt = torch.float64 if precision == R.FP64 else torch.float32
+    tk = torch.as_tensor(2.0 ** rng.uniform(-20, -8, (C, nk)), device=ctx.device).to(dt)
+    tj = torch.as_tensor(2.0 ** rng.uniform(-3, 3, (C, nk)), device=ctx.device).to(dt)
+    geo = synth.SlabGeometry(cell_order=np.arange(C, dtype=np.int64), dx=np.full(C, 0.5),
+                             mu=np.linspace(0.1, 0.9, 16), wmu=np.full(16, 1.0 / 16))
+    rays = R.slab_rays(ctx, geo, ctx.device)
+    out = []
+    for m in (17, claimed):
+        rays.struct.max_dirs = m
+        q = torch.empty((1, nk), dtype=dt, device=ctx.device)
+        I = torch.full((rays.n_dirs, nk), float("nan"), dtype=dt, device=ctx.device)
+        R.trace_rays(ctx, rays, C, tk, tj, synth.Grid(100.0, 200.0, nk), 0, nk, precision, q, I)
+        ctx.sync()
+        out.append(I.cpu().numpy())
+    assert np.all(np.isfinite(out[0])) and np.max(np.abs(out[0] / out[1] - 1.0)) <= (
+        7e-14 if precision == R.FP64 else 3.8e-5)
