@@ -763,12 +763,21 @@ __device__ __forceinline__ unsigned mix32(unsigned x) {
 }
 
 // key[b]: 64-bit hash of bundle b's segments, scale and wall flag (0: not one
-// direction, never paired).  One warp a bundle.
-__global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t B, unsigned long long* __restrict__ key) {
+// direction, never paired); cand[] and partner[] cleared.  One warp a bundle.
+// The points' bundles are [point_off[0], point_off[P]); what a set holds
+// before or after them belongs to no point, and its lists are not read.
+__global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t P, int64_t B,
+                                                  unsigned long long* __restrict__ key, int32_t* __restrict__ cand,
+                                                  int32_t* __restrict__ partner) {
     if (*a.status) return;
     const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (b >= B) return;
+    if (lane == 0) cand[b] = partner[b] = -1;
+    if (b < a.point_off[0] || b >= a.point_off[P]) {
+        if (lane == 0) key[b] = 0ULL;
+        return;
+    }
     const int64_t s0 = a.seg_off[b], s1 = a.seg_off[b + 1], d0 = a.dir_off[b];
     unsigned h0 = 0, h1 = 0;
     for (int64_t i = s0 + lane; i < s1; i += 32) {
@@ -791,18 +800,14 @@ __global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t B, unsign
 }
 
 // cand[b]: the earlier bundle of the point that bundle b may be the partner of
-// (a key's odd ranks go to the one before them), -1 for the others; partner[]
-// cleared.  One block a point, four lanes a bundle.
+// (a key's odd ranks go to the one before them), -1 for the others.  One block
+// a point, four lanes a bundle.
 __global__ void __launch_bounds__(512) k_ray_match(MarchArgs a, const unsigned long long* __restrict__ key,
-                                                   int32_t* __restrict__ cand, int32_t* __restrict__ partner) {
+                                                   int32_t* __restrict__ cand) {
     if (*a.status) return;
     __shared__ unsigned long long ks[M1_PAIR_MAX];
     const int64_t pb0 = a.point_off[blockIdx.x];
     const int64_t nb = a.point_off[blockIdx.x + 1] - pb0;
-    for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) {
-        partner[pb0 + k] = -1;
-        if (nb > M1_PAIR_MAX) cand[pb0 + k] = -1;
-    }
     if (nb > M1_PAIR_MAX) return;
     const int n = (int)nb;
     for (int k = threadIdx.x; k < n; k += blockDim.x) ks[k] = key[pb0 + k];
@@ -1337,8 +1342,9 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
                                  void* part, const M1Plan& pl) {
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
-    if (B > 0) k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.key);
-    k_ray_match<<<(unsigned)P, 512, 0, ctx->stream>>>(a, pl.key, pl.cand, pl.partner);
+    if (B > 0)
+        k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, P, B, pl.key, pl.cand, pl.partner);
+    k_ray_match<<<(unsigned)P, 512, 0, ctx->stream>>>(a, pl.key, pl.cand);
     if (B > 0) k_ray_verify<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.cand, pl.partner);
     k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, pl.cand, G, pl.plan, pl.soff,
                                                              a.status);
