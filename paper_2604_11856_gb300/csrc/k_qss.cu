@@ -54,7 +54,9 @@ __device__ __forceinline__ double recip64(double x) {
 
 __global__ void __launch_bounds__(32 * QW, 4)
     k_qss(rapral_cr_model m, rapral_cells cells, Phys ph, double* n_out, int* status) {
-    if (*status) return;
+    // one decision for the block: its warps fill the shared tables together,
+    // and other blocks of this launch may be setting the status meanwhile
+    if (__syncthreads_or(*status != 0)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     __shared__ uint64_t tab[EXPFIX_N];
     __shared__ double Rs[QW][QMAXL][QMAXL + 1];
