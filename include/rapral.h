@@ -267,7 +267,7 @@ RAPRAL_API int rapral_workspace_bytes(int64_t n_lines, int64_t n_cells, int64_t 
  *   lnpref[c][s] = ln n_{c, density_col[s]} - ln Z_s   (-inf when n = 0).
  * In: sp, cells (Ttr, Tve, n).  Out: lnpref [C][S] FP64 (device).
  * Errors: EINVAL (sizes, S > RAPRAL_MAX_SPECIES; device: T <= 0 or not
- * finite, n < 0). */
+ * finite, n < 0: lnpref is then partly written and must not be used). */
 RAPRAL_API int rapral_populations(rapral_ctx* ctx, const rapral_species* sp,
                        const rapral_cells* cells, double* lnpref);
 

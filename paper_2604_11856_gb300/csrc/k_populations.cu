@@ -48,7 +48,9 @@ __global__ void __launch_bounds__(256) k_populations(rapral_species sp, const do
                                                      const double* __restrict__ Tve, const double* __restrict__ n,
                                                      int32_t ncol, int64_t C, double c2, double* __restrict__ lnpref,
                                                      int* status) {
-    if (*status) return;
+    // one decision for the block: its warps share the tables and sums, and
+    // other blocks of this launch may be setting the status meanwhile
+    if (__syncthreads_or(*status != 0)) return;
     __shared__ uint64_t tab[EXPFIX_N];
     __shared__ double pv[CC][32];      // Boltzmann factors of 32 vibrational levels of a state, with its weight
     __shared__ double red[CC][8];
