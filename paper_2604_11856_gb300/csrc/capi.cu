@@ -425,7 +425,7 @@ int rapral_wall_flux(rapral_ctx* ctx, const void* q_lambda, int precision, const
     cudaSetDevice(ctx->device);
     // the partial sums live at the start of the workspace: every earlier user
     // of the workspace on this stream has been enqueued before
-    st = ws_reserve(ctx, (size_t)wall_flux_parts(nk) * (size_t)n_points * 16 + 256);
+    st = ws_reserve(ctx, (size_t)wall_flux_parts(nk) * (size_t)n_points * sizeof(double) + 256);
     if (st) return st;
     return cuda_status(ctx, launch_wall_flux(ctx, q_lambda, precision, g, grid_h(g), k0, nk, n_points, q, ctx->ws),
                        "wall flux");

@@ -1159,11 +1159,14 @@ __global__ void k_group_sum(const T* __restrict__ part, int G, int64_t P, int64_
 }
 
 // Spectral integral in two deterministic stages: blocks (point, slice)
-// Neumaier-sum a slice of FLUX_SPAN grid points each, eight a thread, then one
-// warp per point adds the slices, each lane a strided part in order.  Weights
-// other than 1 (the grid's ends) are applied to their points, the spacing once
-// at the end: five FP64 operations a point.
-constexpr int FLUX_SPAN = 1024;
+// Neumaier-sum a slice of flux_span(nk) grid points each, eight a thread, then
+// one warp per point adds the slices, each lane a strided part in order.
+// Weights other than 1 (the grid's ends) are applied to their points, the
+// spacing once at the end: five FP64 operations a point.  The slices are a
+// grid's second extent, 65,535 at most: ranges past 65,535 x 1,024 points take
+// slices of 4,096.
+constexpr int64_t MAX_FLUX_PARTS = 65535;
+static int64_t flux_span(int64_t nk) { return nk <= MAX_FLUX_PARTS * 1024 ? 1024 : 4096; }
 
 // (s, c) += x, Neumaier; magnitudes are compared by their bits
 __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
@@ -1176,11 +1179,11 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
 
 template <class T>
 __global__ void __launch_bounds__(128) k_wall_flux_part(const T* __restrict__ qlam, int64_t nk, int64_t k0,
-                                                        int64_t n, double* __restrict__ part,
+                                                        int64_t n, int64_t span, double* __restrict__ part,
                                                         const int* status) {
     if (*status) return;
     const int64_t p = blockIdx.x;
-    const int64_t a = (int64_t)blockIdx.y * FLUX_SPAN, b = min(a + FLUX_SPAN, nk);
+    const int64_t a = (int64_t)blockIdx.y * span, b = min(a + span, nk);
     double s = 0.0, c = 0.0;
     for (int64_t k = a + threadIdx.x; k < b; k += blockDim.x) {
         const int64_t kg = k0 + k;
@@ -1507,7 +1510,7 @@ cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kapp
                           r->node_values != 0);
 }
 
-int64_t wall_flux_parts(int64_t nk) { return (nk + FLUX_SPAN - 1) / FLUX_SPAN; }
+int64_t wall_flux_parts(int64_t nk) { return (nk + flux_span(nk) - 1) / flux_span(nk); }
 
 cudaError_t launch_wall_flux(rapral_ctx* ctx, const void* q_lambda, int precision, const rapral_grid* g, double h,
                              int64_t k0, int64_t nk, int64_t n_points, double* q, void* partials) {
@@ -1518,10 +1521,10 @@ cudaError_t launch_wall_flux(rapral_ctx* ctx, const void* q_lambda, int precisio
     dim3 grid((unsigned)n_points, (unsigned)np);
     if (precision == RAPRAL_FP64)
         k_wall_flux_part<double><<<grid, 128, 0, ctx->stream>>>(reinterpret_cast<const double*>(q_lambda), nk, k0,
-                                                                g->n, part, ctx->d_status);
+                                                                g->n, flux_span(nk), part, ctx->d_status);
     else
         k_wall_flux_part<float><<<grid, 128, 0, ctx->stream>>>(reinterpret_cast<const float*>(q_lambda), nk, k0,
-                                                               g->n, part, ctx->d_status);
+                                                               g->n, flux_span(nk), part, ctx->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_wall_flux_sum<<<(unsigned)n_points, 32, 0, ctx->stream>>>(part, (int)np, h_um, q, ctx->d_status);

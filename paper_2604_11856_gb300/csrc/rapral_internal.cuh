@@ -336,7 +336,7 @@ size_t march_scratch_bytes(const rapral_rays* r, int64_t nk, int precision);
 cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kappa, const void* emis,
                          int64_t ld, const rapral_grid* g, double h, int64_t k0, int64_t nk, int precision,
                          void* q_lambda, void* I_out, const Phys& ph, void* scratch);
-// Spectral flux: needs `partials` of wall_flux_parts(nk) * n_points * 16 bytes.
+// Spectral flux: needs `partials` of wall_flux_parts(nk) * n_points doubles.
 int64_t wall_flux_parts(int64_t nk);
 cudaError_t launch_wall_flux(rapral_ctx* ctx, const void* q_lambda, int precision, const rapral_grid* g,
                              double h, int64_t k0, int64_t nk, int64_t n_points, double* q, void* partials);
