@@ -895,7 +895,7 @@ struct LineSlots {
 // far evaluation with its own reciprocal; the two lines share the one of
 // their denominators' product (20 clocks, beside 17 of the FP32 pipe).
 // |u| is capped so that the product of a point in its window and one far out
-// of it stays in range; points outside a window add zero.
+// of it stays in range.
 template <bool NEAR>
 __device__ __forceinline__ void slot_eval(float k, float2 nmid, float2 half, float2 ub, float2 ubl, float2 s, float2 nc,
                                           float2 r, float2 aj, float2 ak, float& bj, float& bk) {
@@ -924,10 +924,16 @@ __device__ __forceinline__ void slot_eval(float k, float2 nmid, float2 half, flo
         h = __ffma2_rn(__fmul2_rn(c2(0.016f), omr), e2, h);
         h = __ffma2_rn(omr, g, __fmul2_rn(r, h));
     }
-    h.x = fabsf(d.x) <= half.x ? h.x : 0.0f;
-    h.y = fabsf(d.y) <= half.y ? h.y : 0.0f;
-    bj = fmaf(aj.y, h.y, fmaf(aj.x, h.x, bj));
-    bk = fmaf(ak.y, h.y, fmaf(ak.x, h.x, bk));
+    // predicated: outside its window a line adds nothing, whatever its strength
+    // (a strength past the FP32 range times a zeroed profile would be NaN)
+    if (fabsf(d.x) <= half.x) {
+        bj = fmaf(aj.x, h.x, bj);
+        bk = fmaf(ak.x, h.x, bk);
+    }
+    if (fabsf(d.y) <= half.y) {
+        bj = fmaf(aj.y, h.y, bj);
+        bk = fmaf(ak.y, h.y, bk);
+    }
 }
 
 // The n staged lines over the lane's points lane + 32 i of the tile.  Lines
