@@ -600,11 +600,12 @@ __global__ void __launch_bounds__(32 * (DS ? DS : march_warps(MAXD, SL)),
         const int64_t db = a.dir_off[b];
         const int nb = (int)(a.dir_off[b + 1] - db);
         // a warp's share and where its next one starts (a second share only if
-        // max_dirs understates the bundle)
-        const int q = DS ? min((nb + nr - 1) / nr, MAXD) : nb;
-        for (int first = DS ? warp * q : 0; first < nb; first += DS ? nr * q : nb) {
+        // max_dirs understates the bundle: one of several directions is marched
+        // whole in every form)
+        const int q = DS ? min((nb + nr - 1) / nr, MAXD) : MAXD > 1 ? min(nb, MAXD) : nb;
+        for (int first = DS ? warp * q : 0; first < nb; first += DS ? nr * q : q) {
             const int64_t d0 = db + first;
-            const int nd = DS ? min(nb - first, q) : nb;
+            const int nd = min(nb - first, q);
             T I[V][MAXD];
             if constexpr (NODES) {
                 const bool wall = a.wall_row && a.bundle_wall[b];
