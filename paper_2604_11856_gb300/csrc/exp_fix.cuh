@@ -107,7 +107,12 @@ __device__ __forceinline__ double exp_fix(double x, const uint64_t* tab) {
 
 // e^{-b E} for many E >= 0 and a few b > 0 (Boltzmann factors, b = c2 / T):
 // E as 64-bit fixed point with 44 fraction bits, b log2(e) as a normalised
-// 64-bit mantissa, t their product.
+// 64-bit mantissa, t their product.  For b < 2^-10 (T above 1,473 K) E's last
+// bit is worth b 2^-45 < 2^-55 of the result and t's less than 0.7 2^-53, so
+// the error is below 1.8 2^-53 for any E, while the rounding of a double b E
+// alone is b E 2^-53 or less.  With a larger b the fixed point would hold
+// less than a double (b 2^-45: 1e-14 at 3 K), and the product is formed in
+// FP64: exp_fix(-b E).
 constexpr uint64_t EXPFIX_BAD = ~uint64_t(0);
 // E in [0, 2^20) in units of 2^-44, else EXPFIX_BAD
 __device__ __forceinline__ uint64_t expfix_energy(double E) {
@@ -120,19 +125,18 @@ __device__ __forceinline__ uint64_t expfix_energy(double E) {
 }
 struct ExpFixScale {
     uint64_t m;   // b log2(e) = m 2^(-64 - (F - 44))
-    int F;        // fraction bits of the products; 0: b outside (0, 0.69), use exp
+    int F;        // fraction bits of the products; 0: b outside (2^-1022, 2^-10), exp_fix(-b E)
 };
 __device__ __forceinline__ ExpFixScale expfix_scale(double b) {
     ExpFixScale r;
     r.m = 0; r.F = 0;
     const uint64_t bits = (uint64_t)__double_as_longlong(b);
     const int ex = (int)(bits >> 52);
-    if (ex == 0 || ex > 1030) return r;   // zero, negative, inf, NaN or large
+    if (ex == 0 || ex >= 1013) return r;   // zero, negative, inf, NaN or 2^-10 and above
     uint64_t m = __umul64hi((bits << 11) | (uint64_t(1) << 63), EXPFIX_LOG2E);
     int e = ex;
     if (!(m >> 63)) { m <<= 1; --e; }     // b log2(e) = m 2^(e - 1085)
-    int s = 1021 - e;
-    if (s < 0) return r;
+    int s = 1021 - e;                     // 9 or more
     if (s > 19) { m = s - 19 < 64 ? m >> (s - 19) : 0; s = 19; }
     r.m = m;
     r.F = 44 + s;
@@ -140,13 +144,15 @@ __device__ __forceinline__ ExpFixScale expfix_scale(double b) {
 }
 // (out of line, so that its product is not formed ahead of the test: an FP64
 // operation a term)
-static __device__ __noinline__ double expfix_far(double E, double b) { return exp(-b * E); }
+static __device__ __noinline__ double expfix_far(double E, double b, const uint64_t* tab) {
+    return exp_fix(-b * E, tab);
+}
 // e^{-b E}: Ef from expfix_energy(E), sc from expfix_scale(b)
 __device__ __forceinline__ double expfix_boltzmann(uint64_t Ef, const ExpFixScale& sc, double E, double b,
                                                    const uint64_t* tab) {
     const uint64_t P = __umul64hi(Ef, sc.m);
     const int n = (int)(P >> sc.F);
-    if (sc.F == 0 || Ef == EXPFIX_BAD || (P >> sc.F) > 1000) return expfix_far(E, b);
+    if (sc.F == 0 || Ef == EXPFIX_BAD || (P >> sc.F) > 1000) return expfix_far(E, b, tab);
     return expfix_double(expfix_frac(P << (64 - sc.F), tab), n);
 }
 
