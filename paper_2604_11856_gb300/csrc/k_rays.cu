@@ -1365,10 +1365,16 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
     // four adjacent columns a lane where 16-byte loads are aligned (100 x 50
     // cells, 20 points x 512 rays, 16,384 columns: 3.93 ms, two columns 4.16),
     // two where 8-byte ones are (16,382: 4.24), else two columns 32 apart (16,383:
-    // 4.72, four of them 4.95)
+    // 4.72, four of them 4.95).  Four halve the blocks, so they wait for ten
+    // blocks an SM, two and a half waves: 10 points x 512 rays of 80 segments,
+    // 128 / 512 / 1,024 / 1,536 / 2,048 / 4,096 columns (160 to 5,120 blocks of
+    // four) 146 / 252 / 377 / 506 / 637 / 1,199 us with four, 114 / 227 / 365 /
+    // 516 / 656 / 1,251 with two; 200 points x 64 rays, 256 and 512 columns (800,
+    // 1,600) 166 and 255 with four, 156 and 258 with two.
     float* pf = reinterpret_cast<float*>(part);
     const auto grid = [&](int np) { return dim3((unsigned)(P << lgG), div_up(nk, 64 * np)); };
-    if (march1_vec(a, nk, part, 2))
+    const bool four = (P << lgG) * (int64_t)div_up(nk, 128) >= 152 * 10;
+    if (four && march1_vec(a, nk, part, 2))
         k_march1<2, true><<<grid(2), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
     else if (march1_vec(a, nk, part, 1))
         k_march1<1, true><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
