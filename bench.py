@@ -829,8 +829,8 @@ def run_headline(args):
         if kev is not None:
             ctx.set_profile_events(None, None)
         # coefficients: cell records, line plan, count, scan, fill, line sum; march: ray checks with the FP32
-        # copies, hash, match and verify of equal rays, bundle plan, march, group sum; flux: part + sum
-        launches[0] += 6 + 7 + 2
+        # copies, hash and comparison of equal rays, bundle plan, march, group sum; flux: part + sum
+        launches[0] += 6 + 6 + 2
         if j == len(mine) - 1:
             pipe.end()
             with torch.cuda.stream(sa):

@@ -667,7 +667,7 @@ __global__ void __launch_bounds__(32 * (DS ? DS : march_warps(MAXD, SL)),
 //    removes the averaging multiplies;
 //  * the step (m1_step) carries minus the intensity and minus the half length
 //    and takes the series as long as the depth needs;
-//  * equal rays of a point are marched once (k_ray_match, k_ray_verify);
+//  * equal rays of a point are marched once (k_ray_hash, k_ray_match);
 //  * the staged list holds, for step j, the segment's halved length (as the
 //    packed pair the step multiplies by) and the byte offset of the row of the
 //    cell PF steps ahead (row x ld, computed once by the staging lane), so a
@@ -756,6 +756,14 @@ __device__ __forceinline__ void m1_step(float2& M, float2 Kf, float2 Jf, float2 
 // the step below, 100 x 50 cells, 20 points x 512 rays, 16,384 columns: 7.73 ->
 // 4.16 ms.
 constexpr int M1_PAIR_MAX = 2048;   // bundles of a point compared (16 KB of keys); more: no pairs
+// The search takes 12 to 22 us (two launches and a plan of what is left): it
+// pays from about 30 us of march on where a set has equal rays.  10 points x 512
+// rays of 80 segments x 256 / 512 / 1,000 columns, none equal: 146 / 213 / 351 us
+// searched, 131 / 198 / 336 not; every two equal: 99 / 135 / 205 and 132 / 198 /
+// 336.  At 128 columns none would take 103 and 84, every two 72 and 84: below the
+// limits the rays march as they are.
+constexpr int64_t M1_PAIR_WORK = int64_t(1) << 25;   // segments x columns, and
+constexpr int64_t M1_PAIR_COLUMNS = 256;             // columns, from which a set is searched
 
 __device__ __forceinline__ unsigned mix32(unsigned x) {
     x ^= x >> 16; x *= 0x7feb352du;
@@ -774,82 +782,87 @@ __global__ void __launch_bounds__(256) k_ray_hash(MarchArgs a, int64_t P, int64_
     const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (b >= B) return;
-    if (lane == 0) cand[b] = partner[b] = -1;
-    if (b < a.point_off[0] || b >= a.point_off[P]) {
-        if (lane == 0) key[b] = 0ULL;
-        return;
-    }
+    // everything that needs no other value is loaded at once: latency is all this pass costs
+    const int64_t in0 = a.point_off[0], in1 = a.point_off[P];
     const int64_t s0 = a.seg_off[b], s1 = a.seg_off[b + 1], d0 = a.dir_off[b];
-    unsigned h0 = 0, h1 = 0;
-    for (int64_t i = s0 + lane; i < s1; i += 32) {
-        const unsigned x = mix32((unsigned)a.seg_cell[i] * 0x9e3779b1u + (unsigned)(i - s0));
-        const unsigned y = mix32(__float_as_uint(a.seg_ds_f[i]) ^ x);
-        h0 += y;
-        h1 += mix32(y + 0x68bc21ebu);
-    }
-    h0 = __reduce_add_sync(0xffffffffu, h0);
-    h1 = __reduce_add_sync(0xffffffffu, h1);
-    if (lane == 0) {
-        unsigned long long k = 0ULL;
-        if (a.dir_off[b + 1] - d0 == 1) {
-            h0 = mix32(h0 ^ __float_as_uint(a.dir_scale_f[d0]));
-            h1 = mix32(h1 + (unsigned)(s1 - s0) * 2u + (a.bundle_wall[b] != 0));
-            k = ((unsigned long long)h0 << 32 | h1) | 1ULL;
+    const int64_t nd = a.dir_off[b + 1] - d0;
+    const bool wall = a.bundle_wall[b] != 0;
+    if (lane == 0) cand[b] = partner[b] = -1;
+    unsigned long long k = 0ULL;
+    if (b >= in0 && b < in1 && nd == 1) {
+        const unsigned sc = __float_as_uint(a.dir_scale_f[d0]);
+        unsigned h0 = 0, h1 = 0;
+        for (int64_t i = s0 + lane; i < s1; i += 32) {
+            const unsigned x = mix32((unsigned)a.seg_cell[i] * 0x9e3779b1u + (unsigned)(i - s0));
+            const unsigned y = mix32(__float_as_uint(a.seg_ds_f[i]) ^ x);
+            h0 += y;
+            h1 += mix32(y + 0x68bc21ebu);
         }
-        key[b] = k;
+        h0 = __reduce_add_sync(0xffffffffu, h0);
+        h1 = __reduce_add_sync(0xffffffffu, h1);
+        h0 = mix32(h0 ^ sc);
+        h1 = mix32(h1 + (unsigned)(s1 - s0) * 2u + wall);
+        k = ((unsigned long long)h0 << 32 | h1) | 1ULL;
     }
+    if (lane == 0) key[b] = k;
 }
 
-// cand[b]: the earlier bundle of the point that bundle b may be the partner of
-// (a key's odd ranks go to the one before them), -1 for the others.  One block
-// a point, four lanes a bundle.
-__global__ void __launch_bounds__(512) k_ray_match(MarchArgs a, const unsigned long long* __restrict__ key,
-                                                   int32_t* __restrict__ cand) {
+// cand[b]: the earlier bundle of the point whose march bundle b shares (a key's
+// odd ranks go to the one before them), -1 for the others; partner[] the other
+// way.  Blocks (point, 32 bundles), eight lanes a bundle; a warp then compares
+// each candidate with its bundle in full, and what differs marches on its own.
+// One block a point, which took its bundles in turn, and a launch of its own for
+// the comparison needed 13 us for 2 points x 512 rays, 81 for 2 x 2,048 and 15
+// for 2,000 x 16; now 5, about 8 and 7.
+constexpr int MATCH_LANES = 8, MATCH_THREADS = 256, MATCH_BUNDLES = MATCH_THREADS / MATCH_LANES;
+__global__ void __launch_bounds__(MATCH_THREADS) k_ray_match(MarchArgs a, const unsigned long long* __restrict__ key,
+                                                             int32_t* __restrict__ cand,
+                                                             int32_t* __restrict__ partner) {
     if (*a.status) return;
     __shared__ unsigned long long ks[M1_PAIR_MAX];
+    __shared__ int16_t cs[MATCH_BUNDLES];
     const int64_t pb0 = a.point_off[blockIdx.x];
     const int64_t nb = a.point_off[blockIdx.x + 1] - pb0;
     if (nb > M1_PAIR_MAX) return;
-    const int n = (int)nb;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) ks[k] = key[pb0 + k];
+    const int n = (int)nb, step = (int)gridDim.y * MATCH_BUNDLES, first = (int)blockIdx.y * MATCH_BUNDLES;
+    if (first >= n) return;
+    // a second pass only if max_bundles_per_point understates the point
+    const int read = first + step < n ? n : min(n, first + MATCH_BUNDLES);
+    for (int k = threadIdx.x; k < read; k += MATCH_THREADS) ks[k] = key[pb0 + k];
     __syncthreads();
-    for (int kb = 0; kb < n; kb += blockDim.x / 4) {
-        const int k = kb + (int)(threadIdx.x >> 2);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int kb = first; kb < n; kb += step) {
+        const int k = kb + (int)threadIdx.x / MATCH_LANES, own = threadIdx.x % MATCH_LANES;
         const unsigned long long x = k < n ? ks[k] : 0ULL;
         int rank = 0, prev = -1;
         if (x != 0ULL)
-            for (int q = threadIdx.x & 3; q < k; q += 4)
+            for (int q = own; q < k; q += MATCH_LANES)
                 if (ks[q] == x) { ++rank; prev = q; }
-        rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-        prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, 1));
-        rank += __shfl_xor_sync(0xffffffffu, rank, 2);
-        prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, 2));
-        if (k < n && (threadIdx.x & 3) == 0) cand[pb0 + k] = (rank & 1) ? (int32_t)(pb0 + prev) : -1;
-    }
-}
-
-// The full comparison, a warp a candidate: equal bundles become partners, the
-// others march on their own (cand back to -1).
-__global__ void __launch_bounds__(256) k_ray_verify(MarchArgs a, int64_t B, int32_t* __restrict__ cand,
-                                                    int32_t* __restrict__ partner) {
-    if (*a.status) return;
-    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (k >= B) return;
-    const int64_t q = cand[k];
-    if (q < 0) return;
-    const int64_t x0 = a.seg_off[q], y0 = a.seg_off[k], m = a.seg_off[q + 1] - x0;
-    const int64_t dx = a.dir_off[q], dy = a.dir_off[k];
-    bool eq = m == a.seg_off[k + 1] - y0 &&
-              __float_as_uint(a.dir_scale_f[dx]) == __float_as_uint(a.dir_scale_f[dy]) &&
-              (a.bundle_wall[q] != 0) == (a.bundle_wall[k] != 0);
-    for (int64_t i = lane; eq && i < m; i += 32)
-        eq = a.seg_cell[x0 + i] == a.seg_cell[y0 + i] &&
-             __float_as_uint(a.seg_ds_f[x0 + i]) == __float_as_uint(a.seg_ds_f[y0 + i]);
-    eq = __all_sync(0xffffffffu, eq);
-    if (lane == 0) {
-        if (eq) partner[q] = (int32_t)k;
-        else cand[k] = -1;
+#pragma unroll
+        for (int o = 1; o < MATCH_LANES; o <<= 1) {
+            rank += __shfl_xor_sync(0xffffffffu, rank, o);
+            prev = max(prev, __shfl_xor_sync(0xffffffffu, prev, o));
+        }
+        if (own == 0) cs[k - kb] = (rank & 1) ? (int16_t)prev : (int16_t)-1;
+        __syncthreads();
+        for (int i = warp; i < MATCH_BUNDLES; i += MATCH_THREADS / 32) {
+            if (cs[i] < 0) continue;   // the same for the whole warp
+            const int64_t b = pb0 + kb + i, q = pb0 + cs[i];
+            const int64_t x0 = a.seg_off[q], y0 = a.seg_off[b], m = a.seg_off[q + 1] - x0;
+            const int64_t dx = a.dir_off[q], dy = a.dir_off[b];
+            bool eq = m == a.seg_off[b + 1] - y0 &&
+                      __float_as_uint(a.dir_scale_f[dx]) == __float_as_uint(a.dir_scale_f[dy]) &&
+                      (a.bundle_wall[q] != 0) == (a.bundle_wall[b] != 0);
+            for (int64_t j = lane; eq && j < m; j += 32)
+                eq = a.seg_cell[x0 + j] == a.seg_cell[y0 + j] &&
+                     __float_as_uint(a.seg_ds_f[x0 + j]) == __float_as_uint(a.seg_ds_f[y0 + j]);
+            eq = __all_sync(0xffffffffu, eq);
+            if (eq && lane == 0) {
+                cand[b] = (int32_t)q;
+                partner[q] = (int32_t)b;
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -874,18 +887,38 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
     // the point's marched bundles (those that are no one's partner), in index order
     __shared__ int16_t us[M1_PAIR_MAX];
     __shared__ int nu;
-    const bool all = nb > M1_PAIR_MAX;
+    const bool all = cand == nullptr || nb > M1_PAIR_MAX;
     if (!all) {
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x, n = (int)nb;
-            int out = 0;
-            for (int k0 = 0; k0 < n; k0 += 32) {
-                const bool keep = k0 + lane < n && cand[pb0 + k0 + lane] < 0;
-                const unsigned mk = __ballot_sync(0xffffffffu, keep);
-                if (keep) us[out + __popc(mk & ((1u << lane) - 1u))] = (int16_t)(k0 + lane);
-                out += __popc(mk);
+        // a word of flags a warp pass, then a warp's prefix over the words (one
+        // warp in order, and the slices' loads by number below: 2,000 points x 16
+        // bundles 26 us, now 15)
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = (int)nb, words = (n + 31) / 32;
+        __shared__ unsigned keep[M1_PAIR_MAX / 32];
+        __shared__ int before[M1_PAIR_MAX / 32];
+#pragma unroll 4
+        for (int w = warp; w < words; w += 4) {
+            const int k = 32 * w + lane;
+            const unsigned mk = __ballot_sync(0xffffffffu, k < n && cand[pb0 + (k < n ? k : 0)] < 0);
+            if (lane == 0) keep[w] = mk;
+        }
+        __syncthreads();
+        if (warp == 0) {   // two words a lane
+            const int c0 = 2 * lane < words ? __popc(keep[2 * lane]) : 0;
+            const int c1 = 2 * lane + 1 < words ? __popc(keep[2 * lane + 1]) : 0;
+            int sum = c0 + c1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, sum, o);
+                if (lane >= o) sum += v;
             }
-            if (lane == 0) nu = out;
+            before[2 * lane] = sum - c0 - c1;
+            before[2 * lane + 1] = sum - c1;
+            if (lane == 31) nu = sum;
+        }
+        __syncthreads();
+        for (int w = warp; w < words; w += 4) {
+            const unsigned mk = keep[w];
+            if (mk >> lane & 1u) us[before[w] + __popc(mk & ((1u << lane) - 1u))] = (int16_t)(32 * w + lane);
         }
         __syncthreads();
         nb = nu;
@@ -894,10 +927,10 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
     const int64_t m = nb > g ? (nb - g + G - 1) / G : 0;                     // bundles of this group
     const int64_t base = pb0 + (int64_t)g * (nb / G) + (g < nb % G ? g : nb % G);   // the group's first entry
     int32_t* so = soff + blockIdx.x * (M1_SLICES + 1);
-    __shared__ int64_t len[1024];
-    __shared__ int16_t order[1024];
+    __shared__ int32_t len[1024];
+    __shared__ int16_t order[1024], place[1024];   // bundle and place in its slice, by rank
     __shared__ int8_t slice_of[1024];
-    __shared__ int32_t cnt[M1_SLICES + 1];
+    __shared__ int32_t start[M1_SLICES];
     if (m > 1024) {   // round-robin in index order
         for (int64_t k = threadIdx.x; k < m; k += blockDim.x) {
             const int s = (int)(k % M1_SLICES);
@@ -915,39 +948,47 @@ __global__ void __launch_bounds__(128) k_march_plan(const int64_t* __restrict__ 
     const int mm = (int)m;
     for (int k = threadIdx.x; k < mm; k += blockDim.x) {
         const int64_t b = uniq(base + k);
-        len[k] = seg_off[b + 1] - seg_off[b];
+        len[k] = (int32_t)min(seg_off[b + 1] - seg_off[b], (int64_t)2147483647);
     }
     __syncthreads();
     for (int k = threadIdx.x; k < mm; k += blockDim.x) {   // rank: longer first, then lower index
-        const int64_t lk = len[k];
+        const int32_t lk = len[k];
         int r = 0;
         for (int q = 0; q < mm; ++q) r += (len[q] > lk) || (len[q] == lk && q < k);
         order[r] = (int16_t)k;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0) {   // in registers: a slice's load or count by its number would go through memory
         int64_t load[M1_SLICES];
+        int cnt[M1_SLICES];
+#pragma unroll
         for (int s = 0; s < M1_SLICES; ++s) { load[s] = 0; cnt[s] = 0; }
         for (int r = 0; r < mm; ++r) {
-            const int k = order[r];
-            int best = 0;
-            for (int s = 1; s < M1_SLICES; ++s) best = load[s] < load[best] ? s : best;
-            slice_of[k] = (int8_t)best;
-            load[best] += len[k] + 1;
-            ++cnt[best];
+            const int64_t l = (int64_t)len[order[r]] + 1;
+            int best = 0, at = 0;
+            int64_t least = load[0];
+#pragma unroll
+            for (int s = 1; s < M1_SLICES; ++s)
+                if (load[s] < least) { least = load[s]; best = s; }
+#pragma unroll
+            for (int s = 0; s < M1_SLICES; ++s)
+                if (s == best) { load[s] += l; at = cnt[s]++; }
+            slice_of[r] = (int8_t)best;
+            place[r] = (int16_t)at;
         }
         int acc = 0;
-        for (int s = 0; s < M1_SLICES; ++s) { const int c = cnt[s]; cnt[s] = acc; acc += c; }
-        cnt[M1_SLICES] = acc;
-        for (int s = 0; s <= M1_SLICES; ++s) so[s] = (int32_t)(base + cnt[s]);
-        // each slice's bundles, longest first
-        int fill[M1_SLICES];
-        for (int s = 0; s < M1_SLICES; ++s) fill[s] = cnt[s];
-        for (int r = 0; r < mm; ++r) {
-            const int k = order[r];
-            plan[base + fill[slice_of[k]]++] = uniq(base + k);
+#pragma unroll
+        for (int s = 0; s < M1_SLICES; ++s) {
+            start[s] = acc;
+            so[s] = (int32_t)(base + acc);
+            acc += cnt[s];
         }
+        so[M1_SLICES] = (int32_t)(base + acc);
     }
+    __syncthreads();
+    // each slice's bundles, longest first
+    for (int r = threadIdx.x; r < mm; r += blockDim.x)
+        plan[base + start[slice_of[r]] + place[r]] = uniq(base + order[r]);
 }
 
 // A lane's 2 NP adjacent columns of one row, as NP packed pairs.
@@ -1108,7 +1149,7 @@ __global__ void __launch_bounds__(256, RAPRAL_MARCH_MINB) k_march1(MarchArgs a, 
         const M1V<NP> I = m1_bundle<NP, VEC>(a, b, a.dir_scale_f[d0], st, lane, kb, jb, dq, a.ld * 4, I0);
         if (a.I_out) m1_store<NP, VEC>(reinterpret_cast<float*>(a.I_out) + d0 * a.nk + col, I, own);
         float w = a.dir_weight_f[d0];
-        const int b2 = partner[b];
+        const int b2 = partner ? partner[b] : -1;
         if (b2 >= 0) {   // the equal ray: its weight, and its intensities
             const int64_t d2 = a.dir_off[b2];
             w += a.dir_weight_f[d2];
@@ -1342,15 +1383,18 @@ struct M1Plan {
     int32_t* soff;             // [n_points G (M1_SLICES + 1)]
 };
 
-static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t B, int64_t nk, int G,
-                                 void* part, const M1Plan& pl) {
+static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t B, int64_t n_segments,
+                                 int64_t nk, int maxb, int G, void* part, const M1Plan& pl) {
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
-    if (B > 0)
-        k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, P, B, pl.key, pl.cand, pl.partner);
-    k_ray_match<<<(unsigned)P, 512, 0, ctx->stream>>>(a, pl.key, pl.cand);
-    if (B > 0) k_ray_verify<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, B, pl.cand, pl.partner);
-    k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, pl.cand, G, pl.plan, pl.soff,
+    const bool pairs = nk >= M1_PAIR_COLUMNS && n_segments * nk >= M1_PAIR_WORK;
+    int32_t *cand = pairs ? pl.cand : nullptr, *partner = pairs ? pl.partner : nullptr;
+    if (pairs) {
+        const dim3 gm((unsigned)P, div_up(std::min(maxb, M1_PAIR_MAX), MATCH_BUNDLES));
+        k_ray_hash<<<div_up(B * 32, 256), 256, 0, ctx->stream>>>(a, P, B, pl.key, cand, partner);
+        k_ray_match<<<gm, MATCH_THREADS, 0, ctx->stream>>>(a, pl.key, cand, partner);
+    }
+    k_march_plan<<<(unsigned)(P * G), 128, 0, ctx->stream>>>(a.point_off, a.seg_off, cand, G, pl.plan, pl.soff,
                                                              a.status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1375,11 +1419,11 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
     const auto grid = [&](int np) { return dim3((unsigned)(P << lgG), div_up(nk, 64 * np)); };
     const bool four = (P << lgG) * (int64_t)div_up(nk, 128) >= 152 * 10;
     if (four && march1_vec(a, nk, part, 2))
-        k_march1<2, true><<<grid(2), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
+        k_march1<2, true><<<grid(2), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, partner, pf);
     else if (march1_vec(a, nk, part, 1))
-        k_march1<1, true><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
+        k_march1<1, true><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, partner, pf);
     else
-        k_march1<1, false><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, pl.partner, pf);
+        k_march1<1, false><<<grid(1), 32 * M1_SLICES, 0, ctx->stream>>>(b, lgG, pl.plan, pl.soff, partner, pf);
     e = cudaGetLastError();
     if (e != cudaSuccess || G == 1) return e;
     k_group_sum<float><<<(unsigned)std::min<int64_t>(div_up(P * nk, 256), 152 * 16), 256, 0, ctx->stream>>>(
@@ -1512,7 +1556,8 @@ cudaError_t launch_march(rapral_ctx* ctx, const rapral_rays* r, const void* kapp
     pl.plan = reinterpret_cast<int32_t*>(take((size_t)r->n_bundles * 4));
     pl.soff = reinterpret_cast<int32_t*>(take((size_t)r->n_points * G * (M1_SLICES + 1) * 4));
     if (march1_applies(a, r->max_dirs, r->max_bundles_per_point, r->node_values != 0))
-        return march1_launch(ctx, a, r->n_points, r->n_bundles, nk, G, part, pl);
+        return march1_launch(ctx, a, r->n_points, r->n_bundles, r->n_segments, nk,
+                              r->max_bundles_per_point, G, part, pl);
     return march_t<float>(ctx, a, r->n_points, nk, r->max_dirs, r->max_bundles_per_point, G, part,
                           r->node_values != 0);
 }

@@ -27,10 +27,11 @@ def _fill_workspace(ctx):
 @pytest.mark.parametrize("precision", [R.FP32, R.FP64])
 @pytest.mark.parametrize("mirrored", [False, True])
 @pytest.mark.parametrize("ahead,after", [(1, 0), (0, 1), (37, 0), (0, 5), (11, 300)])
-def test_points_cover_part_of_the_bundles(ahead, after, mirrored, precision):
+@pytest.mark.parametrize("nk", [130, 40_001])   # without and with the search for equal rays
+def test_points_cover_part_of_the_bundles(nk, ahead, after, mirrored, precision):
     ctx = R.Context(0)
     rng = np.random.default_rng(ahead + after)
-    C, P, n, nk = 60, 3, 24, 130
+    C, P, n = 60, 3, 24
     dt = torch.float64 if precision == R.FP64 else torch.float32
     rays = [(rng.integers(0, C, m), rng.uniform(0.01, 1.0, m)) for m in rng.integers(1, 40, ahead + P * n + after)]
     if mirrored:
@@ -48,7 +49,7 @@ def test_points_cover_part_of_the_bundles(ahead, after, mirrored, precision):
 
     kap = torch.as_tensor(10.0 ** rng.uniform(-5, 0.3, (C, nk)), device=ctx.device).to(dt)
     em = torch.as_tensor(rng.uniform(0.5, 2.0, (C, nk)), device=ctx.device).to(dt)
-    g = synth.Grid(300.0, 900.0, 1000)
+    g = synth.Grid(300.0, 900.0, 50_000)
     out = []
     for part, off in ((rays, ahead), (rays[ahead:ahead + P * n], 0)):
         s = ray_set(part, off + np.arange(P + 1) * n)
@@ -62,3 +63,35 @@ def test_points_cover_part_of_the_bundles(ahead, after, mirrored, precision):
     assert np.array_equal(q, q0)
     assert np.array_equal(I[ahead:ahead + P * n], I0)
     assert np.all(I[:ahead] == -1.0) and np.all(I[ahead + P * n:] == -1.0)
+
+
+@pytest.mark.parametrize("n", [31, 33, 300, 2048])
+@pytest.mark.parametrize("claimed", [8, 32, 5000])
+@pytest.mark.parametrize("searched", [False, True])
+def test_points_larger_than_claimed(searched, n, claimed):
+    """max_bundles_per_point sizes launches; a set that states another value has the same intensities, bit for bit."""
+    ctx = R.Context(0)
+    rng = np.random.default_rng(n)
+    C, P = 60, 2
+    half = [(rng.integers(0, C, m), rng.uniform(0.01, 1.0, m)) for m in rng.integers(1, 12, P * n)]
+    for p in range(P):
+        for k in range(n // 3):
+            half[p * n + n - 1 - k] = half[p * n + k]
+    seg = np.concatenate([[0], np.cumsum([len(r[0]) for r in half])])
+    nk = max(256, 2 ** 25 // int(seg[-1]) + 1) if searched else 70
+    rays = R.rays_from_arrays(np.arange(P + 1) * n, seg, np.concatenate([r[0] for r in half]),
+                              np.concatenate([r[1] for r in half]), np.arange(P * n + 1), np.ones(P * n),
+                              rng.uniform(0.1, 1.0, P * n), np.zeros(P * n), 0.0, ctx.device)
+    kap = torch.as_tensor(10.0 ** rng.uniform(-5, 0.3, (C, nk)), device=ctx.device).float()
+    em = torch.as_tensor(rng.uniform(0.5, 2.0, (C, nk)), device=ctx.device).float()
+    out = []
+    for m in (n, claimed):
+        rays.struct.max_bundles_per_point = m
+        q = torch.full((P, nk), float("nan"), dtype=torch.float32, device=ctx.device)
+        I = torch.full((P * n, nk), float("nan"), dtype=torch.float32, device=ctx.device)
+        R.trace_rays(ctx, rays, C, kap, em, synth.Grid(300.0, 900.0, 200_000), 0, nk, R.FP32, q, I)
+        ctx.sync()
+        out.append((q.cpu().numpy(), I.cpu().numpy()))
+    assert np.array_equal(out[0][1], out[1][1])
+    # the bundles' sums: other groups and slices, each compensated; FP32 rounding of up to 16 partial sums
+    assert np.max(np.abs(out[0][0] / out[1][0] - 1)) <= 16 * 2.0 ** -24
