@@ -186,9 +186,38 @@ __device__ __forceinline__ int64_t node_below(const double* x, int64_t a, int64_
     return lo > a ? lo - 1 : a;
 }
 
-// one warp per (tile, level): a search for the tile's first point, then a
-// forward walk over the lane's points (a tile spans few nodes)
-template <typename Tp>
+// The lane's first node of a (tile, level): the last at or below the tile's
+// first point, from which its points are walked to, or, in DENSE tables, where
+// the warp's 32 first points span more than 32 nodes (the walk follows them
+// load by load), by a bisection a lane.  24 cells, 100 tables of 20,000 nodes,
+// 1,001 points: 46.8 ms walked, 33.6 so; in the kernel of 100 tables of 120
+// nodes the question alone costs 4 us of the call's 1,001, so models of at most
+// 512 nodes a level on average (dense_tables) keep it out.
+constexpr int NODE_WALK = 32;
+static bool dense_tables(const ContModels& M) {
+    for (int m = 0; m < M.M; ++m)
+        if (M.m[m].n_nodes > (int64_t)512 * M.m[m].n_levels) return true;
+    return false;
+}
+template <bool DENSE>
+__device__ __forceinline__ int64_t lane_node(const double* x, int64_t a, int64_t b, double lam_min, double h,
+                                             int64_t kt) {
+    const int64_t j = node_below(x, a, b, grid_lam(lam_min, h, kt));
+    if (!DENSE || j + NODE_WALK >= b) return j;
+    if (!pos_le(x[j + NODE_WALK], grid_lam(lam_min, h, kt + 31))) return j;   // the same for the warp
+    const double lam = grid_lam(lam_min, h, kt + (threadIdx.x & 31));
+    int64_t lo = j, hi = b;
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (pos_le(x[mid], lam)) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// one warp per (tile, level): a search for the lane's first node, then a
+// forward walk over its points
+template <typename Tp, bool DENSE>
 __global__ void __launch_bounds__(128) k_cont_sigma(ContModels M, const ContLevel* lev, const int* n_lev,
                                                      const int64_t* tab_off, int W, double lam_min, double h,
                                                      int64_t k0, int64_t nk, Tp* tab, const int* status) {
@@ -203,7 +232,7 @@ __global__ void __launch_bounds__(128) k_cont_sigma(ContModels M, const ContLeve
         const int64_t a = m.node_off[L.i], b = m.node_off[L.i + 1] - 1;
         const double* x = m.node_lam;
         const double* y = m.node_sigma;
-        int64_t j = node_below(x, a, b, grid_lam(lam_min, h, k0 + t * W));
+        int64_t j = lane_node<DENSE>(x, a, b, lam_min, h, k0 + t * W);
         for (int p = lane; p < W; p += 32) {
             const int64_t k = t * W + p;
             double sg = 0.0;
@@ -237,6 +266,7 @@ __global__ void k_cont_nodes32(ContModels M, float* yf, float* sf, float* dxf, c
 // inside the table is found in FP64 with the grid's own wavelength formula
 // (so that zero / non-zero is decided as in FP64), the interpolation is FP32
 // from the tile's first wavelength: lam - x_j = (lam_t - x_j) + p h.
+template <bool DENSE>
 __global__ void __launch_bounds__(128) k_cont_sigma32(ContModels M, const ContLevel* lev, const int* n_lev,
                                                        const int64_t* tab_off, int W, double lam_min, double h,
                                                        int64_t k0, int64_t nk, const float* yf, const float* sf,
@@ -256,7 +286,7 @@ __global__ void __launch_bounds__(128) k_cont_sigma32(ContModels M, const ContLe
         const double* x = m.node_lam;
         const int64_t nb = M.node0[L.m];
         const int64_t klo = L.klo, khi = L.khi;
-        int64_t j = node_below(x, a, b, lam_t);   // last node <= the tile's first wavelength (or a)
+        int64_t j = lane_node<DENSE>(x, a, b, lam_min, h, kt);
         float base = (float)(lam_t - x[j]);
         for (int p = lane; p < W; p += 32) {
             const int64_t k = kt + p;
@@ -822,11 +852,12 @@ static int cont_run(rapral_ctx* ctx, const ContModels& Mh, int S, const rapral_c
         int64_t mx = 0;
         for (int m = 0; m < M; ++m) mx = std::max<int64_t>(mx, Mh.m[m].n_nodes);
         k_cont_nodes32<<<dim3(div_up(mx, 256), M), 256, 0, s>>>(Mh, yf, sf, dxf, ctx->d_status);
-        k_cont_sigma32<<<(unsigned)T, 128, 0, s>>>(Mh, lev, n_lev, tab_off, W, g->lam_min, h, k0, nk, yf, sf, dxf,
-                                                  reinterpret_cast<float*>(tab), ctx->d_status);
+        const auto resample = dense_tables(Mh) ? k_cont_sigma32<true> : k_cont_sigma32<false>;
+        resample<<<(unsigned)T, 128, 0, s>>>(Mh, lev, n_lev, tab_off, W, g->lam_min, h, k0, nk, yf, sf, dxf,
+                                             reinterpret_cast<float*>(tab), ctx->d_status);
     } else {
-        k_cont_sigma<Tp><<<(unsigned)T, 128, 0, s>>>(Mh, lev, n_lev, tab_off, W, g->lam_min, h, k0, nk, tab,
-                                                    ctx->d_status);
+        const auto resample = dense_tables(Mh) ? k_cont_sigma<Tp, true> : k_cont_sigma<Tp, false>;
+        resample<<<(unsigned)T, 128, 0, s>>>(Mh, lev, n_lev, tab_off, W, g->lam_min, h, k0, nk, tab, ctx->d_status);
     }
     k_cont_points<Tp><<<div_up(n_pad, 256), 256, 0, s>>>(Mh, n_pad, g->lam_min, h, k0, ph, pts, Dj, Dw,
                                                          ctx->d_status);
