@@ -97,9 +97,12 @@ __global__ void __launch_bounds__(256) k_line_plan(rapral_lines ln, const double
         bool near = true;
         if (!stark && !lb) {
             const float lamf = (float)lam0;
-            const float wf = 100.0f * (5.9e-6f + (float)ln.lamS0[l] * (float)__longlong_as_double((long long)dmax[1]) +
-                                       3.5811651e-7f * lamf * rsqrtf((float)mass[s]) *
-                                           (float)__longlong_as_double((long long)dmax[0]));
+            const float wf =
+                (float)RAPRAL_WINDOW *
+                ((float)RAPRAL_LAM_NATURAL +
+                 (float)ln.lamS0[l] * (float)__longlong_as_double((long long)dmax[1]) +
+                 (float)RAPRAL_DOPPLER_HALF * lamf * rsqrtf((float)mass[s]) *
+                     (float)__longlong_as_double((long long)dmax[0]));
             const double w = (double)(wf * 1.0001f) + 4.0 * h;   // NaN or inf: kept
             near = !(lam0 + w < lam_min + (double)k0 * h || lam0 - w > lam_min + (double)(k0 + nk - 1) * h);
         }
