@@ -182,7 +182,7 @@ int rapral_batch_create(rapral_ctx* ctx, int n_items, const rapral_batch_item* i
         LineSumArgs& a = hitems[i].a;
         a.lp = lps[i]; a.lf = lfs[i]; a.cp = cps[i]; a.lnpref = r.cells.lnpref; a.S = r.sp.n_species; a.C = r.cells.n_cells;
         a.tile_off = plans[i].tile_off; a.tile_lines = plans[i].tile_lines;
-        a.lam_min = r.grid.lam_min; a.h = r.h; a.k0 = r.k0; a.nk = r.nk; a.ld = r.ld; a.tile_w = W;
+        a.lam_min = r.grid.lam_min; a.set_spacing(r.h); a.k0 = r.k0; a.nk = r.nk; a.ld = r.ld; a.tile_w = W;
         a.lb = btabs[i].lb; a.lb32 = btabs[i].lb32; a.cb = btabs[i].cb; a.cb32 = btabs[i].cb32;
         a.kappa = r.kappa; a.emis = r.emis; a.status = ctx->d_status; a.stats = ctx->d_stats; a.count = ctx->count_work;
         hitems[i].unit_off = units;

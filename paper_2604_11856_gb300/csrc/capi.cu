@@ -359,7 +359,7 @@ int rapral_spectral_coeffs(rapral_ctx* ctx, const rapral_species* sp, const rapr
     LineSumArgs a;
     a.lp = lp; a.lf = lf; a.cp = cp; a.lnpref = cells->lnpref; a.S = sp->n_species; a.C = C;
     a.tile_off = plan.tile_off; a.tile_lines = plan.tile_lines;
-    a.lam_min = g->lam_min; a.h = h; a.k0 = k0; a.nk = nk; a.ld = ld; a.tile_w = W;
+    a.lam_min = g->lam_min; a.set_spacing(h); a.k0 = k0; a.nk = nk; a.ld = ld; a.tile_w = W;
     a.kappa = kappa; a.emis = emis; a.status = ctx->d_status; a.stats = ctx->d_stats; a.count = ctx->count_work;
     a.lb = lb; a.lb32 = lb32; a.cb = cb; a.cb32 = cb32;
     if (ctx->dep_lnb) {

@@ -731,6 +731,12 @@ __device__ __forceinline__ float sinpi_series(float d) {
 // r, and the Gaussian e^{-2.772 u^2} below 5e-44, under 1e-30 of it for the r
 // that a natural width of 5.9e-6 nm leaves: both are left out there.
 constexpr float NEAR_U = 6.0f;
+// Constants of the profile whose rounding would lean one way for every line:
+// the Gaussian's exponent -2.772 log2(e) u^2 to the nearest float; the
+// approximate ex2 lies 5.1e-8 low on average over [-20, 0], which a shift of
+// its argument takes back; 1.065 of the normalisation rounds up by 5.4e-8,
+// which its factor 500 takes back (the next float, 6.1e-8 up).
+constexpr float GAUSS_SCALE = -3.9991507f, GAUSS_SHIFT = 7.4e-8f, NORM_FACTOR = 500.00003f;
 
 struct PairF32 {
     float lo, hi;     // window part inside the tile, offsets from kt0
@@ -824,13 +830,13 @@ __device__ __forceinline__ bool setup_pair_f32(const LineSumArgs& a, const LineF
     if (!(Sj > 0.0f) && Sk == 0.0f) return false;
     const float iv = rcp_approx(lamV);
     float r = lamL * iv;
-    float pre = 1e3f * 0.5f * iv * rcp_approx(1.065f + 0.447f * r + 0.058f * r * r);
-    float s = 0.5f * hf * iv;
+    float pre = NORM_FACTOR * iv * rcp_approx(1.065f + 0.447f * r + 0.058f * r * r);   // 1e3 / (2 lamV ..)
+    float s = 0.5f * fmaf(hf, iv, a.h_lo * iv);
     if (VG) {   // exact Voigt: u is x = dlam sqrt(ln 2) / lamG, r is y, pre 1e3 / (sigma sqrt(2 pi))
         const float ig = rcp_approx(lamG);
         r = 0.83255461f * lamL * ig;
         pre = 1e3f * 0.46971864f * ig;
-        s = 0.83255461f * hf * ig;
+        s = 0.83255461f * fmaf(hf, ig, a.h_lo * ig);
     }
     const float u0 = L.delta * s;                    // u of the centre's offset from kc
     {   // signed u at kt0 without rounding loss: (kt0 - kc) is exact, its
@@ -920,7 +926,7 @@ __device__ __forceinline__ void slot_eval(float k, float2 nmid, float2 half, flo
     float2 h = __fmul2_rn(__ffma2_rn(nc, q4, p1), rd);
     if (NEAR) {
         const float2 xc = __fmul2_rn(c2(-0.5770780f), v);  // -0.4 log2(e) v
-        const float2 xg = __fmul2_rn(c2(-3.99915f), u2);   // -2.772 log2(e) u^2
+        const float2 xg = __ffma2_rn(c2(GAUSS_SCALE), u2, c2(GAUSS_SHIFT));
         const float2 e2 = make_float2(ex2_approx(xc.x), ex2_approx(xc.y));
         const float2 g = make_float2(ex2_approx(xg.x), ex2_approx(xg.y));
         const float2 omr = __ffma2_rn(c2(-1.0f), r, c2(1.0f));
@@ -1002,7 +1008,8 @@ __device__ __forceinline__ void sweep_whole(float lanef, float s, float ub, floa
             const int i = i0 + 2 * h;
             float2 br = __fmul2_rn(num[h], make_float2(qp[h].y * rr[h], qp[h].x * rr[h]));
             if (NEAR) {
-                const float2 xc = __fmul2_rn(c2(-0.5770780f), v[h]), xg = __fmul2_rn(c2(-3.99915f), u2[h]);
+                const float2 xc = __fmul2_rn(c2(-0.5770780f), v[h]);
+                const float2 xg = __ffma2_rn(c2(GAUSS_SCALE), u2[h], c2(GAUSS_SHIFT));
                 const float2 e2 = make_float2(ex2_approx(xc.x), ex2_approx(xc.y));    // e^{-0.4 v}
                 const float2 g = make_float2(ex2_approx(xg.x), ex2_approx(xg.y));     // e^{-2.772 u^2}
                 br = __ffma2_rn(c2(c), e2, br);

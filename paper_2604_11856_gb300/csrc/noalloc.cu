@@ -275,7 +275,7 @@ int noalloc_impl(int dev, cudaStream_t stream, const rapral_species* sp, const r
         LineSumArgs a;
         a.lp = lp; a.lf = lf; a.cp = cp; a.lnpref = cells->lnpref; a.S = sp->n_species; a.C = C;
         a.tile_off = plan.tile_off; a.tile_lines = plan.tile_lines;
-        a.lam_min = g->lam_min; a.h = h; a.k0 = k0; a.nk = nk; a.ld = ld; a.tile_w = W;
+        a.lam_min = g->lam_min; a.set_spacing(h); a.k0 = k0; a.nk = nk; a.ld = ld; a.tile_w = W;
         a.kappa = kappa; a.emis = emis; a.status = ctx.d_status; a.stats = ctx.d_stats; a.count = 0;
         e = launch_line_sum(&ctx, a, precision, T);
     }

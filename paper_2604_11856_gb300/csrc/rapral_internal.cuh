@@ -274,6 +274,7 @@ struct LineSumArgs {
     const int* tile_off;
     const int* tile_lines;
     double lam_min, h;
+    float h_lo;               // h - (float)h: the spacing's FP32 rounding would lean one way for every line
     int64_t k0, nk, ld;
     int tile_w;
     void* kappa;
@@ -296,6 +297,11 @@ struct LineSumArgs {
     // exact Voigt line shape instead of Whiting's (rapral_set_profile; the
     // expansion's coefficients are in constant memory, see voigt_upload)
     int voigt = 0;
+
+    void set_spacing(double spacing) {
+        h = spacing;
+        h_lo = (float)(spacing - (double)(float)spacing);
+    }
 };
 
 // Workspace of the optional resonance / van der Waals terms of one request:
