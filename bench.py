@@ -105,22 +105,22 @@ def parse():
 # one-pass ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the kernel
 # source with this digest (source_digest).  Other cell / point counts scale in proportion (the
 # bytes are the kappa / j rows written); a different source (comments aside) gives null.
-LINE_SUM_TRAFFIC = {"sha1": "9cb401bd4549a6eaf0a40186c4f84d5e3c0dda4c", "cells": 200, "grid_points": 1_000_000,
-                    "bytes": 53_932_288 + 1_543_667_712}
+LINE_SUM_TRAFFIC = {"sha1": "de9bd391ea2630ed6a3e9be430af77da5fc68e32", "cells": 200, "grid_points": 1_000_000,
+                    "bytes": 55_652_352 + 1_555_708_160}
 
 
 # DRAM bytes of one FP32 continuum level-sum launch at full size (200 cells x
 # 1e6 points, N and O with 100 levels each), from a one-pass ncu capture of the
 # kernel source with this digest (source_digest); a different source gives null.
-CONT_TRAFFIC = {"sha1": "b20ff15bc5d2a99674fcbc6991e7a0c6b0701352", "cells": 200, "grid_points": 1_000_000, "levels": 100,
-                "bytes": 1_782_987_520 + 1_539_120_640}
+CONT_TRAFFIC = {"sha1": "372f9aa637b5bc21c9cfbdb7247d80d000d15d9a", "cells": 200, "grid_points": 1_000_000, "levels": 100,
+                "bytes": 1_783_207_680 + 1_539_217_408}
 
 # DRAM bytes (read + write) of one FP32 march launch (k_march1) on a full
 # 65,536-point afterbody chunk (80,000 cells, 26,697,080 ray segments), from a
 # one-pass ncu capture of the kernel source with this digest (source_digest);
 # another source or ray set gives null.
-MARCH_TRAFFIC = {"sha1": "156f11f3f01ceca0c87329b7dcd4e547185c0877", "cells": 80_000, "segments": 26_697_080,
-                 "grid_points": 65_536, "bytes": 356_842_381_824 + 468_259_328}
+MARCH_TRAFFIC = {"sha1": "2698538858ef375ded21d642d03c690b7e2f3279", "cells": 80_000, "segments": 26_697_080,
+                 "grid_points": 65_536, "bytes": 969_241_906_688 + 83_612_584_192}
 
 
 def source_digest(name):
@@ -920,8 +920,8 @@ def run_headline(args):
                                 "here, are marched once) x columns",
             "peak_source": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in peaks else "fallback",
             "served_from": "L2: the gathers hit L2, whose measured gather bandwidth is in march.l2_gather_peak; "
-                           "DRAM (traffic) sees the chunk's kappa / j once and the segment lists once per "
-                           "128-column wavelength tile",
+                           "DRAM (traffic) sees the chunk's kappa / j several times: a 128-column tile's rows "
+                           "are 82 MB, beside the segment lists of its points, in 129 MB of L2",
             "frac_of_l2_gather_peak": gather / l2_peak}
     out = {"metric": METRIC, "value": value, "unit": "cell·λ points/s", "n_gpus": world, "steps": K,
            "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",

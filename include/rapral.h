@@ -299,8 +299,10 @@ RAPRAL_API int rapral_spectral_coeffs(rapral_ctx* ctx, const rapral_species* sp,
  *   I <- I e^{-dtau} + a j_far + b j_near,  dtau = kappa_far ds scale,
  *   a = (f - e^{-dtau}) / kappa_far,  b = (1 - f) / kappa_far,
  *   f = (1 - e^{-dtau}) / dtau,
- * with the series of a and b when |dtau| < 4e-4 (FP64, three terms) or
- * |dtau| < 0.5 (FP32, seven terms).
+ * evaluated, where |dtau| < 0.5, by the series of (1 - f) / dtau instead:
+ * FP64 with 3, 4, 5, 6, 9 or 14 terms below 2^-17, 2^-13, 2^-10, 2^-7, 2^-4
+ * and 1/2 (truncation below 2e-17 of the result), FP32 with four terms below
+ * 2^-5 (3e-9) and seven above (4e-8).
  * The march starts from 0 (far field) or the Planck intensity at T_wall.
  * Then q_lambda[p][k] = sum over the point's directions of weight * I.
  * In: kappa, emis [C][ld] for grid points [k0, k0+nk) (as written by

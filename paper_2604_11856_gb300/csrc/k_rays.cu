@@ -297,11 +297,7 @@ __device__ __forceinline__ double planck(double lam_nm, double T, const Phys& ph
     return 1e-7 * 2.0 * ph.h * ph.c * ph.c / (1e4 * l2 * l2 * lcm * expm1(ph.h * ph.c / (lcm * ph.kB * T)));
 }
 
-// The march of one bundle over the lane's V columns: staged segment list,
-// next-cell gathers one step ahead, all MAXD directions per segment.  A
-// bundle with nd < MAXD directions marches the others with scale 0, which
-// leaves their intensity at its start value (e = 1, zero source): no
-// per-direction check in the loop.  Returns the intensities in I[v][d].
+// One staged segment of a warp's bundle (march_nodes, march_multi, march_bundle).
 template <class T> struct __align__(16) SegStage {
     const char* row;   // kappa row of the segment's next cell
     T ds;              // path length (x the direction scale for one-direction bundles)
@@ -517,20 +513,22 @@ __device__ __forceinline__ void march_bundle(const MarchArgs& a, int64_t b, int6
     }
 }
 
-// k_march: the segment march with the angular reduction.  A block of eight
-// warps covers one (surface point, bundle group) and a tile of wavelength
-// columns; its warps are SL bundle slices x CW = 8 / SL column groups, and
-// lane l of a column group takes columns l, l + 32, ..., l + 32 (V - 1) of
-// the group's 32 V.  Each gather of a segment is then V coalesced row
-// reads, and the per-segment work (next cell, length, row address) is
-// shared by the V columns and the bundle's directions.  SL = 8 (many bundles
-// a point, as the axisymmetric rays): the eight warps take the bundles of
-// the group round-robin; SL = 1 (a few bundles of many directions, as the
-// tangent slab): all warps march every bundle over eight column groups.
+// k_march: the segment march with the angular reduction.  A block covers one
+// (surface point, bundle group) and a tile of wavelength columns; lane l of a
+// column group takes columns l, l + 32, ..., l + 32 (V - 1) of the group's 32
+// V.  Each gather of a segment is then V coalesced row reads, and the
+// per-segment work (next cell, length, row address) is shared by the V columns
+// and the warp's directions.  Three forms:
+//   SL = 8 (many bundles a point, as the axisymmetric rays): eight warps on the
+//     same columns take the bundles of the group round-robin;
+//   SL = 1, MAXD > 1 (a few bundles of many directions, as the tangent slab):
+//     one warp a block, all of a bundle's directions, or DS > 0: up to DS warps
+//     on the same columns share each bundle's directions;
+//   SL = 1, MAXD = 1: eight warps on eight column groups, every bundle.
 // A warp stages the next cell's row address and the length of 32 segments at
 // a time in shared memory (one coalesced read of the segment list), so no
-// kappa / j gather waits on a dependent load of the list, and loads the next
-// segment's values one step ahead; the last segment of a bundle, whose near
+// kappa / j gather waits on a dependent load of the list, and loads cells'
+// values one step (march_multi: two) ahead; the last segment of a bundle, whose near
 // node is its own cell, is taken after the loop.  A point's bundles are
 // split over 2^lgG blocks (groups) so that enough blocks share a wavelength
 // tile for its kappa / j rows to stay in L2.  Each slice Kahan-sums its
@@ -678,6 +676,8 @@ __global__ void __launch_bounds__(32 * (DS ? DS : march_warps(MAXD, SL)),
 //    (k_march_plan), so the warps finish together at the block's reduction.
 // Every slice still Kahan-sums its bundles in a fixed order and the slices
 // and groups are added in fixed order: results do not depend on timing.
+// Four columns a lane at the 64 registers of four blocks an SM spill 184 bytes
+// a thread (244 loaded); two columns do not, and are 6 % slower on wide ranges.
 
 #ifndef RAPRAL_M1_PF
 #define RAPRAL_M1_PF 2
@@ -1462,7 +1462,9 @@ cudaError_t march_t(rapral_ctx* ctx, const MarchArgs& a, int64_t P, int64_t nk, 
     // keeps it fed at every size: 60 cells x 17 directions x 5,000 / 20,000 /
     // 60,000 / 100,001 columns 1,160 / 1,405 / 2,762 / 3,240 us in one warp, 465 /
     // 840 / 1,820 / 2,820 by threes, 680 / 1,048 / 1,864 / 2,680 by sevens, which
-    // are taken above the line.
+    // are taken above the line.  In FP32 fives are the best form at 55,000 and
+    // 65,000 columns and no branch takes them: where they stop paying has not
+    // been measured.
     if (maxd <= 17 && P * div_up(nk, 32) <= 152 * 11)
         return march_launch<T, 1, 3, 1, false, 6>(ctx, a, P, nk, G, part, std::max(1, (int)div_up(maxd, 3)));
     if constexpr (sizeof(T) == 8) {

@@ -47,8 +47,7 @@ struct BroadArgs {
 #define RAPRAL_LAM_NATURAL 5.9e-6        // natural HWHM, nm
 #define RAPRAL_DOPPLER_HALF (7.16233e-7 / 2.0)
 #define RAPRAL_WINDOW 100.0              // lines reach |dlam| <= 100 lamV
-#define RAPRAL_THIN_F64 4e-4             // |dtau| below which the series is used
-#define RAPRAL_THIN_F32 0.5               // with seven-term series in FP32
+#define RAPRAL_THIN_F32 0.5               // |dtau| below which the FP32 march takes its series (FP64: thin_series)
 #define RAPRAL_SLAB_DIRS 17              // directions per tangent-slab bundle
 
 // Status word layout (device int[8]).
