@@ -1387,7 +1387,7 @@ static cudaError_t march1_launch(rapral_ctx* ctx, const MarchArgs& a, int64_t P,
                                  int64_t nk, int maxb, int G, void* part, const M1Plan& pl) {
     int lgG = 0;
     while ((1 << lgG) < G) ++lgG;
-    const bool pairs = nk >= M1_PAIR_COLUMNS && n_segments * nk >= M1_PAIR_WORK;
+    const bool pairs = B > 0 && nk >= M1_PAIR_COLUMNS && n_segments * nk >= M1_PAIR_WORK;
     int32_t *cand = pairs ? pl.cand : nullptr, *partner = pairs ? pl.partner : nullptr;
     if (pairs) {
         const dim3 gm((unsigned)P, div_up(std::min(maxb, M1_PAIR_MAX), MATCH_BUNDLES));

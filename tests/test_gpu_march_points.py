@@ -95,3 +95,19 @@ def test_points_larger_than_claimed(searched, n, claimed):
     assert np.array_equal(out[0][1], out[1][1])
     # the bundles' sums: other groups and slices, each compensated; FP32 rounding of up to 16 partial sums
     assert np.max(np.abs(out[0][0] / out[1][0] - 1)) <= 16 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("precision", [R.FP32, R.FP64])
+@pytest.mark.parametrize("nk", [70, 40_001])
+def test_points_without_bundles(nk, precision):
+    """Segments that no bundle holds and points without bundles: nothing is marched, the flux is zero."""
+    ctx = R.Context(0)
+    rays = R.rays_from_arrays([0, 0, 0], [0], np.zeros(2000, int), np.ones(2000), [0], np.ones(1), np.ones(1),
+                              np.zeros(1), 0.0, ctx.device)
+    rays.struct.max_dirs, rays.struct.max_bundles_per_point = 1, 9
+    dt = torch.float64 if precision == R.FP64 else torch.float32
+    kap = torch.ones((3, nk), dtype=dt, device=ctx.device)
+    q = torch.full((2, nk), float("nan"), dtype=dt, device=ctx.device)
+    R.trace_rays(ctx, rays, 3, kap, kap, synth.Grid(300.0, 900.0, 50_000), 0, nk, precision, q)
+    ctx.sync()
+    assert float(q.abs().max()) == 0.0
