@@ -119,8 +119,8 @@ CONT_TRAFFIC = {"sha1": "372f9aa637b5bc21c9cfbdb7247d80d000d15d9a", "cells": 200
 # 65,536-point afterbody chunk (80,000 cells, 26,697,080 ray segments), from a
 # one-pass ncu capture of the kernel source with this digest (source_digest);
 # another source or ray set gives null.
-MARCH_TRAFFIC = {"sha1": "2698538858ef375ded21d642d03c690b7e2f3279", "cells": 80_000, "segments": 26_697_080,
-                 "grid_points": 65_536, "bytes": 969_241_906_688 + 83_612_584_192}
+MARCH_TRAFFIC = {"sha1": "f05901564bac6f7d9872a892e7c9433b3f14d21a", "cells": 80_000, "segments": 26_697_080,
+                 "grid_points": 65_536, "bytes": 966_499_450_624 + 83_398_436_352}
 
 
 def source_digest(name):
